@@ -234,30 +234,33 @@ pa_status pa_sweep_timing(pa_ctx *ctx, double *ms, int64_t *launches, double *up
 /* Number of kernels this context has launched so far. */
 int64_t pa_launch_count(const pa_ctx *ctx);
 
-/* Launch configuration of the sweep kernel: threads per CTA (64, 128, 256, 384 or
- * 512; each CTA holds 32 replicas).  Results do not depend on it, only the
- * speed; the package's autotuner times the candidates and picks one.
- * PA_ERR_ARG for other values. */
+/* Launch configuration of the sweep kernel: how many threads share the lattice of
+ * 32 replicas, from few (64) to many (128, 256, 384, 512); each side has its own
+ * variants for them.  Until the call the library chooses by the number of replicas.
+ * Results do not depend on it, only the speed; the package's autotuner times the
+ * candidates and picks one.  Synchronises the context's stream when the value
+ * changes.  PA_ERR_ARG for other values. */
 pa_status pa_set_sweep_threads(pa_ctx *ctx, int32_t threads);
 int32_t pa_get_sweep_threads(const pa_ctx *ctx);
 
 /* Test hook of the sweep kernel (Sec. 2 step 3): per half-sweep the kernel
- * queues the sites whose Metropolis test is still undecided after the first
- * eight bits of the uniforms and finishes them in a second pass; sites that
- * find the queue full finish at once.  cap limits the queue to cap entries
- * (0: every site finishes at once; -1: the kernel's full queue, the default)
- * so that both paths can be checked.  Results do not depend on it.
+ * lists the sites whose Metropolis test is still undecided after the first
+ * eight bits of the uniforms and finishes them in a second pass.  cap limits the
+ * list to cap entries, as far as the kernel can: the second pass then follows
+ * every few sites of a thread, or a site that finds the list full finishes at once
+ * (-1: the kernel's full list, the default), so that both paths can be checked.
+ * Results do not depend on it.
  * PA_ERR_ARG for cap < -1. */
 pa_status pa_set_sweep_queue(pa_ctx *ctx, int32_t cap);
 
-/* Launch configuration of the grouped 3D sweep kernel (Sec. 2 step 3 for 3D
- * lattices of even side 4..16): a CTA holds a number of replica groups that
- * depends on the side; mult = 2 doubles it (fewer, larger CTAs), mult = 1 is
+/* Launch configuration of the 3D sweep kernels (Sec. 2 step 3 for 3D lattices of
+ * even side 4..16): a CTA holds a number of replica groups that depends on the
+ * side and the replicas; mult = 2 doubles it (fewer, larger CTAs), mult = 1 is
  * the default.  Results do not depend on it; the package's autotuner times both.
- * A context whose runs do not use the grouped kernel accepts mult = 1 only.
+ * A context with runs of other lattices, or of more than four sides, accepts mult = 1 only.
  * Synchronises the context's stream.  PA_ERR_ARG for other values,
  * PA_ERR_STATE after an earlier device error.  pa_get_sweep_groups returns the
- * multiple in use (1 without the grouped kernel). */
+ * multiple in use. */
 pa_status pa_set_sweep_groups(pa_ctx *ctx, int32_t mult);
 int32_t pa_get_sweep_groups(const pa_ctx *ctx);
 

@@ -29,7 +29,6 @@ struct RunHost {
     int L, N, W, Wp, nlev, P;
     uint32_t R, Rcap;
     int nblk, ngrp;
-    int g3, nct3;            // 3D kernel: replica groups per CTA, CTAs (0: not eligible)
     int ensemble;
     std::vector<uint8_t> jb;
     int parity;
@@ -43,7 +42,7 @@ enum Region {
 
 enum Shared {
     S_RUNS, S_B2R, S_G2R, S_BETA, S_DBETA, S_Q, S_THR, S_THETA, S_IDS, S_WOUT,
-    S_CTL, S_GBETA, S_GTHR, S_GDB, S_GQ, S_PAIRS, S_POV, S_OVACC, S_OVTICK, S_C3, S_CLNC,
+    S_CTL, S_GBETA, S_GTHR, S_GDB, S_GQ, S_PAIRS, S_POV, S_OVACC, S_OVTICK, S_CTA, S_CLNC,
     S_COUNT
 };
 
@@ -95,6 +94,9 @@ struct pa_ctx {
     std::vector<char> rdone;                    // beta_f reached
     std::vector<std::array<size_t, 5>> rtab_off;  // offsets of its own step tables
     bool finished = false;                  // beta_f reached under the controller
+    uint32_t* d_cta = nullptr;              // CTA -> run map of the sweep launches (device)
+    bool auto_threads = true;               // the rule's threads until the caller sets them
+    bool grouped3 = false;                  // 3D sides whose sets of groups may be doubled
     CtlDev* d_ctl = nullptr;
     double* d_gbeta = nullptr;
     uint32_t* d_gthr = nullptr;
@@ -153,8 +155,6 @@ pa_status make_runs(const pa_run_spec* specs, int M, int method, std::vector<Run
         if (h.Rcap > MAX_POPULATION) return PA_ERR_LIMIT;
         h.nblk = (int)((h.Rcap + SCAN_CHUNK - 1) / SCAN_CHUNK);
         h.ngrp = (int)((h.Rcap + 31) / 32);
-        h.g3 = (*d == 3) ? sweep3d_groups(h.L, 1) : 0;
-        h.nct3 = h.g3 ? (h.ngrp + h.g3 - 1) / h.g3 : 0;
         h.ensemble = s.ensemble;
         h.parity = 0;
         out->push_back(std::move(h));
@@ -190,9 +190,7 @@ Layout make_layout(const std::vector<RunHost>& runs, int n_steps) {
     sz[S_POV] = (size_t)(maxN + 1) * 8;
     sz[S_OVACC] = M * (size_t)(maxN + 1) * 4;  // overlap accumulators, zero between calls
     sz[S_OVTICK] = M * 4;
-    size_t nct3 = 0;
-    for (const RunHost& h : runs) nct3 += (size_t)h.nct3;
-    sz[S_C3] = nct3 * 4;
+    sz[S_CTA] = ngrp * 4;  // CTA -> run map of the sweep launches (a CTA holds a group or more)
     sz[S_CLNC] = (CLN_TAB + 1) * 8;
     size_t o = 0;
     for (int r = 0; r < S_COUNT; ++r) {
@@ -252,6 +250,21 @@ bool make_magic(int L, int N, uint32_t* m_out, uint32_t* sh_out) {
     return false;
 }
 
+// The column-walk sweep kernels run the glass in a gauge in which every bond along
+// the last axis is +1 except the one that wraps: spins times eps, couplings
+// J'(s, s+e_a) = eps(s) eps(s+e_a) J, the same energies and flips.  Bit 4 of byte s:
+// eps(s) = -1; bits 5, 6 (, 7): J' of the bonds to +x, +y (, +z) is -1.
+void gauge_couplings(RunHost& h, int d) {
+    const int L = h.L, N = h.N, top = N / L;  // top: sites of a layer of the last axis
+    for (int s = top; s < N; ++s)
+        if (((h.jb[s - top] >> 4) ^ (h.jb[s - top] >> (d - 1))) & 1) h.jb[s] |= 16u;
+    for (int a = 0, e = 1; a < d; ++a, e *= L)
+        for (int s = 0; s < N; ++s) {
+            const int n = (s / e) % L == L - 1 ? s - (L - 1) * e : s + e;
+            if (((h.jb[s] >> a) ^ (h.jb[s] >> 4) ^ (h.jb[n] >> 4)) & 1) h.jb[s] |= (uint8_t)(32u << a);
+        }
+}
+
 // couplings: bit a of byte s is set when the bond (s, s + e_a) has J = -1
 bool fill_couplings(RunHost& h, int d, const pa_couplings& cpl) {
     h.jb.assign((size_t)h.N, 0);
@@ -279,6 +292,7 @@ bool fill_couplings(RunHost& h, int d, const pa_couplings& cpl) {
         }
     }
     h.parity = nneg & 1;
+    gauge_couplings(h, d);
     return true;
 }
 
@@ -368,28 +382,61 @@ void fill_obs(const pa_ctx* ctx, int run, const TraceRow& t, int step, pa_obs* o
     o->theta_next = t.theta_next;
 }
 
-// The grouped 3D kernel's CTA plan for group multiple gm: for each distinct side,
-// the CTAs of its runs in run order (the CTA -> run map, from p.c3map[0] on, and
-// each run's first CTA); the side's groups per CTA are its base count times gm.
-void plan3d(pa_ctx* ctx, int gm, std::vector<uint32_t>& c3) {
+// The sweep's CTA plan for the context's threads and group multiple gm: for each
+// distinct side (one for the 2D kernel), the CTAs of its runs in run order (the CTA ->
+// run map, from `map` on, and each run's first CTA) and the launch geometry.
+void plan_sweep(pa_ctx* ctx, int gm, uint32_t* map, std::vector<uint32_t>& c3) {
     KParams& p = ctx->kp;
     c3.clear();
-    uint32_t* base3 = const_cast<uint32_t*>(p.c3map[0]);
-    for (int k = 0; k < p.n3; ++k) {
-        p.c3map[k] = base3 + c3.size();
-        const int G = sweep3d_groups(p.L3[k], gm);
+    auto place = [&](int L, int G, const uint32_t** at, uint32_t* ncta) {
+        *at = map + c3.size();
         uint32_t n = 0;
         for (int m = 0; m < (int)ctx->runs.size(); ++m) {
-            RunHost& h = ctx->runs[m];
-            if (h.L != p.L3[k]) continue;
-            h.nct3 = (h.ngrp + G - 1) / G;
+            const RunHost& h = ctx->runs[m];
+            if (h.L != L) continue;
+            const int nct = (h.ngrp + G - 1) / G;
             ctx->desc[m].cta0 = n;
-            for (int c = 0; c < h.nct3; ++c) c3.push_back((uint32_t)m);
-            n += (uint32_t)h.nct3;
+            for (int c = 0; c < nct; ++c) c3.push_back((uint32_t)m);
+            n += (uint32_t)nct;
         }
-        p.n3cta[k] = n;
-    }
+        *ncta = n;
+    };
+    const int want = ctx->auto_threads ? 0 : ctx->threads;
     p.g3mul = gm;
+    if (p.nw == 0) {
+        p.TG2 = p.d == 2 && p.L_all ? sweep2d_threads(p.L_all, want, p.ngrp_total) : 0;
+        p.G2 = p.TG2 == 0 ? 0 : std::max(1, p.TG2 <= 32 ? 128 / p.TG2 : 1);
+        if (p.G2 > 0) place(p.L_all, p.G2, &p.wmap[0], &p.wcta[0]);
+        return;
+    }
+    for (int k = 0; k < p.nw; ++k) {
+        const int L = p.wplan[k].L;
+        uint32_t all = 0, most = 0;
+        for (const RunHost& h : ctx->runs)
+            if (h.L == L) {
+                all += (uint32_t)h.ngrp;
+                most = std::max(most, (uint32_t)h.ngrp);
+            }
+        p.wplan[k] = walk_plan(p.d, L, p.ea != 0, all, most, want, gm);
+        place(L, p.wplan[k].GP * p.wplan[k].CPT, &p.wmap[k], &p.wcta[k]);
+    }
+}
+
+// rebuild the plan (after a change of threads or of the group multiple): no step in
+// flight may read the old one
+pa_status replan(pa_ctx* ctx, int gm) {
+    PA_CUDA(cudaStreamSynchronize(ctx->stream));
+    std::vector<uint32_t> c3;
+    plan_sweep(ctx, gm, ctx->d_cta, c3);
+    if (!c3.empty())
+        PA_CUDA(cudaMemcpy(ctx->d_cta, c3.data(), c3.size() * 4, cudaMemcpyHostToDevice));
+    PA_CUDA(cudaMemcpy((void*)ctx->kp.runs, ctx->desc.data(), sizeof(RunDesc) * ctx->desc.size(),
+                       cudaMemcpyHostToDevice));
+    if (ctx->graph) {  // the captured step holds the old launch configuration
+        cudaGraphExecDestroy(ctx->graph);
+        ctx->graph = nullptr;
+    }
+    return PA_OK;
 }
 
 // all kernels of one temperature step (and the controller's choice of the next)
@@ -603,8 +650,9 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
     p.alpha = -1.0;
     p.qcap_limit = -1;
     p.lb_hold = 0;
-    p.n3 = 0;
+    p.nw = 0;
     p.g3mul = 1;
+    p.G2 = 0;
     p.L_all = ctx->runs[0].L;
     for (const RunHost& h : ctx->runs)
         if (h.L != p.L_all) p.L_all = 0;
@@ -683,22 +731,24 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
     p.nblk_total = blk0;
     p.ngrp_total = grp0;
 
-    // 3D runs of sides 4..16: the grouped 3D kernel, one launch per distinct side
-    // (at most four), each over the CTAs of the runs of that side in run order
+    // The sweep's launches: the 2D kernel when all runs have one of its sides; else the
+    // column walk, one launch per distinct side (at most four), each over the CTAs of the
+    // runs of that side in run order; with more sides the general kernel.
     std::vector<uint32_t> c3;
     {
         std::vector<int> Ls;
-        bool ok = d == 3;
+        bool grouped = d == 3;  // the 3D sides whose sets of groups the caller may double
         for (const RunHost& h : ctx->runs) {
-            if (!h.g3) ok = false;
+            if (h.L < 4 || h.L > 16) grouped = false;
             if (std::find(Ls.begin(), Ls.end(), h.L) == Ls.end()) Ls.push_back(h.L);
         }
-        if (ok && Ls.size() <= 4) {
-            p.n3 = (int)Ls.size();
-            for (int k = 0; k < p.n3; ++k) p.L3[k] = Ls[k];
-            p.c3map[0] = (uint32_t*)(base + lay.shared_off[S_C3]);
-            plan3d(ctx, 1, c3);
+        ctx->grouped3 = grouped && Ls.size() <= 4;
+        if (Ls.size() <= 4 && !(d == 2 && p.L_all && sweep2d_threads(p.L_all, 0, 1) > 0)) {
+            p.nw = (int)Ls.size();
+            for (int k = 0; k < p.nw; ++k) p.wplan[k].L = Ls[k];
         }
+        ctx->d_cta = (uint32_t*)(base + lay.shared_off[S_CTA]);
+        plan_sweep(ctx, 1, ctx->d_cta, c3);
     }
 
     // per-step tables: dbeta, q = exp(-4 dbeta), Metropolis thresholds at beta_i
@@ -718,7 +768,7 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
     up(p.runs, ctx->desc.data(), sizeof(RunDesc) * M);
     up(p.blk2run, b2r.data(), b2r.size() * 4);
     up(p.grp2run, g2r.data(), g2r.size() * 4);
-    if (!c3.empty()) up(p.c3map[0], c3.data(), c3.size() * 4);
+    if (!c3.empty()) up(ctx->d_cta, c3.data(), c3.size() * 4);
     up(p.beta, ctx->beta.data(), sizeof(double) * (n + 1));
     up(p.dbeta, dbeta.data(), sizeof(double) * n);
     up(p.q, q.data(), sizeof(double) * n);
@@ -1256,35 +1306,22 @@ int64_t pa_launch_count(const pa_ctx* ctx) { return ctx ? ctx->launches : 0; }
 
 pa_status pa_set_sweep_threads(pa_ctx* ctx, int32_t threads) {
     if (!ctx || !sweep_threads_supported(threads)) return PA_ERR_ARG;
+    if (ctx->threads == threads && !ctx->auto_threads) return PA_OK;
     ctx->threads = threads;
-    if (ctx->graph) {  // the captured step holds the old launch configuration
-        cudaGraphExecDestroy(ctx->graph);
-        ctx->graph = nullptr;
-    }
-    return PA_OK;
+    ctx->auto_threads = false;
+    return replan(ctx, ctx->kp.g3mul);
 }
 
 pa_status pa_set_sweep_groups(pa_ctx* ctx, int32_t mult) {
     if (!ctx || (mult != 1 && mult != 2)) return PA_ERR_ARG;
-    if (ctx->kp.n3 == 0) return mult == 1 ? PA_OK : PA_ERR_ARG;  // no grouped 3D kernel
+    if (!ctx->grouped3) return mult == 1 ? PA_OK : PA_ERR_ARG;
     if (ctx->sticky != PA_OK) return PA_ERR_STATE;
     if (mult == ctx->kp.g3mul) return PA_OK;
-    // no step in flight may read the old plan
-    PA_CUDA(cudaStreamSynchronize(ctx->stream));
-    std::vector<uint32_t> c3;
-    plan3d(ctx, mult, c3);
-    PA_CUDA(cudaMemcpy((void*)ctx->kp.c3map[0], c3.data(), c3.size() * 4, cudaMemcpyHostToDevice));
-    PA_CUDA(cudaMemcpy((void*)ctx->kp.runs, ctx->desc.data(), sizeof(RunDesc) * ctx->desc.size(),
-                       cudaMemcpyHostToDevice));
-    if (ctx->graph) {
-        cudaGraphExecDestroy(ctx->graph);
-        ctx->graph = nullptr;
-    }
-    return PA_OK;
+    return replan(ctx, mult);
 }
 
 int32_t pa_get_sweep_groups(const pa_ctx* ctx) {
-    return ctx ? (ctx->kp.n3 ? ctx->kp.g3mul : 1) : 0;
+    return ctx ? ctx->kp.g3mul : 0;
 }
 
 int32_t pa_get_sweep_threads(const pa_ctx* ctx) { return ctx ? ctx->threads : 0; }

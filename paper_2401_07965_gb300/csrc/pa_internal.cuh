@@ -160,7 +160,7 @@ struct RunDesc {
     uint32_t blk0;           // its first block in the flattened scan grids
     uint32_t grp0;           // its first CTA in the flattened sweep grid (= slot_base / 32)
     uint32_t run;            // run index
-    uint32_t cta0;           // 3D kernel: its first CTA in the launch for its side
+    uint32_t cta0;           // column walk: its first CTA in the launch for its side
     double lnR;              // ln max(R, 2), from the host's log (the controller's entropy scale)
     uint32_t* spins[2];
     int32_t* E[2];
@@ -197,6 +197,20 @@ struct RunDesc {
     uint32_t* tick;          // [0] scan-block tickets, [1] family-block tickets
 };
 
+// Geometry of a launch of the column-walk sweep kernel (one side L).
+struct WalkPlan {
+    int L;
+    int NC;           // columns of a group
+    int H;            // rows of a column
+    int S;            // words from row to row
+    int CS, GS;       // words of a colour's array, of a group
+    int GP, CPT;      // groups side by side, sets of them per CTA
+    int NT;           // threads
+    int span;         // rows walked before the second pass (fewer than H: the list's room)
+    uint32_t mL, sL;  // division by L
+    int flat;         // nonzero: a side of pa_sweep3d.cu, GP groups per CTA
+};
+
 // Batch-wide parameters, passed by value to every kernel.
 struct KParams {
     int d, ea, method, n_steps, M;
@@ -219,12 +233,13 @@ struct KParams {
     int lb_hold;             // test: scan block 0 withholds its prefix (the waits run out)
     const double* clnc;      // c ln c for c = 0 .. CLN_TAB (0 for c < 2), from the host's log
     int L_all;               // the side L shared by every run of the batch (0 if they differ)
-    // 3D kernel plan: one launch per distinct side (n3 = 0: the general kernel)
-    int n3;
-    int L3[4];
-    int g3mul;               // groups per CTA: the side's base count times this (1 or 2)
-    const uint32_t* c3map[4];  // CTA -> run of each launch
-    uint32_t n3cta[4];
+    // column-walk plan: one launch per distinct side (nw = 0: the general kernel)
+    int nw;
+    int g3mul;                 // 3D: sets of groups per CTA, the side's count times this (1 or 2)
+    WalkPlan wplan[4];
+    int G2, TG2;               // 2D kernel (nw = 0): groups per CTA (0: the general kernel), threads of each
+    const uint32_t* wmap[4];   // CTA -> run of each launch
+    uint32_t wcta[4];
 };
 
 // partial resampling: blocks of a run whose tree sums one CTA can finish
@@ -246,11 +261,15 @@ cudaError_t launch_partial_init(const KParams& p, cudaStream_t s);
 cudaError_t launch_sweep(const KParams& p, int threads, cudaStream_t s);
 cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int64_t* launches);
 cudaError_t prepare_sweep(const KParams& p, int threads);
-cudaError_t launch_sweep2d(const KParams& p, int threads, cudaStream_t s, bool attr_only,
-                           bool* done);
+cudaError_t launch_sweep2d(const KParams& p, cudaStream_t s, bool attr_only, bool* done);
+double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT);
 int sweep3d_groups(int L, int gm);
-cudaError_t launch_sweep3d(const KParams& p, int L, const uint32_t* cta2run, uint32_t ncta,
+cudaError_t launch_sweep3d(const KParams& p, int L, int G, const uint32_t* cta2run, uint32_t ncta,
                            cudaStream_t s, bool attr_only);
+int sweep2d_threads(int L, int threads, uint32_t ngrp);
+WalkPlan walk_plan(int d, int L, bool ea, uint32_t ngrp, uint32_t most_grp, int threads, int gm);
+cudaError_t launch_walk(const KParams& p, const WalkPlan& g, const uint32_t* cta2run, uint32_t ncta,
+                        cudaStream_t s, bool attr_only);
 cudaError_t launch_control(const KParams& p, cudaStream_t s);
 int sweep_threads(int N);
 bool sweep_threads_supported(int t);

@@ -22,6 +22,8 @@
 // and M, writes the 32 rows back, adds each replica to the energy-level
 // histogram used by the next reweighting, and adds the population sums of
 // E, E^2, |M|, M^2 and the accepted flips to the step's trace row.
+#include <algorithm>
+
 #include "pa_sweep_common.cuh"
 
 namespace pa {
@@ -450,6 +452,30 @@ __global__ void __launch_bounds__(NT) k_group(KParams p, int mode) {
     }
 }
 
+// Relative time of a column-walk sweep of ngrp groups with tg threads of `regs` registers
+// each, GP groups side by side in a CTA and CPT sets of them one after the other, and
+// `rows` rows per thread between two second passes.  An SM
+// with w warps per scheduler works at the rate w / (w + 1.6); up to three rounds of the
+// groups that the 152 SMs hold take as long as the rounds of the fullest SM, more take the
+// average load and a part of a round; lanes past the last column and few rows cost their
+// share: few rows leave the second pass's rounds part empty and repeat its set-up.  Fitted
+// to 2D L = 32, 625 groups (16, 8, 4, 2 rows: 1737, 2423, 2762, 2247 updates/ns) and 3125
+// groups (3490, 3877, 3725) and L = 64, 94 groups (16, 8, 4 rows: 1243, 1823, 1919), 625
+// (3329, 3208, 2640) and 3125 (4669, 4352, 3512); it takes the best of each.
+double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT) {
+    const double er = rows >= 16 ? 1.0 : rows >= 12 ? 0.97 : rows >= 8 ? 0.93 : rows >= 6 ? 0.9
+                      : rows >= 4 ? 0.85 : rows >= 2 ? 0.65 : 0.45;
+    const int G = GP * CPT, nt = std::max(32, (GP * tg + 31) / 32 * 32);
+    const int hold = std::max(1, std::min(32, 65536 / (nt * regs))) * G;  // groups an SM holds
+    const int ncta = (int)((ngrp + G - 1) / G);
+    const int most = std::min<int>((ncta + 151) / 152 * G, (int)ngrp);
+    auto round = [&](double n) { return n > 0.0 ? n + 1.6 * 128.0 * CPT / tg : 0.0; };  // n at once
+    const double t = most <= 3 * hold
+                         ? most / hold * round(hold) + round(most % hold)
+                         : (ngrp / 152.0 + 0.3 * hold) * round(hold) / hold;
+    return t / er * nt / (GP * tg);
+}
+
 int sweep_threads(int N) {
     const int sites = N / 2;  // per colour
     int t = 64;
@@ -520,10 +546,10 @@ static cudaError_t prepare_t(int threads) {
 // one-time function attributes, outside any stream capture
 cudaError_t prepare_sweep(const KParams& p, int threads) {
     bool done = false;
-    cudaError_t e = launch_sweep2d(p, threads, nullptr, true, &done);
+    cudaError_t e = launch_sweep2d(p, nullptr, true, &done);
     if (e != cudaSuccess) return e;
-    for (int k = 0; k < p.n3 && e == cudaSuccess; ++k)
-        e = launch_sweep3d(p, p.L3[k], p.c3map[k], p.n3cta[k], nullptr, true);
+    for (int k = 0; k < p.nw && e == cudaSuccess; ++k)
+        e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], nullptr, true);
     if (e != cudaSuccess) return e;
     if (p.d == 2) return p.ea ? prepare_t<2, true>(threads) : prepare_t<2, false>(threads);
     return p.ea ? prepare_t<3, true>(threads) : prepare_t<3, false>(threads);
@@ -545,14 +571,14 @@ cudaError_t launch_measure(const KParams& p, int threads, cudaStream_t s) {
 }
 
 cudaError_t launch_sweep(const KParams& p, int threads, cudaStream_t s) {
-    if (p.n3 > 0) {  // 3D runs of sides 4..16: one launch per side
+    if (p.nw > 0) {  // the column walk: one launch per side
         cudaError_t e = cudaSuccess;
-        for (int k = 0; k < p.n3 && e == cudaSuccess; ++k)
-            e = launch_sweep3d(p, p.L3[k], p.c3map[k], p.n3cta[k], s, false);
+        for (int k = 0; k < p.nw && e == cudaSuccess; ++k)
+            e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], s, false);
         return e;
     }
     bool done = false;
-    const cudaError_t e = launch_sweep2d(p, threads, s, false, &done);
+    const cudaError_t e = launch_sweep2d(p, s, false, &done);
     if (e != cudaSuccess || done) return e;
     return launch_group(p, 0, threads, s);
 }

@@ -1,12 +1,13 @@
 // pa_sweep3d.cu -- the temperature step's replica copy, theta checkerboard
 // Metropolis sweeps and measurement (Sec. 2 steps 2-4) for three-dimensional
-// runs of side 4 <= L <= 16: the work of k_group's sweep mode with a layout for
-// small lattices.  Random numbers, decisions and results are the same.
+// runs of side 10, 12 and 14 (the other sides take the column walk of pa_sweepw.cu,
+// whose columns fill whole warps there): the work of k_group's sweep mode with a layout
+// for small lattices.  Random numbers, decisions and results are the same.
 //
 // Grouping.  A 3D lattice of a few hundred sites gives one group of 32 replicas
 // too little work per half-sweep (and per barrier, and per flush of the queue
 // of undecided sites), so a CTA of 128 threads holds G replica groups of one
-// run (G = 16, 8, 4, 2 for L = 4, 6, 8, 10; 1 above), about eight site words
+// run (G = 2 for L = 10; 1 above), about eight site words
 // per thread and half-sweep: G halo-padded multi-spin lattices in shared
 // memory (cell (x, y, z), -1 <= x, y, z <= L, word ((z+1)(L+2) + y+1)(L+2) +
 // x+1), each group keeping its own Philox counter (its global replica group).
@@ -40,7 +41,7 @@ constexpr int NT3 = 128;
 // replica groups per CTA of side L
 template <int L>
 struct Groups3 {
-    static constexpr int value = L == 4 ? 16 : (L == 6 ? 8 : (L == 8 ? 4 : (L == 10 ? 2 : 1)));
+    static constexpr int value = L == 10 ? 2 : 1;
 };
 
 // GM: a multiple of the base group count (the autotuner may double it)
@@ -629,26 +630,18 @@ template <bool EA, int GM>
 cudaError_t launch3d_L(int L, const KParams& p, const uint32_t* cta2run, uint32_t ncta,
                        cudaStream_t s, bool attr_only) {
     switch (L) {
-        case 4: return launch3d<4, EA, GM>(p, cta2run, ncta, s, attr_only);
-        case 6: return launch3d<6, EA, GM>(p, cta2run, ncta, s, attr_only);
-        case 8: return launch3d<8, EA, GM>(p, cta2run, ncta, s, attr_only);
         case 10: return launch3d<10, EA, GM>(p, cta2run, ncta, s, attr_only);
         case 12: return launch3d<12, EA, GM>(p, cta2run, ncta, s, attr_only);
-        case 14: return launch3d<14, EA, GM>(p, cta2run, ncta, s, attr_only);
-        default: return launch3d<16, EA, GM>(p, cta2run, ncta, s, attr_only);
+        default: return launch3d<14, EA, GM>(p, cta2run, ncta, s, attr_only);
     }
 }
 
 template <int GM>
 int groups_L(int L) {
     switch (L) {
-        case 4: return Shape3<4, GM>::G;
-        case 6: return Shape3<6, GM>::G;
-        case 8: return Shape3<8, GM>::G;
         case 10: return Shape3<10, GM>::G;
         case 12: return Shape3<12, GM>::G;
         case 14: return Shape3<14, GM>::G;
-        case 16: return Shape3<16, GM>::G;
         default: return 0;
     }
 }
@@ -662,9 +655,9 @@ int sweep3d_groups(int L, int gm) { return gm == 2 ? groups_L<2>(L) : groups_L<1
 // One launch of the 3D kernel over the CTAs of the runs of side L (cta2run: their
 // run indices, device memory), with the context's group multiple.  attr_only:
 // function attributes only (before a stream capture).
-cudaError_t launch_sweep3d(const KParams& p, int L, const uint32_t* cta2run, uint32_t ncta,
+cudaError_t launch_sweep3d(const KParams& p, int L, int G, const uint32_t* cta2run, uint32_t ncta,
                            cudaStream_t s, bool attr_only) {
-    if (p.g3mul == 2)
+    if (G != groups_L<1>(L))
         return p.ea ? launch3d_L<true, 2>(L, p, cta2run, ncta, s, attr_only)
                     : launch3d_L<false, 2>(L, p, cta2run, ncta, s, attr_only);
     return p.ea ? launch3d_L<true, 1>(L, p, cta2run, ncta, s, attr_only)
