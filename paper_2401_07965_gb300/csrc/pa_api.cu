@@ -75,6 +75,8 @@ struct pa_ctx {
     cudaGraphExec_t graph = nullptr;
     int graph_threads = 0;
     int64_t graph_kernels = 0;
+    cudaStream_t cap = nullptr, side = nullptr;  // the captured step and its branch
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::vector<cudaEvent_t> ev_start, ev_stop;  // pool of timing events, reused
     size_t ev_used = 0;
     std::vector<int> timed_steps;
@@ -439,13 +441,55 @@ pa_status replan(pa_ctx* ctx, int gm) {
     return PA_OK;
 }
 
-// all kernels of one temperature step (and the controller's choice of the next)
-pa_status enqueue_step(pa_ctx* ctx, int64_t* launches) {
-    PA_CUDA(launch_resample(ctx->kp, ctx->stream, launches));
-    PA_CUDA(launch_sweep(ctx->kp, ctx->threads, ctx->stream));
+// n more start/stop event pairs for timing mode (created outside the timed steps)
+pa_status grow_event_pool(pa_ctx* ctx, size_t n) {
+    for (size_t k = 0; k < n; ++k) {
+        cudaEvent_t a = nullptr, b = nullptr;
+        PA_CUDA(cudaEventCreate(&a));
+        if (cudaEventCreate(&b) != cudaSuccess) {
+            cudaEventDestroy(a);
+            ctx->sticky = PA_ERR_CUDA;
+            return PA_ERR_CUDA;
+        }
+        ctx->ev_start.push_back(a);
+        ctx->ev_stop.push_back(b);
+    }
+    return PA_OK;
+}
+
+// All kernels of one temperature step (and the controller's choice of the next).  The
+// family statistics need the ancestors only: while a step is captured they go to a
+// branch beside the sweep (side != nullptr).  Under partial resampling they carry
+// weighted sums of the sweep's energies and follow it.
+pa_status enqueue_step(pa_ctx* ctx, int64_t* launches, cudaStream_t stream,
+                       cudaStream_t side) {
+    const bool partial = ctx->kp.alpha >= 0.0;
+    PA_CUDA(launch_resample(ctx->kp, stream, launches));
+    if (!partial) {
+        if (side) {
+            PA_CUDA(cudaEventRecord(ctx->ev_fork, stream));
+            PA_CUDA(cudaStreamWaitEvent(side, ctx->ev_fork, 0));
+        }
+        PA_CUDA(launch_family_finish(ctx->kp, 0, side ? side : stream, launches));
+        if (side) PA_CUDA(cudaEventRecord(ctx->ev_join, side));
+    }
+    const bool timed = ctx->timing && !side;
+    if (timed) {
+        if (ctx->ev_used == ctx->ev_start.size()) {
+            const pa_status ps = grow_event_pool(ctx, 1);
+            if (ps != PA_OK) return ps;
+        }
+        PA_CUDA(cudaEventRecord(ctx->ev_start[ctx->ev_used], stream));
+    }
+    PA_CUDA(launch_sweep(ctx->kp, ctx->threads, stream));
     if (launches) *launches += 1;
-    // the family kernel's last CTA of each run also takes the controller's decision
-    PA_CUDA(launch_family_finish(ctx->kp, 0, ctx->stream, launches));
+    if (timed) PA_CUDA(cudaEventRecord(ctx->ev_stop[ctx->ev_used++], stream));
+    if (partial) PA_CUDA(launch_family_finish(ctx->kp, 0, stream, launches));
+    else if (side) PA_CUDA(cudaStreamWaitEvent(stream, ctx->ev_join, 0));
+    if (ctx->kp.ctl) {
+        PA_CUDA(launch_control(ctx->kp, stream));
+        if (launches) *launches += 1;
+    }
     return PA_OK;
 }
 
@@ -490,11 +534,22 @@ pa_status build_graph(pa_ctx* ctx) {
         ctx->graph = nullptr;
     }
     PA_CUDA(prepare_sweep(ctx->kp, ctx->threads));
+    if (!ctx->side) {
+        int least = 0, greatest = 0;
+        PA_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+        PA_CUDA(cudaStreamCreateWithPriority(&ctx->cap, cudaStreamNonBlocking, greatest));
+        PA_CUDA(cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, least));
+        PA_CUDA(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
+        PA_CUDA(cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming));
+    }
     cudaGraph_t g = nullptr;
-    PA_CUDA(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
+    // captured on streams of the context's own, whose priorities go to the kernels: the
+    // sweep's CTAs are placed before those of the family branch, which would otherwise
+    // take their places on some SMs and leave the sweep unevenly spread
+    PA_CUDA(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
     int64_t n = 0;
-    const pa_status s = enqueue_step(ctx, &n);
-    const cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
+    const pa_status s = enqueue_step(ctx, &n, ctx->cap, ctx->side);
+    const cudaError_t e = cudaStreamEndCapture(ctx->cap, &g);
     if (s != PA_OK) {
         if (g) cudaGraphDestroy(g);
         return s;
@@ -527,22 +582,6 @@ bool valid_schedule(const pa_schedule* sched) {
 }
 
 bool valid_run(const pa_ctx* ctx, int run) { return ctx && run >= 0 && run < ctx->M; }
-
-// n more start/stop event pairs for timing mode (created outside the timed steps)
-pa_status grow_event_pool(pa_ctx* ctx, size_t n) {
-    for (size_t k = 0; k < n; ++k) {
-        cudaEvent_t a = nullptr, b = nullptr;
-        PA_CUDA(cudaEventCreate(&a));
-        if (cudaEventCreate(&b) != cudaSuccess) {
-            cudaEventDestroy(a);
-            ctx->sticky = PA_ERR_CUDA;
-            return PA_ERR_CUDA;
-        }
-        ctx->ev_start.push_back(a);
-        ctx->ev_stop.push_back(b);
-    }
-    return PA_OK;
-}
 
 }  // namespace
 
@@ -851,22 +890,9 @@ pa_status pa_step(pa_ctx* ctx, int32_t n) {
         if (graph) {
             PA_CUDA(cudaGraphLaunch(ctx->graph, ctx->stream));
             ctx->launches += ctx->graph_kernels;
-        } else if (ctx->timing) {
-            PA_CUDA(launch_resample(ctx->kp, ctx->stream, &ctx->launches));
-            if (ctx->ev_used == ctx->ev_start.size()) {
-                const pa_status ps = grow_event_pool(ctx, 1);
-                if (ps != PA_OK) return ps;
-            }
-            cudaEvent_t a = ctx->ev_start[ctx->ev_used], b = ctx->ev_stop[ctx->ev_used];
-            ctx->ev_used += 1;
-            ctx->timed_steps.push_back(i);
-            PA_CUDA(cudaEventRecord(a, ctx->stream));
-            PA_CUDA(launch_sweep(ctx->kp, ctx->threads, ctx->stream));
-            ctx->launches += 1;
-            PA_CUDA(cudaEventRecord(b, ctx->stream));
-            PA_CUDA(launch_family_finish(ctx->kp, 0, ctx->stream, &ctx->launches));
         } else {
-            const pa_status s = enqueue_step(ctx, &ctx->launches);
+            if (ctx->timing) ctx->timed_steps.push_back(i);
+            const pa_status s = enqueue_step(ctx, &ctx->launches, ctx->stream, nullptr);
             if (s != PA_OK) return s;
         }
         ctx->host_step = i;
@@ -1353,6 +1379,10 @@ pa_status pa_destroy(pa_ctx* ctx) {
         cudaEventDestroy(ctx->ev_stop[k]);
     }
     if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
+    if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
+    if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+    if (ctx->cap) cudaStreamDestroy(ctx->cap);
+    if (ctx->side) cudaStreamDestroy(ctx->side);
     if (ctx->owns && ctx->ws) cudaFree(ctx->ws);
     delete ctx;
     return PA_OK;

@@ -1,8 +1,7 @@
 // pa_control.cuh -- the learned schedule controller's step (adaptive temperature
 // steps and sweep numbers, cited as established practice in Sec. 5 of the
-// paper), shared by the kernel that makes the first decision of a run and by
-// the family kernel, whose last CTA of a run makes the decision after every
-// step (one kernel boundary less per step).
+// paper), run by k_control for the first decision of a run and after every step (when the
+// sweep and the family statistics beside it are done).
 //
 // Network: 8 population statistics -> 64 -> 64 -> 2 (ReLU), BF16 parameters,
 // FP32 accumulation in a fixed order (bias added last), no fused multiply-add.

@@ -100,7 +100,7 @@ __device__ __forceinline__ void mulhilo(uint32_t a, uint32_t b, uint32_t& hi, ui
 
 // Device state shared by the kernels of a run (one per context).
 struct DevState {
-    int32_t step;      // completed temperature steps
+    int32_t step;      // completed temperature steps; during a step its index (k_weights)
     int32_t status;    // DevStatus
     uint32_t R_cur;    // current population size
     uint32_t R_prev;   // size that the last resampling started from
@@ -263,6 +263,7 @@ cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int
 cudaError_t prepare_sweep(const KParams& p, int threads);
 cudaError_t launch_sweep2d(const KParams& p, cudaStream_t s, bool attr_only, bool* done);
 double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT);
+size_t spread_smem(size_t sm, uint32_t ncta, int nt, int regs);
 int sweep3d_groups(int L, int gm);
 cudaError_t launch_sweep3d(const KParams& p, int L, int G, const uint32_t* cta2run, uint32_t ncta,
                            cudaStream_t s, bool attr_only);

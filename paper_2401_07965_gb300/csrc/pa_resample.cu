@@ -21,7 +21,7 @@
 // and its weight is rescaled by a power of two (k_family).
 #include <climits>
 
-#include "pa_control.cuh"
+#include "pa_internal.cuh"
 
 namespace pa {
 
@@ -227,6 +227,7 @@ __global__ void __launch_bounds__(1024) k_weights(KParams p) {
         __syncthreads();
         for (int k = threadIdx.x; k < K; k += blockDim.x) r.hist[lmin + k] = 0u;
         if (threadIdx.x == 0) {
+            st->step = i;  // the step's other kernels read its index here
             st->R_prev = Rprev;
             st->lmin = (uint32_t)lmin;
             st->K = (uint32_t)K;
@@ -321,6 +322,7 @@ __global__ void __launch_bounds__(1024) k_weights(KParams p) {
     __syncthreads();
     for (int k = threadIdx.x; k < K; k += blockDim.x) r.hist[lmin + k] = 0u;
     if (threadIdx.x == 0) {
+        st->step = i;  // the step's other kernels read its index here
         st->T = tsum[0];
         st->Tres = tsum[1];
         st->Rres = (uint64_t)r.R - ((tsum[0] - tsum[1]) >> FRAC_BITS);
@@ -356,7 +358,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_pw_update(KParams p) {
     const DevState* st = r.st;
     if (st->status != S_OK) return;
     __shared__ double sh[SCAN_THREADS];
-    const int i = st->step + 1;
+    const int i = st->step;
     const int32_t* E = r.E[(i - 1) & 1];
     const uint32_t Rprev = st->R_prev, lmin = st->lmin;
     const int dN = p.d * r.N;
@@ -394,7 +396,7 @@ __global__ void __launch_bounds__(1024) k_pw_final(KParams p) {
     DevState* st = r.st;
     if (st->status != S_OK) return;
     __shared__ double sh[1024];
-    const int i = st->step + 1;
+    const int i = st->step;
     const int nb = r.nblk;  // <= PARTIAL_MAX_BLOCKS = LEAVES leaves x 1024 threads
     constexpr int LEAVES = PARTIAL_MAX_BLOCKS / 1024;
     double S[3];
@@ -465,7 +467,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_fsum(KParams p) {
     if (st->status != S_OK) return;
     if (p.alpha >= 0.0 && !st->resample) return;  // partial: population kept
     __shared__ uint64_t sh[33];
-    const int i = st->step + 1;
+    const int i = st->step;
     const int32_t* E = r.E[(i - 1) & 1];
     const uint32_t Rprev = st->R_prev, lmin = st->lmin;
     const int dN = p.d * r.N;
@@ -540,7 +542,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_counts(KParams p) {
     DevState* st = r.st;
     if (st->status != S_OK) return;
     __shared__ uint64_t sh[33];
-    const int i = st->step + 1;
+    const int i = st->step;
     const int32_t* E = r.E[(i - 1) & 1];
     const int dN = p.d * r.N;
     const uint32_t Rprev = st->R_prev, lmin = st->lmin;
@@ -554,6 +556,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_counts(KParams p) {
             if ((uint32_t)j < Rprev) {
                 r.counts[j] = 1u;
                 r.anc[j] = (uint32_t)j;
+                r.fam[i & 1][j] = r.fam[(i - 1) & 1][j];
             }
         }
         if (threadIdx.x == 0) r.partD[b] = 0.0;
@@ -634,7 +637,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_draws(KParams p) {
     const DevState* st = r.st;
     if (st->status != S_OK) return;
     if (p.alpha >= 0.0 && !st->resample) return;  // partial: no resampling this step
-    const int i = st->step + 1;
+    const int i = st->step;
     const uint32_t Rprev = st->R_prev;
     uint64_t n;
     const uint64_t* box;
@@ -713,7 +716,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scatter(KParams p) {
     if (p.alpha >= 0.0 && !st->resample) return;  // identity written by k_counts
     __shared__ uint64_t sh[33];
     __shared__ double sd[SCAN_THREADS];
-    const int i = st->step + 1;
+    const int i = st->step;
     const int32_t* E = r.E[(i - 1) & 1];
     const int dN = p.d * r.N;
     const uint32_t Rprev = st->R_prev, lmin = st->lmin;
@@ -732,7 +735,11 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scatter(KParams p) {
     for (int e = 0; e < SCAN_ITEMS; ++e) {
         const int j = j0 + e;
         if ((uint32_t)j >= Rprev) break;
-        for (uint32_t c = 0; c < rc[e]; ++c) r.anc[o + c] = (uint32_t)j;
+        const uint32_t fj = rc[e] ? r.fam[(i - 1) & 1][j] : 0u;
+        for (uint32_t c = 0; c < rc[e]; ++c) {
+            r.anc[o + c] = (uint32_t)j;
+            r.fam[i & 1][o + c] = fj;
+        }
         o += rc[e];
         const double tau = scalbn((double)f_of(j, p, r, st, dN, E, lmin), -FRAC_BITS);
         const double dl = __dsub_rn((double)rc[e], tau);
@@ -755,10 +762,10 @@ template <bool PARTIAL>
 __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int mode, double* a,
                            double* b, double* ws);
 
-// PARTIAL: partial resampling (weighted sums); CTL: the run's last CTA then
-// takes the learned controller's decision for the next step.  Separate
-// instances keep the registers of the plain step's kernel low.
-template <bool PARTIAL, bool CTL>
+// Without partial resampling everything here is known once the ancestors are, so the
+// kernel runs beside the step's sweep (a branch of the captured step).  PARTIAL: partial
+// resampling, after the sweep (weighted sums of its energies).
+template <bool PARTIAL>
 __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
     const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
     const uint32_t b = blockIdx.x - r.blk0;
@@ -767,7 +774,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
     __shared__ double sd[SCAN_THREADS], fa[SCAN_THREADS], fb[SCAN_THREADS];
     __shared__ unsigned long long sc2;
     __shared__ int last;
-    const int i = (mode == 0) ? st->step + 1 : st->step;
+    const int i = st->step;
     const uint32_t Ri = st->R_cur;
     const uint32_t* fam = r.fam[i & 1];
     const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
@@ -904,10 +911,6 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
     if (threadIdx.x == 0) r.tick[1] = 0u;
     __threadfence();
     finish_run<PARTIAL>(p, r, st, mode, fa, fb, sd);
-    if (CTL && mode == 0) {
-        __syncthreads();  // the trace row and the step count are written
-        control_after_step(p, r, st);
-    }
 }
 
 // fixed-order sums of the run's per-block partials, close the step (one CTA of
@@ -915,7 +918,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
 template <bool PARTIAL>
 __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int mode, double* a,
                            double* b, double* ws) {
-    const int i = (mode == 0) ? st->step + 1 : st->step;
+    const int i = st->step;
     const int nb_sv = (mode == 0) ? (int)((st->R_prev + SCAN_CHUNK - 1) / SCAN_CHUNK) : 0;
     const int nb_f = (int)((st->R_cur + SCAN_CHUNK - 1) / SCAN_CHUNK);
     double sa = 0.0, sb = 0.0;
@@ -956,8 +959,7 @@ __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int
         tr->sv_sum = a[0];
         tr->c_ln_c = b[0];
         tr->R_i = st->R_cur;
-        if (mode == 0) st->step = i;
-        else tr->R_prev = st->R_cur;
+        if (mode != 0) tr->R_prev = st->R_cur;
     }
 }
 
@@ -1065,7 +1067,7 @@ __device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDe
                                                    const uint32_t (&rc)[SCAN_ITEMS], uint64_t* sh,
                                                    double* sd, int* flag_sh,
                                                    const uint64_t (&fv)[SCAN_ITEMS], bool have_f) {
-    const int i = st->step + 1;
+    const int i = st->step;
     const int32_t* E = r.E[(i - 1) & 1];
     const int dN = p.d * r.N;
     const uint32_t Rprev = st->R_prev, lmin = st->lmin;
@@ -1089,21 +1091,55 @@ __device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDe
         if (threadIdx.x == 0) atomicCAS(&st->status, S_OK, S_TIMEOUT);
         return;
     }
-    uint64_t o = pre + ex;
+    // The block's slots [pre, pre + tot): the total over blocks is known only to the last
+    // block, so slots past the capacity are not written (the last block then stops the run
+    // with the capacity error).
+    const uint32_t* fam0 = r.fam[(i - 1) & 1];
+    uint32_t* fam1 = r.fam[i & 1];
+    const uint64_t room = pre < (uint64_t)r.Rcap ? (uint64_t)r.Rcap - pre : 0ull;
+    const uint32_t nslot = (uint32_t)(tot < room ? tot : room);
+    __shared__ uint32_t so[SCAN_CHUNK], sfam[SCAN_CHUNK];  // first slot and family of each parent
+    uint32_t o = (uint32_t)(ex < 0xFFFFFFFFull ? ex : 0xFFFFFFFFull);
     double sv = 0.0;
+    int skew = 0;
 #pragma unroll
     for (int e = 0; e < SCAN_ITEMS; ++e) {
-        const int j = j0 + e;
-        if ((uint32_t)j >= Rprev) break;
-        // the total is known only to the last block: slots past the capacity are
-        // not written (the last block then stops the run with the capacity error)
-        for (uint32_t c = 0; c < rc[e]; ++c)
-            if (o + c < (uint64_t)r.Rcap) r.anc[o + c] = (uint32_t)j;
+        const int j = j0 + e, l = threadIdx.x * SCAN_ITEMS + e;
+        const bool in = (uint32_t)j < Rprev;
+        so[l] = o;
+        sfam[l] = in && rc[e] ? fam0[j] : 0u;
         o += rc[e];
+        skew |= rc[e] > 4u;
+        if (!in) continue;
         const double tau =
             scalbn((double)(have_f ? fv[e] : f_of(j, p, r, st, dN, E, lmin)), -FRAC_BITS);
         const double dl = __dsub_rn((double)rc[e], tau);
         sv = __dadd_rn(sv, __dmul_rn(dl, dl));
+    }
+    // Parents of at most four copies write their slots themselves; a block with a larger
+    // one gives every slot a thread, which finds its parent in the offsets (a thread that
+    // wrote hundreds of copies one by one held up its block and, by the look-back, the
+    // run: +-J L = 4, 6, 8, R = 50000, beta step 0.15: 499 -> 89 us for 24 runs).
+    if (!__syncthreads_or(skew)) {
+#pragma unroll
+        for (int e = 0; e < SCAN_ITEMS; ++e) {
+            const int l = threadIdx.x * SCAN_ITEMS + e;
+#pragma unroll
+            for (uint32_t c = 0; c < 4u; ++c)
+                if (c < rc[e] && so[l] + c < nslot) {
+                    r.anc[pre + so[l] + c] = (uint32_t)(j0 + e);
+                    fam1[pre + so[l] + c] = sfam[l];
+                }
+        }
+    } else {
+        for (uint32_t q = threadIdx.x; q < nslot; q += SCAN_THREADS) {
+            int lo = 0;  // the last parent whose first slot is not after q
+#pragma unroll
+            for (int w = SCAN_CHUNK / 2; w >= 1; w >>= 1)
+                if (so[lo + w] <= q) lo += w;
+            r.anc[pre + q] = (uint32_t)(b * SCAN_CHUNK + lo);
+            fam1[pre + q] = sfam[lo];
+        }
     }
     // fixed-order tree reduction of the block's sampling-variance terms
     sd[threadIdx.x] = sv;
@@ -1138,7 +1174,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
     __shared__ int sb, okf;
     __shared__ unsigned long long pre[2];
     const int b = take_ticket(&r.tick[0], &sb);
-    const int i = st->step + 1;
+    const int i = st->step;
     const int32_t* E = r.E[(i - 1) & 1];
     const int dN = p.d * r.N;
     const uint32_t Rprev = st->R_prev, lmin = st->lmin;
@@ -1303,9 +1339,8 @@ cudaError_t launch_partial_init(const KParams& p, cudaStream_t s) {
 }
 
 cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int64_t* launches) {
-    if (p.alpha >= 0.0) k_family<true, false><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode);
-    else if (p.ctl) k_family<false, true><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode);
-    else k_family<false, false><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode);
+    if (p.alpha >= 0.0) k_family<true><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode);
+    else k_family<false><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode);
     if (launches) *launches += 1;
     return cudaGetLastError();
 }

@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(NT) k_group(KParams p, int mode) {
 
     const DevState* st = r.st;
     if (st->status != S_OK) return;
-    const int i = (mode == 0) ? st->step + 1 : st->step;
+    const int i = st->step;
     const uint32_t R = st->R_cur;
     const uint32_t base = (blockIdx.x - r.grp0) * 32u;
     if (base >= R) return;
@@ -244,7 +244,6 @@ __global__ void __launch_bounds__(NT) k_group(KParams p, int mode) {
     const bool valid = (uint32_t)lane < nval;
     uint32_t my_src = base + lane;
     if (mode == 0 && valid) my_src = r.anc[base + lane];
-    if (mode == 0 && warp == 0 && valid) r.fam[i & 1][base + lane] = r.fam[(i - 1) & 1][my_src];
 
     // gather the 32 parent rows and transpose them into the multi-spin layout
     for (int c4 = warp; 4 * c4 < W; c4 += nwarp) {
@@ -474,6 +473,19 @@ double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT) {
                          ? most / hold * round(hold) + round(most % hold)
                          : (ngrp / 152.0 + 0.3 * hold) * round(hold) / hold;
     return t / er * nt / (GP * tg);
+}
+
+// Dynamic shared memory for a sweep launch of ncta CTAs of nt threads (regs registers each)
+// that need sm bytes.  A launch that the 152 SMs hold at once ends with its fullest SM, and
+// beside another kernel (the family branch) its CTAs are not spread evenly: it asks for so
+// much that no SM takes more than its share (+-J L = 48, 626 CTAs where 7 fit an SM: the
+// step 249 us without, 227 us with the limit), less 8 KB for the other kernel.
+size_t spread_smem(size_t sm, uint32_t ncta, int nt, int regs) {
+    constexpr size_t SM_BYTES = 227 * 1024, FIXED = 2560;  // static part and the system's
+    const size_t fit = std::min<size_t>(65536 / (size_t)(nt * regs), SM_BYTES / (sm + FIXED));
+    const size_t want = (ncta + 151) / 152;
+    if (want == 0 || want >= fit) return sm;
+    return std::max(sm, std::min<size_t>((SM_BYTES - 8192) / want - FIXED, SM_BYTES - 8192 - FIXED));
 }
 
 int sweep_threads(int N) {

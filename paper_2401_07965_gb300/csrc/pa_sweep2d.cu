@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
     const RunDesc& r = p.runs[cta2run[blockIdx.x]];
     const DevState* st = r.st;
     if (st->status != S_OK) return;
-    const int i = st->step + 1;
+    const int i = st->step;
     const uint32_t R = st->R_cur;
     const uint32_t gfirst = (blockIdx.x - r.cta0) * G;  // the CTA's first group in its run
     if (gfirst * 32u >= R) return;
@@ -104,8 +104,6 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
     for (int k = threadIdx.x; k < G * 32; k += NT) {
         sU[k >> 5][k & 31] = 0;
         sNup[k >> 5][k & 31] = 0;
-        const uint32_t slot = gfirst * 32u + k;  // families of the new slots
-        if (slot < R) r.fam[i & 1][slot] = r.fam[(i - 1) & 1][r.anc[slot]];
     }
     uint2* list = lists + warp * S2::QW;
     const uint32_t list0 = (uint32_t)__cvta_generic_to_shared(list);
@@ -394,24 +392,26 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
     add_to_trace(sums, r, i);
 }
 
-// dynamic shared memory a CTA may take (the opt-in limit less the kernel's static part)
-constexpr size_t SMEM2D_MAX = 227 * 1024 - 4096;
+// dynamic shared memory a CTA of G groups may take (the opt-in limit less the static part)
+constexpr size_t smem2d_max(int G) { return 227 * 1024 - 2048 - 520 * (size_t)G; }
 
 template <int L, int NT, int G, bool EA>
 cudaError_t launch2d(const KParams& p, const uint32_t* cta2run, uint32_t ncta, cudaStream_t s,
                      bool attr_only) {
     constexpr size_t sm = Shape2<L, NT, G, EA>::SMEM;
-    static_assert(sm <= SMEM2D_MAX, "2D sweep shared memory");
+    static_assert(sm <= smem2d_max(G), "2D sweep shared memory");
     constexpr int MINB = 65536 / (NT * 96);
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(k_sweep2d<L, NT, G, EA, MINB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem2d_max(G));
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     if (attr_only || ncta == 0) return cudaSuccess;
-    k_sweep2d<L, NT, G, EA, MINB><<<ncta, NT, sm, s>>>(p, cta2run);
+    k_sweep2d<L, NT, G, EA, MINB>
+        <<<ncta, NT, spread_smem(sm, ncta, NT, NT == 512 ? 128 : 96), s>>>(p, cta2run);
     return cudaGetLastError();
 }
 

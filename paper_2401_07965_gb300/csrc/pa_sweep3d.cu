@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(NT3, 6) k_sweep3d(KParams p, const uint32_t* c
     const RunDesc& r = p.runs[cta2run[blockIdx.x]];
     const DevState* st = r.st;
     if (st->status != S_OK) return;
-    const int i = st->step + 1;
+    const int i = st->step;
     const uint32_t R = st->R_cur;
     const uint32_t gfirst = (blockIdx.x - r.cta0) * G;   // the CTA's first group in its run
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -359,11 +359,6 @@ __global__ void __launch_bounds__(NT3, 6) k_sweep3d(KParams p, const uint32_t* c
         sNup[k >> 5][k & 31] = 0;
     }
     if (threadIdx.x == 0) sAcc = 0ull;
-    // families of the new slots
-    for (int k = threadIdx.x; k < G * 32; k += NT3) {
-        const uint32_t slot = (gfirst + (k >> 5)) * 32u + (k & 31);
-        if (slot < R) r.fam[i & 1][slot] = r.fam[(i - 1) & 1][r.anc[slot]];
-    }
     // gather the parent rows of every group and transpose them into the multi-spin form
     for (int k = warp; k < G * (WP / 4); k += NW) {
         const int g = k / (WP / 4), c4 = k % (WP / 4);

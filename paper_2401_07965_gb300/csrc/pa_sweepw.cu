@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
     const RunDesc& r = p.runs[cta2run[blockIdx.x]];
     const DevState* st = r.st;
     if (st->status != S_OK) return;
-    const int i = st->step + 1;
+    const int i = st->step;
     const uint32_t R = st->R_cur;
     const uint32_t gfirst = (blockIdx.x - r.cta0) * (uint32_t)G;
     if (gfirst * 32u >= R) return;
@@ -167,11 +167,7 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
         return ((x + y + z) & 1) * CS + z * S + y * TPR + (x >> 1);
     };
 
-    // families of the new slots; Philox parts of the step and the groups
-    for (int k = tid; k < gact * 32; k += NT) {
-        const uint32_t slot = gfirst * 32u + k;
-        if (slot < R) r.fam[i & 1][slot] = r.fam[(i - 1) & 1][r.anc[slot]];
-    }
+    // Philox parts of the step and the groups
     uint32_t B1k, h1a;
     {
         uint32_t l1a;
@@ -570,7 +566,8 @@ cudaError_t launch_walk_t(const KParams& p, const WalkPlan& g, const uint32_t* c
         attr_set = true;
     }
     if (attr_only || ncta == 0) return cudaSuccess;
-    k_walk<D, LT, EA><<<ncta, g.NT, walk_smem(g, D, EA).total, s>>>(p, g, cta2run);
+    const size_t sm = spread_smem((size_t)walk_smem(g, D, EA).total, ncta, g.NT, 96);
+    k_walk<D, LT, EA><<<ncta, g.NT, sm, s>>>(p, g, cta2run);
     return cudaGetLastError();
 }
 
