@@ -6,6 +6,7 @@
 // tree) lives in one file-scope __device__ array, so the call allocates
 // nothing.  The arithmetic is the one of the context path's weights kernel,
 // operation for operation, so both give the same bits.
+#include <algorithm>
 #include <cmath>
 
 #include "../../include/pa.h"
@@ -14,110 +15,182 @@
 namespace {
 
 constexpr int STATIC_MAX_LEVELS = 65536;  // d*N/2 + 1 <= 65536 energy levels
-constexpr int STATIC_THREADS = 1024;
+constexpr int STATIC_THREADS = 512;
 
+// zero at load time and between calls, except flev, tree and the call's results
 struct StaticScratch {
     uint32_t hist[STATIC_MAX_LEVELS];
     uint64_t flev[STATIC_MAX_LEVELS];
     double tree[STATIC_MAX_LEVELS];
-    int32_t bad;  // set when an energy lies outside the lattice's range
+    int32_t bad;       // an energy lies outside the lattice's range
+    int32_t lo_c, hi;  // STATIC_MAX_LEVELS - lowest level, highest level + 1
+    uint32_t tick;     // CTAs that have added their counts
+    int32_t lmin, ok;  // results: lowest level; whether the weights are valid
 };
 
 // One copy per device that loads the library (about 1.3 MB), kept until exit.
 static __device__ __align__(256) StaticScratch g_scratch;
 
-__device__ __forceinline__ double pow_bin_s(double q, uint32_t k) {
-    double r = 1.0, b = q;
-    while (k) {
-        if (k & 1u) r = __dmul_rn(r, b);
-        b = __dmul_rn(b, b);
-        k >>= 1;
-    }
+// q^k as the product of the squares q^(2^m) of k's set bits, least significant first
+__device__ __forceinline__ double pow_sq(const double* qsq, uint32_t k) {
+    double r = 1.0;
+    for (int m = 0; k; ++m, k >>= 1)
+        if (k & 1u) r = __dmul_rn(r, qsq[m]);
     return r;
 }
 
+constexpr int STATIC_SMEM_TREE = 2048;  // tree entries that fit the smallest shared array
+constexpr int STATIC_SMEM_MIN = STATIC_SMEM_TREE * 8;
+
+// Level counts over all CTAs; the last CTA to finish (a ticket) turns them into S, ln Q
+// and the fixed-point weights of the levels and leaves the counts at zero.  With one CTA
+// for the whole population 10^5 energies took 83 us; the counts are bound by the read of
+// E, the last CTA by latency (the FP64 tree and the logarithms, about 5 us).
 __global__ void __launch_bounds__(STATIC_THREADS)
-k_weights_static(StaticScratch* sc, const int32_t* __restrict__ E, uint32_t R_prev, uint32_t R,
+k_static_weights(StaticScratch* sc, const int32_t* __restrict__ E, uint32_t R_prev, uint32_t R,
                  int d, int N, int parity, double dbeta, double q, double* lnQ_out,
                  uint64_t* f_out) {
-    __shared__ int smin[32], smax[32];
+    extern __shared__ __align__(16) uint32_t sh[];  // counts of the nlev levels; then the tree
+    __shared__ double qsq[32], S_sh, lnS_sh, lnR_sh;
+    __shared__ int s_lo, s_hi, s_bad, s_last;
     const int nlev = d * N / 2 + 1;
-    // the array keeps the previous call's contents: clear what must start at zero
-    for (int l = threadIdx.x; l < nlev; l += blockDim.x) sc->hist[l] = 0u;
-    if (threadIdx.x == 0) sc->bad = 0;
-    __threadfence_block();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int l = threadIdx.x; l < nlev; l += STATIC_THREADS) sh[l] = 0u;
+    if (threadIdx.x == 0) {
+        s_lo = nlev;
+        s_hi = -1;
+        s_bad = 0;
+    }
     __syncthreads();
-    for (uint32_t j = threadIdx.x; j < R_prev; j += blockDim.x) {
+    int lo = nlev, hi = -1, bad = 0;
+    for (uint64_t j = (uint64_t)blockIdx.x * STATIC_THREADS + threadIdx.x; j < R_prev;
+         j += gridDim.x * STATIC_THREADS) {
         // 2U = E + dN (U unsatisfied bonds) in 64 bits: no overflow for any int32 E.
         // A valid energy has 0 <= U <= dN and U = parity (mod 2).
         const long long twoU = (long long)E[j] + (long long)d * N;
         if (twoU < 0 || twoU > 2LL * d * N || (twoU & 1) || (((twoU >> 1) & 1) != parity)) {
-            atomicExch(&sc->bad, 1);
+            bad = 1;
             continue;
         }
-        atomicAdd(&sc->hist[(int)(twoU >> 2)], 1u);
+        const int l = (int)(twoU >> 2);
+        lo = min(lo, l);
+        hi = max(hi, l);
+        atomicAdd(&sh[l], 1u);
     }
-    __threadfence_block();
-    __syncthreads();
-    volatile uint32_t* hist = sc->hist;
-    int lo = 0x7fffffff, hi = -1;
-    for (int l = threadIdx.x; l < nlev; l += blockDim.x)
-        if (hist[l]) {
-            lo = min(lo, l);
-            hi = max(hi, l);
-        }
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    bad = __any_sync(0xffffffffu, bad);
     if (lane == 0) {
-        smin[warp] = lo;
-        smax[warp] = hi;
+        if (hi >= 0) {
+            atomicMin(&s_lo, lo);
+            atomicMax(&s_hi, hi);
+        }
+        if (bad) atomicOr(&s_bad, 1);
     }
     __syncthreads();
-    lo = 0x7fffffff;
-    hi = -1;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        lo = min(lo, smin[w]);
-        hi = max(hi, smax[w]);
+    for (int l = s_lo + threadIdx.x; l <= s_hi; l += STATIC_THREADS)
+        if (sh[l]) atomicAdd(&sc->hist[l], sh[l]);
+    if (threadIdx.x == 0) {
+        if (s_hi >= 0) {
+            atomicMax(&sc->lo_c, STATIC_MAX_LEVELS - s_lo);
+            atomicMax(&sc->hi, s_hi + 1);
+        }
+        if (s_bad) atomicOr(&sc->bad, 1);
     }
-    volatile int32_t* bad = &sc->bad;
-    if (hi < 0 || *bad) {  // no valid energy: report NaN, write no weights
-        if (threadIdx.x == 0) *lnQ_out = NAN;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&sc->tick, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const int lmin = STATIC_MAX_LEVELS - *(volatile int32_t*)&sc->lo_c;
+    const int K = *(volatile int32_t*)&sc->hi - lmin;
+    const bool valid = *(volatile int32_t*)&sc->hi > 0 && *(volatile int32_t*)&sc->bad == 0;
+    volatile uint32_t* hist = sc->hist;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sc->tick = 0u;
+        sc->lo_c = sc->hi = 0;
+        sc->bad = 0;
+        sc->lmin = lmin;
+        sc->ok = valid;
+        if (!valid) *lnQ_out = NAN;  // no valid energy, or an invalid one: no weights
+        double b = q;
+        const int nb = K > 1 ? 32 - __clz(K - 1) : 0;
+        for (int m = 0; m < nb; ++m) {
+            qsq[m] = b;
+            b = __dmul_rn(b, b);
+        }
+    }
+    __syncthreads();
+    if (!valid) {
+        for (int l = threadIdx.x; l < nlev; l += STATIC_THREADS) sc->hist[l] = 0u;
         return;
     }
-    const int lmin = lo, K = hi - lo + 1;
     int P = 1;
     while (P < K) P <<= 1;
-    volatile double* t = sc->tree;
-    for (int k = threadIdx.x; k < P; k += blockDim.x)
-        t[k] = (k < K) ? __dmul_rn((double)hist[lmin + k], pow_bin_s(q, (uint32_t)k)) : 0.0;
+    // S = sum_k n_k w_k as the fixed pairwise tree (t_k += t_{k+h}, h = P/2 ... 1)
+    const bool tree_sh = P <= STATIC_SMEM_TREE;
+    double* ts = reinterpret_cast<double*>(sh);
+    volatile double* tg = sc->tree;
+    for (int k = threadIdx.x; k < P; k += STATIC_THREADS) {
+        const double v = k < K ? __dmul_rn((double)hist[lmin + k], pow_sq(qsq, (uint32_t)k)) : 0.0;
+        if (tree_sh) ts[k] = v;
+        else tg[k] = v;
+    }
     __threadfence_block();
     __syncthreads();
-    for (int h = P >> 1; h >= 1; h >>= 1) {
-        for (int k = threadIdx.x; k < h; k += blockDim.x) t[k] = __dadd_rn(t[k], t[k + h]);
+    int h = P >> 1;
+    for (; h >= 32; h >>= 1) {
+        for (int k = threadIdx.x; k < h; k += STATIC_THREADS) {
+            if (tree_sh) ts[k] = __dadd_rn(ts[k], ts[k + h]);
+            else tg[k] = __dadd_rn(tg[k], tg[k + h]);
+        }
         __threadfence_block();
         __syncthreads();
     }
-    const double S = t[0];
+    if (warp == 0) {  // the last levels by shuffles, the same pairs
+        const int live = h > 0 ? 2 * h : 1;
+        double v = 0.0;
+        if (lane < live) v = tree_sh ? ts[lane] : tg[lane];
+        for (; h >= 1; h >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, h));
+        if (lane == 0) S_sh = v;
+    }
+    __syncthreads();
+    const double S = S_sh;
+    if (warp == STATIC_THREADS / 32 - 1) {  // the two logarithms beside the divisions
+        const double lx = log(lane == 0 ? S : (double)R_prev);
+        if (lane == 0) lnS_sh = lx;
+        if (lane == 1) lnR_sh = lx;
+    }
     const double Rd = (double)R;
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        double a = __dmul_rn(Rd, pow_bin_s(q, (uint32_t)k));
+    for (int k = threadIdx.x; k < K; k += STATIC_THREADS) {
+        double a = __dmul_rn(Rd, pow_sq(qsq, (uint32_t)k));
         a = __ddiv_rn(a, S);
         a = scalbn(a, pa::FRAC_BITS);
         sc->flev[k] = (uint64_t)floor(a);
     }
     __threadfence_block();
     __syncthreads();
-    volatile uint64_t* flev = sc->flev;
-    for (uint32_t j = threadIdx.x; j < R_prev; j += blockDim.x)
-        f_out[j] = flev[(((E[j] + d * N) >> 1) >> 1) - lmin];
+    for (int k = threadIdx.x; k < K; k += STATIC_THREADS) sc->hist[lmin + k] = 0u;
+    if (f_out)  // one CTA holds the whole population: f at once
+        for (uint32_t j = threadIdx.x; j < R_prev; j += STATIC_THREADS)
+            f_out[j] = ((volatile uint64_t*)sc->flev)[((E[j] + d * N) >> 2) - lmin];
     if (threadIdx.x == 0) {
         const int32_t Umin = 2 * lmin + parity;
         const int32_t Emin = 2 * Umin - d * N;
-        *lnQ_out = __dsub_rn(__dsub_rn(log(S), log((double)R_prev)), __dmul_rn(dbeta, (double)Emin));
+        *lnQ_out = __dsub_rn(__dsub_rn(lnS_sh, lnR_sh), __dmul_rn(dbeta, (double)Emin));
     }
+}
+
+// f_j of every replica from the level table (a launch of its own: every CTA needs it)
+__global__ void __launch_bounds__(256)
+k_static_f(const StaticScratch* __restrict__ sc, const int32_t* __restrict__ E, uint32_t R_prev,
+           int dN, uint64_t* __restrict__ f_out) {
+    if (!sc->ok) return;
+    const int lmin = sc->lmin;
+    for (uint64_t j = (uint64_t)blockIdx.x * 256u + threadIdx.x; j < R_prev; j += gridDim.x * 256u)
+        f_out[j] = sc->flev[((E[j] + dN) >> 2) - lmin];
 }
 
 }  // namespace
@@ -141,7 +214,19 @@ extern "C" pa_status pa_weights_static(const int32_t* E, uint32_t R_prev, uint32
     if (cudaGetSymbolAddress(&ptr, g_scratch) != cudaSuccess || !ptr) return PA_ERR_CUDA;
     StaticScratch* sc = (StaticScratch*)ptr;
     const double q = std::exp(-(4.0 * dbeta));
-    k_weights_static<<<1, STATIC_THREADS, 0, (cudaStream_t)cuda_stream>>>(
-        sc, E, R_prev, R, dim, (int)N, parity, dbeta, q, lnQ, f);
+    const cudaStream_t st = (cudaStream_t)cuda_stream;
+    // four energies per thread, at most one CTA per SM
+    const uint32_t per = 4 * STATIC_THREADS;
+    const unsigned na = (unsigned)std::min<uint64_t>(((uint64_t)R_prev + per - 1) / per, 152u);
+    const int sm = std::max(STATIC_SMEM_MIN, (int)(dim * N / 2 + 1) * 4);  // at most 197 KB
+    if (sm > 48 * 1024 - 512 &&
+        cudaFuncSetAttribute(k_static_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) !=
+            cudaSuccess)
+        return PA_ERR_CUDA;
+    k_static_weights<<<na, STATIC_THREADS, sm, st>>>(sc, E, R_prev, R, dim, (int)N, parity, dbeta, q,
+                                                     lnQ, na == 1 ? f : nullptr);
+    if (na == 1) return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
+    const unsigned nf = (unsigned)std::min<uint64_t>(((uint64_t)R_prev + 1023u) / 1024u, 152u * 8u);
+    k_static_f<<<nf, 256, 0, st>>>(sc, E, R_prev, dim * (int)N, f);
     return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
 }

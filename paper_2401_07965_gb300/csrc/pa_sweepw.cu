@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
     ls.to_cta(&sums, lane);
     __syncthreads();
     if (hist_sm)
-        for (int l = sums.lo + tid; l <= sums.hi; l += NT)
+        for (int l = (sums.hi < 0 ? 0 : sums.lo) + tid; l <= sums.hi; l += NT)
             if (shist[l]) atomicAdd(&r.hist[l], shist[l]);
     add_to_trace(sums, r, i);
 }
