@@ -34,15 +34,18 @@ struct RunHost {
     int parity;
 };
 
+// R_ANC .. R_TICK start at zero (one fill per run)
 enum Region {
-    R_SPIN0, R_SPIN1, R_E0, R_E1, R_F0, R_F1, R_M, R_ANC, R_CNT, R_C, R_G, R_HIST, R_FLEV, R_TREE,
-    R_PA, R_PB, R_OA, R_OB, R_PD, R_PCL, R_W, R_WP, R_OP, R_JB, R_ST, R_TRACE, R_LB1, R_LB2,
-    R_TICK, R_SB, R_SDB, R_SQ, R_STHR, R_STH, R_COUNT
+    R_SPIN0, R_SPIN1, R_E0, R_E1, R_F0, R_F1, R_M, R_C, R_G, R_FLEV, R_TREE,
+    R_PA, R_PB, R_OA, R_OB, R_PD, R_PCL, R_W, R_WP, R_OP,
+    R_ANC, R_CNT, R_HIST, R_TRACE, R_LB1, R_LB2, R_TICK,
+    R_SB, R_SDB, R_SQ, R_STHR, R_STH, R_COUNT
 };
 
 enum Shared {
     S_RUNS, S_B2R, S_G2R, S_BETA, S_DBETA, S_Q, S_THR, S_THETA, S_IDS, S_WOUT,
     S_CTL, S_GBETA, S_GTHR, S_GDB, S_GQ, S_PAIRS, S_POV, S_OVACC, S_OVTICK, S_CTA, S_CLNC,
+    S_ST, S_JB,  // the runs' states and coupling bits, one copy each way for all runs
     S_COUNT
 };
 
@@ -60,6 +63,7 @@ struct pa_ctx {
     KParams kp;
     std::vector<RunHost> runs;
     std::vector<RunDesc> desc;
+    std::vector<DevState> states;           // the runs' states at the last pa_sync
     int d = 0, n_steps = 0, method = 0, M = 0;
     uint64_t seed = 0;
     cudaStream_t stream = nullptr;
@@ -194,6 +198,9 @@ Layout make_layout(const std::vector<RunHost>& runs, int n_steps) {
     sz[S_OVTICK] = M * 4;
     sz[S_CTA] = ngrp * 4;  // CTA -> run map of the sweep launches (a CTA holds a group or more)
     sz[S_CLNC] = (CLN_TAB + 1) * 8;
+    sz[S_ST] = M * sizeof(DevState);
+    sz[S_JB] = 0;
+    for (const RunHost& h : runs) sz[S_JB] += align256((size_t)h.N);
     size_t o = 0;
     for (int r = 0; r < S_COUNT; ++r) {
         L.shared_off[r] = o;
@@ -213,8 +220,6 @@ Layout make_layout(const std::vector<RunHost>& runs, int n_steps) {
         rs[R_W] = rows * 8;
         rs[R_WP] = (size_t)h.nblk * 4 * 8;
         rs[R_OP] = (size_t)h.nblk * 5 * 8;
-        rs[R_JB] = (size_t)h.N;
-        rs[R_ST] = sizeof(DevState);
         rs[R_TRACE] = (size_t)(n_steps + 1) * sizeof(TraceRow);
         rs[R_LB1] = rs[R_LB2] = (size_t)h.nblk * sizeof(LBDesc);
         rs[R_TICK] = 2 * sizeof(uint32_t);
@@ -323,12 +328,6 @@ cudaError_t clear_lookback(const RunDesc& r, const RunHost& h, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaMemsetAsync(r.lb2, 0, (size_t)h.nblk * sizeof(LBDesc), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(r.tick, 0, 2 * sizeof(uint32_t), s);
     return e;
-}
-
-pa_status read_state(pa_ctx* ctx, int run, DevState* st) {
-    PA_CUDA(cudaStreamSynchronize(ctx->stream));
-    PA_CUDA(cudaMemcpy(st, ctx->desc[run].st, sizeof(DevState), cudaMemcpyDeviceToHost));
-    return PA_OK;
 }
 
 pa_status enqueue_measure(pa_ctx* ctx) {
@@ -705,6 +704,7 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
     std::vector<uint32_t> b2r, g2r;
     ctx->desc.resize(M);
     uint32_t blk0 = 0, grp0 = 0;
+    size_t jb0 = 0;
     for (int m = 0; m < M; ++m) {
         const RunHost& h = ctx->runs[m];
         const auto& off = lay.run_off[m];
@@ -754,8 +754,9 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
         r.w = (double*)(base + off[R_W]);
         r.wpart = (double*)(base + off[R_WP]);
         r.opart = (double*)(base + off[R_OP]);
-        r.jbits = (const uint8_t*)(base + off[R_JB]);
-        r.st = (DevState*)(base + off[R_ST]);
+        r.jbits = (const uint8_t*)(base + lay.shared_off[S_JB] + jb0);
+        jb0 += align256((size_t)h.N);
+        r.st = (DevState*)(base + lay.shared_off[S_ST]) + m;
         r.trace = (TraceRow*)(base + off[R_TRACE]);
         r.sbeta = (double*)(base + lay.shared_off[S_BETA]);
         r.sdbeta = (double*)(base + lay.shared_off[S_DBETA]);
@@ -816,24 +817,24 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
     double clnc[CLN_TAB + 1];
     for (int c = 0; c <= CLN_TAB; ++c) clnc[c] = c > 1 ? (double)c * std::log((double)c) : 0.0;
     up(p.clnc, clnc, sizeof(clnc));
+    std::vector<uint8_t> jball(jb0, 0);
+    ctx->states.assign(M, DevState{});
+    jb0 = 0;
     for (int m = 0; m < M && e == cudaSuccess; ++m) {
         const RunHost& h = ctx->runs[m];
-        const RunDesc& r = ctx->desc[m];
-        DevState st0;
+        DevState& st0 = ctx->states[m];
         std::memset(&st0, 0, sizeof(st0));
         st0.R_cur = h.R;
         st0.R_prev = h.R;
         st0.hlo = 0x7FFFFFFF;
         st0.hhi = -1;
-        up(r.jbits, h.jb.data(), h.jb.size());
-        up(r.st, &st0, sizeof(st0));
-        if (e == cudaSuccess) e = cudaMemsetAsync(r.hist, 0, (size_t)h.nlev * 4, ctx->stream);
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(r.trace, 0, (size_t)(n + 1) * sizeof(TraceRow), ctx->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(r.counts, 0, (size_t)h.Rcap * 4, ctx->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(r.anc, 0, (size_t)h.Rcap * 4, ctx->stream);
-        if (e == cudaSuccess) e = clear_lookback(r, h, ctx->stream);
+        std::memcpy(&jball[jb0], h.jb.data(), h.jb.size());
+        jb0 += align256((size_t)h.N);
+        const size_t z0 = lay.run_off[m][R_ANC], z1 = lay.run_off[m][R_SB];
+        e = cudaMemsetAsync(base + z0, 0, z1 - z0, ctx->stream);
     }
+    up(ctx->desc[0].jbits, jball.data(), jball.size());
+    up(ctx->desc[0].st, ctx->states.data(), sizeof(DevState) * M);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(ctx->d_ovacc, 0, (size_t)M * (maxN + 1) * 4, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_ovtick, 0, (size_t)M * 4, ctx->stream);
@@ -906,9 +907,10 @@ pa_status pa_sync(pa_ctx* ctx) {
     PA_CUDA(cudaStreamSynchronize(ctx->stream));
     bool all_done = true;
     int most = 0;
+    PA_CUDA(cudaMemcpy(ctx->states.data(), ctx->desc[0].st, sizeof(DevState) * ctx->M,
+                       cudaMemcpyDeviceToHost));
     for (int m = 0; m < ctx->M; ++m) {
-        DevState st;
-        PA_CUDA(cudaMemcpy(&st, ctx->desc[m].st, sizeof(DevState), cudaMemcpyDeviceToHost));
+        DevState st = ctx->states[m];
         if (ctx->controlled) {
             // runs of a controlled batch reach beta_f after different step counts
             ctx->rstep[m] = st.step;
@@ -970,9 +972,7 @@ pa_status pa_run_free_energy(pa_ctx* ctx, int32_t run, double* minus_beta_F, dou
     if (!valid_run(ctx, run)) return PA_ERR_ARG;
     pa_status s = pa_sync(ctx);
     if (s != PA_OK) return s;
-    DevState st;
-    s = read_state(ctx, run, &st);
-    if (s != PA_OK) return s;
+    const DevState& st = ctx->states[run];  // as pa_sync read it
     const double N = ctx->runs[run].N;
     const double mbf = N * std::log(2.0) + st.sum_lnQ;
     const double b = run_beta(ctx, run, run_step(ctx, run));
@@ -990,9 +990,7 @@ pa_status pa_run_get_array(pa_ctx* ctx, int32_t run, pa_array which, void* host,
     if (!valid_run(ctx, run) || !host) return PA_ERR_ARG;
     pa_status s = pa_sync(ctx);
     if (s != PA_OK) return s;
-    DevState st;
-    s = read_state(ctx, run, &st);
-    if (s != PA_OK) return s;
+    const DevState& st = ctx->states[run];  // as pa_sync read it
     const int par = run_step(ctx, run) & 1;
     const RunDesc& r = ctx->desc[run];
     const RunHost& h = ctx->runs[run];

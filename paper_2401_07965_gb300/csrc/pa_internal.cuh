@@ -98,8 +98,9 @@ __device__ __forceinline__ void mulhilo(uint32_t a, uint32_t b, uint32_t& hi, ui
     lo = (uint32_t)p;
 }
 
-// Device state shared by the kernels of a run (one per context).
-struct DevState {
+// Device state shared by the kernels of a run (the runs' states stand side by side; a
+// cache line each).
+struct alignas(128) DevState {
     int32_t step;      // completed temperature steps; during a step its index (k_weights)
     int32_t status;    // DevStatus
     uint32_t R_cur;    // current population size
