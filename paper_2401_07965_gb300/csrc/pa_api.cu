@@ -37,7 +37,7 @@ struct RunHost {
 // R_ANC .. R_TICK start at zero (one fill per run)
 enum Region {
     R_SPIN0, R_SPIN1, R_E0, R_E1, R_F0, R_F1, R_M, R_C, R_G, R_FLEV, R_TREE,
-    R_PA, R_PB, R_OA, R_OB, R_PD, R_PCL, R_W, R_WP, R_OP,
+    R_PD, R_PCL, R_W, R_WP, R_OP,
     R_ANC, R_CNT, R_HIST, R_TRACE, R_LB1, R_LB2, R_TICK,
     R_SB, R_SDB, R_SQ, R_STHR, R_STH, R_COUNT
 };
@@ -216,7 +216,7 @@ Layout make_layout(const std::vector<RunHost>& runs, int n_steps) {
         rs[R_HIST] = (size_t)h.nlev * 4;
         rs[R_FLEV] = (size_t)h.nlev * 8;
         rs[R_TREE] = (size_t)h.P * 8;
-        rs[R_PA] = rs[R_PB] = rs[R_OA] = rs[R_OB] = rs[R_PD] = rs[R_PCL] = (size_t)h.nblk * 8;
+        rs[R_PD] = rs[R_PCL] = (size_t)h.nblk * 8;
         rs[R_W] = rows * 8;
         rs[R_WP] = (size_t)h.nblk * 4 * 8;
         rs[R_OP] = (size_t)h.nblk * 5 * 8;
@@ -745,10 +745,6 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
         r.hist = (uint32_t*)(base + off[R_HIST]);
         r.flev = (uint64_t*)(base + off[R_FLEV]);
         r.tree = (double*)(base + off[R_TREE]);
-        r.partA = (uint64_t*)(base + off[R_PA]);
-        r.partB = (uint64_t*)(base + off[R_PB]);
-        r.offA = (uint64_t*)(base + off[R_OA]);
-        r.offB = (uint64_t*)(base + off[R_OB]);
         r.partD = (double*)(base + off[R_PD]);
         r.partCL = (double*)(base + off[R_PCL]);
         r.w = (double*)(base + off[R_W]);

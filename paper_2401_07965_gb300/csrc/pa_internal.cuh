@@ -174,11 +174,7 @@ struct RunDesc {
     uint32_t* hist;          // level histogram of the current population
     uint64_t* flev;          // fixed-point tau-hat per level
     double* tree;            // pairwise-sum scratch (power of two >= nlev)
-    uint64_t* partA;         // per-block partial sums
-    uint64_t* partB;
-    uint64_t* offA;          // per-block exclusive offsets
-    uint64_t* offB;
-    double* partD;
+    double* partD;           // per-block partial sums
     double* partCL;
     double* w;               // partial resampling: replica weights
     double* wpart;           // per-block tree sums of the weights (4 per block)

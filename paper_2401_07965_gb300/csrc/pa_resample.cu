@@ -18,7 +18,9 @@
 // replica index (blocks of SCAN_CHUNK aligned replicas, then the blocks:
 // k_pw_final), and resamples with f_j = floor(2^40 (R wn_j) / S_new) only if
 // (sum wn)^2 / sum wn^2 < alpha R_{i-1}; otherwise every replica is kept once
-// and its weight is rescaled by a power of two (k_family).
+// and its weight is rescaled by a power of two (k_family).  The f_j and their total come
+// from k_fsum, the rest from the kernels of the plain step (its look-back scans replaced
+// six kernels: 2D L = 64, R = 10^4, 200 steps 52.9 -> 40.4 ms).
 #include <climits>
 
 #include "pa_internal.cuh"
@@ -54,6 +56,41 @@ __device__ __forceinline__ double exp_taylor(double x) {
 #pragma unroll
     for (int k = 12; k >= 0; --k) pp = __dadd_rn(__dmul_rn(pp, r), c[k]);
     return scalbn(pp, (int)nd);
+}
+
+// Poisson draw of mean lc in [0, 16] by sequential inversion of the CDF: the first k with
+// u < P_k, u = bits >> 11 in 2^-53 units, P_k summed in explicitly rounded FP64.  The search
+// runs in FP32 first: its P_k is within 1e-5 of the FP64 one (k <= 64: each term carries at
+// most 2 + 2k roundings of 2^-24, the terms sum to 1), so u farther than 2e-5 from every
+// P_k it passes decides alike; the others (about 1e-4 of the draws) repeat it in FP64, whose
+// operations occupy the pipe for 16 cycles per warp (k_resample, +-J L = 48, R = 20001:
+// 34 -> 27 us).
+__device__ __forceinline__ uint32_t poisson_draw(double lc, uint64_t bits, bool& kmax) {
+    {
+        const float l = (float)lc, u = (float)(uint32_t)(bits >> 40) * 0x1p-24f;
+        float pr = expf(-l), Pc = pr;
+        uint32_t k = 0;
+        while (u - Pc > 2e-5f && k < 64u) {
+            k += 1;
+            pr = __fdividef(pr * l, (float)k);
+            Pc += pr;
+        }
+        if (u - Pc < -2e-5f) return k;
+    }
+    const double u = scalbn((double)(bits >> 11), -53);
+    double pr = exp_taylor(-lc);
+    double Pc = pr;
+    uint32_t k = 0;
+    while (u >= Pc) {
+        k += 1;
+        if (k > POISSON_KMAX) {
+            kmax = true;
+            break;
+        }
+        pr = __ddiv_rn(__dmul_rn(pr, lc), (double)k);
+        Pc = __dadd_rn(Pc, pr);
+    }
+    return k;
 }
 
 struct U128 {
@@ -133,36 +170,56 @@ __device__ __forceinline__ double tree_regs(const double* a) {
     return t[0];
 }
 
-__device__ double tree_threads(double v, double* sh) {
+// the same tree over the threads of a CTA for NV values at once (sh: NV x 33 doubles), of
+// which the first `leaves` threads hold any but zeros (the other warps skip their adds: an
+// FP64 operation occupies this part's pipe for 16 cycles per warp); the roots end in every
+// thread
+template <int NV>
+__device__ __forceinline__ void tree_threads(double (&v)[NV], double* sh, int leaves = 1024) {
     // levels inside a warp by shuffles (lane t adds lane t + w for t a multiple
     // of 2w: the same pairs as the tree), then the same over the warps' sums
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (warp * 32 < leaves)
 #pragma unroll
-    for (int w = 1; w < 32; w <<= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, w));
-    if (lane == 0) sh[warp] = v;
+        for (int w = 1; w < 32; w <<= 1)
+#pragma unroll
+            for (int q = 0; q < NV; ++q) v[q] = __dadd_rn(v[q], __shfl_down_sync(0xffffffffu, v[q], w));
+    if (lane == 0)
+#pragma unroll
+        for (int q = 0; q < NV; ++q) sh[33 * q + warp] = v[q];
     __syncthreads();
-    if (warp == 0) {
-        double u = lane < nw ? sh[lane] : 0.0;
-        for (int w = 1; w < nw; w <<= 1) u = __dadd_rn(u, __shfl_down_sync(0xffffffffu, u, w));
-        if (lane == 0) sh[32] = u;
+    if (warp < NV) {  // warp q finishes value q
+        double u = lane < nw ? sh[33 * warp + lane] : 0.0;
+        for (int w = 1; w < nw && w * 32 < leaves; w <<= 1)
+            u = __dadd_rn(u, __shfl_down_sync(0xffffffffu, u, w));
+        if (lane == 0) sh[33 * warp + 32] = u;
     }
     __syncthreads();
-    const double root = sh[32];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = sh[33 * q + 32];
     __syncthreads();
-    return root;
 }
 
-__device__ double max_threads(double v, double* sh) {
-    const int t = threadIdx.x, n = blockDim.x;
-    sh[t] = v;
-    __syncthreads();
-    for (int w = n >> 1; w >= 1; w >>= 1) {
-        if (t < w) sh[t] = fmax(sh[t], sh[t + w]);
-        __syncthreads();
+// largest of the first n threads' values (non-negative), in every thread
+__device__ __forceinline__ double max_threads(double v, double* sh, int n = 1024) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nw = min((int)blockDim.x >> 5, (n + 31) / 32);
+    if (warp < nw) {  // the bit patterns of non-negative doubles are ordered like the values
+        unsigned long long u = (unsigned long long)__double_as_longlong(v);
+        for (int w = 16; w >= 1; w >>= 1) {
+            const unsigned long long o = __shfl_xor_sync(0xffffffffu, u, w);
+            u = o > u ? o : u;
+        }
+        if (lane == 0) sh[warp] = __longlong_as_double((long long)u);
     }
-    const double root = sh[0];
     __syncthreads();
-    return root;
+    unsigned long long u = 0ull;
+    for (int k = 0; k < nw; ++k) {
+        const unsigned long long o = (unsigned long long)__double_as_longlong(sh[k]);
+        u = o > u ? o : u;
+    }
+    __syncthreads();
+    return __longlong_as_double((long long)u);
 }
 
 // --------------------------------------------------------------------------
@@ -357,7 +414,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_pw_update(KParams p) {
     const uint32_t b = blockIdx.x - r.blk0;
     const DevState* st = r.st;
     if (st->status != S_OK) return;
-    __shared__ double sh[SCAN_THREADS];
+    __shared__ double sh[3 * 33];
     const int i = st->step;
     const int32_t* E = r.E[(i - 1) & 1];
     const uint32_t Rprev = st->R_prev, lmin = st->lmin;
@@ -378,45 +435,56 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_pw_update(KParams p) {
             mx = fmax(mx, wn[e]);
         }
     }
-    const double s_old = tree_threads(tree_regs<SCAN_ITEMS>(wo), sh);
-    const double s_new = tree_threads(tree_regs<SCAN_ITEMS>(wn), sh);
-    const double s2 = tree_threads(tree_regs<SCAN_ITEMS>(w2), sh);
+    double v[3] = {tree_regs<SCAN_ITEMS>(wo), tree_regs<SCAN_ITEMS>(wn), tree_regs<SCAN_ITEMS>(w2)};
+    tree_threads(v, sh);
     mx = max_threads(mx, sh);
     if (threadIdx.x == 0) {
-        r.wpart[4 * b + 0] = s_old;
-        r.wpart[4 * b + 1] = s_new;
-        r.wpart[4 * b + 2] = s2;
+        r.wpart[4 * b + 0] = v[0];
+        r.wpart[4 * b + 1] = v[1];
+        r.wpart[4 * b + 2] = v[2];
         r.wpart[4 * b + 3] = mx;
     }
 }
 
-// one CTA per run: tree over the blocks, ln Q, effective size, decision
+// One CTA per run: tree over the blocks, ln Q, effective size, decision.  Up to 1024
+// blocks a thread holds one leaf (the tree over PARTIAL_MAX_BLOCKS leaves is the same: the
+// others are zeros) and warps past the last leaf skip their FP64 adds: 29 -> 7.9 us at
+// R = 10^4 (16 leaves in every thread, whatever the population, and one sum after the
+// other).
 __global__ void __launch_bounds__(1024) k_pw_final(KParams p) {
     const RunDesc& r = p.runs[blockIdx.x];
     DevState* st = r.st;
     if (st->status != S_OK) return;
-    __shared__ double sh[1024];
+    __shared__ double sh[3 * 33], lg[2];
     const int i = st->step;
     const int nb = r.nblk;  // <= PARTIAL_MAX_BLOCKS = LEAVES leaves x 1024 threads
     constexpr int LEAVES = PARTIAL_MAX_BLOCKS / 1024;
     double S[3];
-    for (int q = 0; q < 3; ++q) {
-        double x[LEAVES];
 #pragma unroll
-        for (int k = 0; k < LEAVES; ++k) {
-            const int bb = LEAVES * threadIdx.x + k;
-            x[k] = bb < nb ? r.wpart[4 * bb + q] : 0.0;
+    for (int q = 0; q < 3; ++q) {
+        if (nb <= 1024) {
+            S[q] = (int)threadIdx.x < nb ? r.wpart[4 * threadIdx.x + q] : 0.0;
+        } else {
+            double x[LEAVES];
+#pragma unroll
+            for (int k = 0; k < LEAVES; ++k) {
+                const int bb = LEAVES * threadIdx.x + k;
+                x[k] = bb < nb ? r.wpart[4 * bb + q] : 0.0;
+            }
+            S[q] = tree_regs<LEAVES>(x);
         }
-        S[q] = tree_threads(tree_regs<LEAVES>(x), sh);
     }
     double mx = 0.0;
     for (int bb = threadIdx.x; bb < nb; bb += blockDim.x) mx = fmax(mx, r.wpart[4 * bb + 3]);
-    mx = max_threads(mx, sh);
+    tree_threads(S, sh, nb <= 1024 ? nb : 1024);
+    mx = max_threads(mx, sh, nb);
+    if (threadIdx.x < 2) lg[threadIdx.x] = log(S[threadIdx.x]);  // two lanes, one pass
+    __syncwarp();
     if (threadIdx.x == 0) {
         const uint32_t Rprev = st->R_prev;
         const int32_t Umin = 2 * (int32_t)st->lmin + r.parity;
         const int32_t Emin = 2 * Umin - p.d * r.N;
-        const double lnQ = __dsub_rn(__dsub_rn(log(S[1]), log(S[0])),
+        const double lnQ = __dsub_rn(__dsub_rn(lg[1], lg[0]),
                                      __dmul_rn(r.sdbeta[i - 1], (double)Emin));
         const double ess = __ddiv_rn(__dmul_rn(S[1], S[1]), S[2]);
         const int res = ess < __dmul_rn(p.alpha, (double)Rprev) ? 1 : 0;
@@ -425,6 +493,9 @@ __global__ void __launch_bounds__(1024) k_pw_final(KParams p) {
         st->resample = res;
         st->wexp = e;
         st->S_new = S[1];
+        st->T = st->Tres = 0ull;  // summed by k_fsum
+        st->epoch += 1u;
+        st->kmax = 0;
         st->sum_lnQ = __dadd_rn(st->sum_lnQ, lnQ);
         TraceRow* tr = r.trace + i;
         tr->lnQ = lnQ;
@@ -442,191 +513,54 @@ __global__ void k_pw_init(KParams p) {
 }
 
 // --------------------------------------------------------------------------
-// per-block sums of f (and of its 2^-40 fractional part)
+// partial resampling, a step that resamples: the expected copies of the replicas (kept
+// in C until the prefix takes its place) and their total, which the copy-count kernels
+// need before any scan; the run's last block to finish sets the residual draws
 // --------------------------------------------------------------------------
-// expected copies of parent j in 2^-40 units: the level table, or under
-// partial resampling floor(2^40 (R wn_j) / S_new) when the step resamples and
-// exactly one copy when it does not
-__device__ __forceinline__ uint64_t f_of(int j, const KParams& p, const RunDesc& r,
-                                         const DevState* st, int dN, const int32_t* E,
-                                         uint32_t lmin) {
-    if (p.alpha >= 0.0) {
-        if (!st->resample) return 1ull << FRAC_BITS;
-        double a = __dmul_rn((double)r.R, r.w[j]);
-        a = __ddiv_rn(a, st->S_new);
-        a = scalbn(a, FRAC_BITS);
-        return (uint64_t)floor(a);
-    }
-    return r.flev[level_of(E[j], dN) - (int)lmin];
-}
-
 __global__ void __launch_bounds__(SCAN_THREADS) k_fsum(KParams p) {
     const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
     const uint32_t b = blockIdx.x - r.blk0;
-    const DevState* st = r.st;
-    if (st->status != S_OK) return;
-    if (p.alpha >= 0.0 && !st->resample) return;  // partial: population kept
-    __shared__ uint64_t sh[33];
-    const int i = st->step;
-    const int32_t* E = r.E[(i - 1) & 1];
-    const uint32_t Rprev = st->R_prev, lmin = st->lmin;
-    const int dN = p.d * r.N;
+    DevState* st = r.st;
+    if (st->status != S_OK || !st->resample) return;  // the population is kept
+    __shared__ unsigned long long tot[2];
+    const uint32_t Rprev = st->R_prev;
     const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
-    uint64_t sf = 0, sg = 0;
+    unsigned long long sf = 0, sg = 0;
+#pragma unroll
     for (int e = 0; e < SCAN_ITEMS; ++e) {
         const int j = j0 + e;
         if ((uint32_t)j < Rprev) {
-            const uint64_t f = f_of(j, p, r, st, dN, E, lmin);
+            double a = __dmul_rn((double)r.R, r.w[j]);
+            a = __ddiv_rn(a, st->S_new);
+            a = scalbn(a, FRAC_BITS);
+            const uint64_t f = (uint64_t)floor(a);
+            r.C[j] = f;
             sf += f;
             sg += f & ((1ull << FRAC_BITS) - 1);
         }
     }
-    uint64_t tot;
-    block_excl_scan(sf, sh, &tot);
-    if (threadIdx.x == 0) r.partA[b] = tot;
-    block_excl_scan(sg, sh, &tot);
-    if (threadIdx.x == 0) r.partB[b] = tot;
-}
-
-// exclusive scan of the per-block partials (one CTA of 1024 threads)
-__device__ void scan_partials(const uint64_t* part, uint64_t* off, int n, uint64_t* total_out) {
-    __shared__ uint64_t sh[33];
-    __shared__ uint64_t carry;
-    if (threadIdx.x == 0) carry = 0;
+    if (threadIdx.x == 0) tot[0] = tot[1] = 0ull;
     __syncthreads();
-    for (int b0 = 0; b0 < n; b0 += blockDim.x) {
-        const int b = b0 + threadIdx.x;
-        const uint64_t v = (b < n) ? part[b] : 0ull;
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        uint64_t incl = warp_incl_scan(v, lane);
-        if (lane == 31) sh[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            uint64_t w = (lane < (int)(blockDim.x >> 5)) ? sh[lane] : 0ull;
-            uint64_t wi = warp_incl_scan(w, lane);
-            sh[lane] = wi - w;
-            if (lane == 31) sh[32] = wi;
-        }
-        __syncthreads();
-        if (b < n) off[b] = carry + sh[warp] + incl - v;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += sh[32];
-        __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) {
+        sf += __shfl_xor_sync(0xffffffffu, sf, o);
+        sg += __shfl_xor_sync(0xffffffffu, sg, o);
     }
-    if (threadIdx.x == 0) *total_out = carry;
-}
-
-__global__ void __launch_bounds__(1024) k_fscan(KParams p) {
-    const RunDesc& r = p.runs[blockIdx.x];
-    DevState* st = r.st;
-    if (st->status != S_OK) return;
-    if (p.alpha >= 0.0 && !st->resample) return;
-    __shared__ uint64_t tA, tB;
-    scan_partials(r.partA, r.offA, r.nblk, &tA);
-    scan_partials(r.partB, r.offB, r.nblk, &tB);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&tot[0], sf);
+        atomicAdd(&tot[1], sg);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        st->T = tA;
-        st->Tres = tB;
-        const uint64_t A = (tA - tB) >> FRAC_BITS;  // sum of floor(f / 2^40)
-        st->Rres = (uint64_t)r.R - A;
-    }
-}
-
-// --------------------------------------------------------------------------
-// prefix sums C (and G) and the copy counts of the rules that need no search
-// --------------------------------------------------------------------------
-__global__ void __launch_bounds__(SCAN_THREADS) k_counts(KParams p) {
-    const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
-    const uint32_t b = blockIdx.x - r.blk0;
-    DevState* st = r.st;
-    if (st->status != S_OK) return;
-    __shared__ uint64_t sh[33];
-    const int i = st->step;
-    const int32_t* E = r.E[(i - 1) & 1];
-    const int dN = p.d * r.N;
-    const uint32_t Rprev = st->R_prev, lmin = st->lmin;
-    const uint64_t T = st->T;
-    const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
-    if (p.alpha >= 0.0 && !st->resample) {
-        // partial resampling keeps every replica once: identity counts and
-        // ancestors, no sampling variance (the scan kernels return at once)
-        for (int e = 0; e < SCAN_ITEMS; ++e) {
-            const int j = j0 + e;
-            if ((uint32_t)j < Rprev) {
-                r.counts[j] = 1u;
-                r.anc[j] = (uint32_t)j;
-                r.fam[i & 1][j] = r.fam[(i - 1) & 1][j];
-            }
+        atomicAdd((unsigned long long*)&st->T, tot[0]);
+        atomicAdd((unsigned long long*)&st->Tres, tot[1]);
+        __threadfence();
+        if (atomicAdd(&r.tick[0], 1u) == (uint32_t)r.nblk - 1u) {
+            __threadfence();
+            const uint64_t T = *(volatile uint64_t*)&st->T, G = *(volatile uint64_t*)&st->Tres;
+            st->Rres = (uint64_t)r.R - ((T - G) >> FRAC_BITS);
+            r.tick[0] = 0u;
         }
-        if (threadIdx.x == 0) r.partD[b] = 0.0;
-        return;
     }
-    uint64_t f[SCAN_ITEMS];
-    uint64_t sf = 0, sg = 0;
-#pragma unroll
-    for (int e = 0; e < SCAN_ITEMS; ++e) {
-        const int j = j0 + e;
-        f[e] = ((uint32_t)j < Rprev) ? f_of(j, p, r, st, dN, E, lmin) : 0ull;
-        sf += f[e];
-        sg += f[e] & ((1ull << FRAC_BITS) - 1);
-    }
-    uint64_t tot;
-    uint64_t cf = block_excl_scan(sf, sh, &tot) + r.offA[b];
-    uint64_t cg = block_excl_scan(sg, sh, &tot) + r.offB[b];
-    const int method = p.method;
-    uint32_t usys = 0;
-    if (method == M_SYSTEMATIC)
-        usys = philox(0u, DOM_RESAMPLE | (r.run << 8) | RULE_SYSTEMATIC, (uint32_t)i, 0u, p.k0, p.k1).x;
-    bool kmax = false;
-#pragma unroll 1
-    for (int e = 0; e < SCAN_ITEMS; ++e) {
-        const int j = j0 + e;
-        if ((uint32_t)j >= Rprev) break;
-        const uint64_t prevC = cf;
-        cf += f[e];
-        cg += f[e] & ((1ull << FRAC_BITS) - 1);
-        r.C[j] = cf;
-        if (method == M_RESIDUAL) r.G[j] = cg;
-        uint32_t cnt = 0;
-        if (method == M_NEAREST) {
-            const uint4x x = philox((uint32_t)j, DOM_RESAMPLE | (r.run << 8) | RULE_NEAREST, (uint32_t)i, 0u,
-                                    p.k0, p.k1);
-            const uint64_t u40 = (((uint64_t)x.y << 32) | x.x) >> 24;
-            cnt = (uint32_t)(f[e] >> FRAC_BITS) +
-                  (u40 < (f[e] & ((1ull << FRAC_BITS) - 1)) ? 1u : 0u);
-        } else if (method == M_SYSTEMATIC) {
-            cnt = (uint32_t)(sys_below(cf, r.R, T, usys) - sys_below(prevC, r.R, T, usys));
-        } else if (method == M_RESIDUAL) {
-            cnt = (uint32_t)(f[e] >> FRAC_BITS);
-        } else if (method == M_POISSON) {
-            const double lam = scalbn((double)f[e], -FRAC_BITS);
-            const uint32_t M = (uint32_t)(f[e] >> 44) + 1u;
-            const double lc = __ddiv_rn(lam, (double)M);
-            uint32_t total = 0;
-            for (uint32_t m = 0; m < M; ++m) {
-                const uint4x x = philox((uint32_t)j, DOM_RESAMPLE | (r.run << 8) | RULE_POISSON, (uint32_t)i, m,
-                                        p.k0, p.k1);
-                const double u = scalbn((double)((((uint64_t)x.y << 32) | x.x) >> 11), -53);
-                double pr = exp_taylor(-lc);
-                double Pc = pr;
-                uint32_t k = 0;
-                while (u >= Pc) {
-                    k += 1;
-                    if (k > POISSON_KMAX) {
-                        kmax = true;
-                        break;
-                    }
-                    pr = __ddiv_rn(__dmul_rn(pr, lc), (double)k);
-                    Pc = __dadd_rn(Pc, pr);
-                }
-                total += k;
-            }
-            cnt = total;
-        }
-        r.counts[j] = cnt;
-    }
-    if (kmax) atomicCAS(&st->status, S_OK, S_KMAX);
 }
 
 // multinomial draws (multinomial rule: R draws over C; residual rule: R_res
@@ -669,90 +603,6 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_draws(KParams p) {
         }
         atomicAdd(&r.counts[lo], 1u);
     }
-}
-
-// --------------------------------------------------------------------------
-// scan of the counts and scatter of the ancestor array
-// --------------------------------------------------------------------------
-__global__ void __launch_bounds__(SCAN_THREADS) k_rsum(KParams p) {
-    const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
-    const uint32_t b = blockIdx.x - r.blk0;
-    const DevState* st = r.st;
-    if (st->status != S_OK) return;
-    if (p.alpha >= 0.0 && !st->resample) return;
-    __shared__ uint64_t sh[33];
-    const uint32_t Rprev = st->R_prev;
-    const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
-    uint64_t s = 0;
-    for (int e = 0; e < SCAN_ITEMS; ++e) {
-        const int j = j0 + e;
-        if ((uint32_t)j < Rprev) s += r.counts[j];
-    }
-    uint64_t tot;
-    block_excl_scan(s, sh, &tot);
-    if (threadIdx.x == 0) r.partA[b] = tot;
-}
-
-__global__ void __launch_bounds__(1024) k_rscan(KParams p) {
-    const RunDesc& r = p.runs[blockIdx.x];
-    DevState* st = r.st;
-    if (st->status != S_OK) return;
-    if (p.alpha >= 0.0 && !st->resample) return;  // R_i = R_{i-1}
-    __shared__ uint64_t tA;
-    scan_partials(r.partA, r.offA, r.nblk, &tA);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // a population that outgrows its capacity, or dies out, stops the run
-        if (tA > (uint64_t)r.Rcap || tA == 0) st->status = S_CAPACITY;
-        else st->R_cur = (uint32_t)tA;
-    }
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_scatter(KParams p) {
-    const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
-    const uint32_t b = blockIdx.x - r.blk0;
-    const DevState* st = r.st;
-    if (st->status != S_OK) return;
-    if (p.alpha >= 0.0 && !st->resample) return;  // identity written by k_counts
-    __shared__ uint64_t sh[33];
-    __shared__ double sd[SCAN_THREADS];
-    const int i = st->step;
-    const int32_t* E = r.E[(i - 1) & 1];
-    const int dN = p.d * r.N;
-    const uint32_t Rprev = st->R_prev, lmin = st->lmin;
-    const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
-    uint32_t rc[SCAN_ITEMS];
-    uint64_t s = 0;
-#pragma unroll
-    for (int e = 0; e < SCAN_ITEMS; ++e) {
-        const int j = j0 + e;
-        rc[e] = ((uint32_t)j < Rprev) ? r.counts[j] : 0u;
-        s += rc[e];
-    }
-    uint64_t tot;
-    uint64_t o = block_excl_scan(s, sh, &tot) + r.offA[b];
-    double sv = 0.0;
-    for (int e = 0; e < SCAN_ITEMS; ++e) {
-        const int j = j0 + e;
-        if ((uint32_t)j >= Rprev) break;
-        const uint32_t fj = rc[e] ? r.fam[(i - 1) & 1][j] : 0u;
-        for (uint32_t c = 0; c < rc[e]; ++c) {
-            r.anc[o + c] = (uint32_t)j;
-            r.fam[i & 1][o + c] = fj;
-        }
-        o += rc[e];
-        const double tau = scalbn((double)f_of(j, p, r, st, dN, E, lmin), -FRAC_BITS);
-        const double dl = __dsub_rn((double)rc[e], tau);
-        sv = __dadd_rn(sv, __dmul_rn(dl, dl));
-    }
-    // fixed-order tree reduction of the block's sampling-variance terms
-    sd[threadIdx.x] = sv;
-    __syncthreads();
-    for (int h = SCAN_THREADS / 2; h >= 1; h >>= 1) {
-        if ((int)threadIdx.x < h) sd[threadIdx.x] = __dadd_rn(sd[threadIdx.x], sd[threadIdx.x + h]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) r.partD[b] = sd[0];
 }
 
 // --------------------------------------------------------------------------
@@ -896,10 +746,13 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
             v[3][e] = __dmul_rn(w, fabs(M));
             v[4][e] = __dmul_rn(w, __dmul_rn(M, M));
         }
-        for (int q = 0; q < 5; ++q) {
-            const double root = tree_threads(tree_regs<SCAN_ITEMS>(v[q]), sd);
-            if (threadIdx.x == 0) r.opart[5 * b + q] = root;
-        }
+        double t5[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) t5[q] = tree_regs<SCAN_ITEMS>(v[q]);
+        tree_threads(t5, sd);
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int q = 0; q < 5; ++q) r.opart[5 * b + q] = t5[q];
     }
     // the run's last family block to finish closes the step: its ticket says every
     // other block's partials are written (each fenced them before its ticket)
@@ -939,19 +792,31 @@ __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int
         // (PARTIAL_MAX_BLOCKS leaves in all, zero past the run's blocks)
         const int nb = r.nblk;
         constexpr int LEAVES = PARTIAL_MAX_BLOCKS / 256;
-        for (int q = 0; q < 5; ++q) {
-            double x[LEAVES];
+        double t5[5];
 #pragma unroll
-            for (int k = 0; k < LEAVES; ++k) {
-                const int bb = LEAVES * threadIdx.x + k;
-                x[k] = bb < nb ? __ldcg(&r.opart[5 * bb + q]) : 0.0;
+        for (int q = 0; q < 5; ++q) {
+            if (nb <= 256) {  // a leaf per thread; the leaves past it are zeros
+                t5[q] = (int)threadIdx.x < nb ? __ldcg(&r.opart[5 * threadIdx.x + q]) : 0.0;
+            } else {  // the thread's LEAVES leaves as a tree, in eighths
+                double x8[8];
+                for (int h = 0; h < 8; ++h) {
+                    double x[LEAVES / 8];
+#pragma unroll
+                    for (int k = 0; k < LEAVES / 8; ++k) {
+                        const int bb = LEAVES * threadIdx.x + LEAVES / 8 * h + k;
+                        x[k] = bb < nb ? __ldcg(&r.opart[5 * bb + q]) : 0.0;
+                    }
+                    x8[h] = tree_regs<LEAVES / 8>(x);
+                }
+                t5[q] = tree_regs<8>(x8);
             }
-            const double root = tree_threads(tree_regs<LEAVES>(x), ws);
-            if (threadIdx.x == 0) {
-                TraceRow* tr = r.trace + i;
-                double* dst[5] = {&tr->wsum, &tr->wE, &tr->wE2, &tr->wAM, &tr->wM2};
-                *dst[q] = root;
-            }
+        }
+        tree_threads(t5, ws, nb <= 256 ? nb : 256);
+        if (threadIdx.x == 0) {
+            TraceRow* tr = r.trace + i;
+            double* dst[5] = {&tr->wsum, &tr->wE, &tr->wE2, &tr->wAM, &tr->wM2};
+#pragma unroll
+            for (int q = 0; q < 5; ++q) *dst[q] = t5[q];
         }
     }
     if (threadIdx.x == 0) {
@@ -1066,11 +931,9 @@ __device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDe
                                                    DevState* st, int b,
                                                    const uint32_t (&rc)[SCAN_ITEMS], uint64_t* sh,
                                                    double* sd, int* flag_sh,
-                                                   const uint64_t (&fv)[SCAN_ITEMS], bool have_f) {
+                                                   const uint64_t (&fv)[SCAN_ITEMS]) {
     const int i = st->step;
-    const int32_t* E = r.E[(i - 1) & 1];
-    const int dN = p.d * r.N;
-    const uint32_t Rprev = st->R_prev, lmin = st->lmin;
+    const uint32_t Rprev = st->R_prev;
     const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
     uint64_t sum = 0;
 #pragma unroll
@@ -1111,8 +974,7 @@ __device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDe
         o += rc[e];
         skew |= rc[e] > 4u;
         if (!in) continue;
-        const double tau =
-            scalbn((double)(have_f ? fv[e] : f_of(j, p, r, st, dN, E, lmin)), -FRAC_BITS);
+        const double tau = scalbn((double)fv[e], -FRAC_BITS);
         const double dl = __dsub_rn((double)rc[e], tau);
         sv = __dadd_rn(sv, __dmul_rn(dl, dl));
     }
@@ -1169,6 +1031,20 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
     const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
     DevState* st = r.st;
     if (st->status != S_OK) return;
+    if (p.alpha >= 0.0 && !st->resample) {
+        // partial resampling keeps every replica once: identity counts, ancestors and
+        // families, no sampling variance
+        const int i = st->step;
+        const uint32_t b = blockIdx.x - r.blk0, Rprev = st->R_prev;
+        for (uint32_t j = b * SCAN_CHUNK + threadIdx.x; j < min(Rprev, (b + 1) * SCAN_CHUNK);
+             j += SCAN_THREADS) {
+            r.counts[j] = 1u;
+            r.anc[j] = j;
+            r.fam[i & 1][j] = r.fam[(i - 1) & 1][j];
+        }
+        if (threadIdx.x == 0) r.partD[b] = 0.0;
+        return;
+    }
     __shared__ uint64_t sh[33];
     __shared__ double sd[SCAN_THREADS];
     __shared__ int sb, okf;
@@ -1185,7 +1061,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
 #pragma unroll
     for (int e = 0; e < SCAN_ITEMS; ++e) {
         const int j = j0 + e;
-        f[e] = ((uint32_t)j < Rprev) ? f_of(j, p, r, st, dN, E, lmin) : 0ull;
+        f[e] = 0ull;
+        if ((uint32_t)j < Rprev) f[e] = p.alpha >= 0.0 ? r.C[j] : r.flev[level_of(E[j], dN) - (int)lmin];
         sf += f[e];
         sg += f[e] & ((1ull << FRAC_BITS) - 1);
     }
@@ -1240,27 +1117,16 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
         } else if (method == M_MULTINOMIAL) {
             r.C[j] = cf;
         } else {  // Poisson
+            // sequential inversion per chunk of mean lc <= 16; poisson_draw decides in FP32
+            // where that is certain
             const double lam = scalbn((double)f[e], -FRAC_BITS);
             const uint32_t M = (uint32_t)(f[e] >> 44) + 1u;
-            const double lc = __ddiv_rn(lam, (double)M);
+            const double lc = M == 1u ? lam : __ddiv_rn(lam, (double)M);
             uint32_t total = 0;
             for (uint32_t m = 0; m < M; ++m) {
                 const uint4x x = philox((uint32_t)j, DOM_RESAMPLE | (r.run << 8) | RULE_POISSON, (uint32_t)i, m,
                                         p.k0, p.k1);
-                const double u = scalbn((double)((((uint64_t)x.y << 32) | x.x) >> 11), -53);
-                double pr = exp_taylor(-lc);
-                double Pc = pr;
-                uint32_t k = 0;
-                while (u >= Pc) {
-                    k += 1;
-                    if (k > POISSON_KMAX) {
-                        kmax = true;
-                        break;
-                    }
-                    pr = __ddiv_rn(__dmul_rn(pr, lc), (double)k);
-                    Pc = __dadd_rn(Pc, pr);
-                }
-                total += k;
+                total += poisson_draw(lc, ((uint64_t)x.y << 32) | x.x, kmax);
             }
             cnt = total;
         }
@@ -1275,14 +1141,14 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
         if (threadIdx.x == 0 && b == r.nblk - 1) r.tick[0] = 0u;
         return;
     }
-    count_scan_scatter(p, r, st, b, rc, sh, sd, &okf, f, true);
+    count_scan_scatter(p, r, st, b, rc, sh, sd, &okf, f);
 }
 
 // multinomial / residual: the copy numbers are complete after k_draws
 __global__ void __launch_bounds__(SCAN_THREADS) k_cscan(KParams p) {
     const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
     DevState* st = r.st;
-    if (st->status != S_OK) return;
+    if (st->status != S_OK || (p.alpha >= 0.0 && !st->resample)) return;
     __shared__ uint64_t sh[33];
     __shared__ double sd[SCAN_THREADS];
     __shared__ int sb, okf;
@@ -1290,13 +1156,15 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_cscan(KParams p) {
     const uint32_t Rprev = st->R_prev;
     const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
     uint32_t rc[SCAN_ITEMS];
+    uint64_t f[SCAN_ITEMS];  // from the prefix C
 #pragma unroll
     for (int e = 0; e < SCAN_ITEMS; ++e) {
         const int j = j0 + e;
-        rc[e] = ((uint32_t)j < Rprev) ? r.counts[j] : 0u;
+        const bool in = (uint32_t)j < Rprev;
+        rc[e] = in ? r.counts[j] : 0u;
+        f[e] = in ? r.C[j] - (j > 0 ? r.C[j - 1] : 0ull) : 0ull;
     }
-    const uint64_t nof[SCAN_ITEMS] = {};
-    count_scan_scatter(p, r, st, b, rc, sh, sd, &okf, nof, false);
+    count_scan_scatter(p, r, st, b, rc, sh, sd, &okf, f);
 }
 
 // --------------------------------------------------------------------------
@@ -1305,22 +1173,13 @@ cudaError_t launch_resample(const KParams& p, cudaStream_t s, int64_t* launches)
     int n = 1;
     if (p.alpha >= 0.0) {
         // partial resampling: the expected copies depend on per-replica weights, so
-        // their total comes from a scan over the replicas
+        // their total comes from a sum over the replicas
         k_pw_update<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
         k_pw_final<<<p.M, 1024, 0, s>>>(p);
         k_fsum<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
-        k_fscan<<<p.M, 1024, 0, s>>>(p);
-        k_counts<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
-        n += 5;
-        if (p.method == M_MULTINOMIAL || p.method == M_RESIDUAL) {
-            k_draws<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
-            ++n;
-        }
-        k_rsum<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
-        k_rscan<<<p.M, 1024, 0, s>>>(p);
-        k_scatter<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
         n += 3;
-    } else if (p.method == M_MULTINOMIAL || p.method == M_RESIDUAL) {
+    }
+    if (p.method == M_MULTINOMIAL || p.method == M_RESIDUAL) {
         k_resample<false><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
         k_draws<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
         k_cscan<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
