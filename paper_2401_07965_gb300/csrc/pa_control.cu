@@ -11,6 +11,7 @@
 // then after every temperature step: it writes the next step's entries of the step
 // tables from tables precomputed on the host, so the PA step itself is unchanged and
 // stays bit-exact.
+#include <algorithm>
 #include <cmath>
 #include <cuda_bf16.h>
 
@@ -44,18 +45,16 @@ cudaError_t launch_control(const KParams& p, cudaStream_t s) {
 }
 
 // --------------------------------------------------------------------------
-// training: forward over a batch (parameters rounded to BF16 as in inference)
+// inference over a batch (BF16 parameters; one product after the other in index
+// order, bias last, no fused multiply-add: the order of the controller's step)
 // --------------------------------------------------------------------------
-template <bool MASTER>
-__global__ void __launch_bounds__(64) k_mlp_fwd(const void* params, const float* __restrict__ X,
-                                                int B, float* __restrict__ H1,
-                                                float* __restrict__ H2, float* __restrict__ Y) {
+__global__ void __launch_bounds__(64) k_mlp_fwd(const uint16_t* __restrict__ params,
+                                                const float* __restrict__ X, int B,
+                                                float* __restrict__ Y) {
     __shared__ float xs[ROWS][MLP_IN], a1[ROWS][MLP_HID], a2[ROWS][MLP_HID];
     __shared__ float W2s[MLP_HID * MLP_HID];
     const int t = threadIdx.x, r0 = blockIdx.x * ROWS;
-    auto P = [&](int idx) -> float {
-        return MASTER ? bf_round(((const float*)params)[idx]) : bf(((const uint16_t*)params)[idx]);
-    };
+    auto P = [&](int idx) -> float { return bf(params[idx]); };
     for (int e = t; e < ROWS * MLP_IN; e += 64) {
         const int rr = e / MLP_IN, k = e % MLP_IN;
         xs[rr][k] = (r0 + rr < B) ? X[(size_t)(r0 + rr) * MLP_IN + k] : 0.0f;
@@ -84,116 +83,274 @@ __global__ void __launch_bounds__(64) k_mlp_fwd(const void* params, const float*
     for (int k = 0; k < MLP_HID; ++k) acc = __fadd_rn(acc, __fmul_rn(P(OFF_W3 + o * MLP_HID + k), a2[rr][k]));
     acc = __fadd_rn(acc, P(OFF_B3 + o));
     if (r0 + rr < B) Y[(size_t)(r0 + rr) * MLP_OUT + o] = acc;
-    if (H1)
-        for (int q = 0; q < ROWS; ++q)
-            if (r0 + q < B) {
-                H1[(size_t)(r0 + q) * MLP_HID + t] = a1[q][t];
-                H2[(size_t)(r0 + q) * MLP_HID + t] = a2[q][t];
-            }
 }
 
-// backward of the mean squared error over masked outputs; per-CTA partial
-// gradients (row order fixed) in part[block][MLP_NPARAM + 1] (last: loss)
-__global__ void __launch_bounds__(64) k_mlp_bwd(const float* __restrict__ params,
-                                                const float* __restrict__ X,
-                                                const float* __restrict__ Yt,
-                                                const float* __restrict__ mask, int B,
-                                                float norm, const float* __restrict__ H1,
-                                                const float* __restrict__ H2,
-                                                const float* __restrict__ Y,
-                                                float* __restrict__ part) {
-    __shared__ float dY[ROWS][MLP_OUT], d2[ROWS][MLP_HID], d1[ROWS][MLP_HID];
-    __shared__ float a1[ROWS][MLP_HID], a2[ROWS][MLP_HID], xs[ROWS][MLP_IN];
-    __shared__ float lossv[64];
-    const int t = threadIdx.x, r0 = blockIdx.x * ROWS;
-    for (int e = t; e < ROWS * MLP_HID; e += 64) {
-        const int rr = e / MLP_HID, j = e % MLP_HID;
-        const bool in = r0 + rr < B;
-        a1[rr][j] = in ? H1[(size_t)(r0 + rr) * MLP_HID + j] : 0.0f;
-        a2[rr][j] = in ? H2[(size_t)(r0 + rr) * MLP_HID + j] : 0.0f;
+// --------------------------------------------------------------------------
+// Training gradients (FP32, parameters rounded to BF16 as in inference).  A CTA of 8 GR
+// threads takes `rows` consecutive rows, GR at a time, through the forward and the backward
+// pass in shared memory and adds up its part of every gradient in registers; the parts are
+// summed in CTA order by k_mlp_reduce.  The products with W2 and the sum over rows of its
+// gradient are 64 x 64 x GR each: a thread holds a 4 x 2 tile of the result and reads a
+// 128-bit and a 64-bit word of shared memory per 8 fused multiply-adds.
+// What bounds it: shared-memory latency on one CTA per SM (30 k flops per row).  GR = 32, 64
+// or 96, the least that takes the rows of one of 152 CTAs in one pass: 12040 rows are 151
+// CTAs of 80 rows; two passes of 64 with 256 threads took 33 us, one pass 22 us (the whole
+// update of 12040 rows: 66 us with the forward pass stored and read back, now 30).
+// --------------------------------------------------------------------------
+constexpr int LDW = MLP_HID + 4;  // padded rows of units: 16-byte aligned
+
+template <int GR>
+struct GradSmem {
+    static constexpr int LDR = GR + 4;  // padded rows of batch rows
+    float w2[MLP_HID * LDW];            // W2[j][k]
+    float w2t[MLP_HID * LDW];           // W2 transposed
+    float a1t[MLP_HID * LDR];           // H1[k][row]
+    float a2t[MLP_HID * LDR];           // H2[j][row]
+    float d2t[MLP_HID * LDR];           // dH2[j][row]
+    float d1t[MLP_HID * LDR];           // dH1[k][row]
+    float d2[GR * LDW];                 // dH2[row][j]
+    float a1[GR * LDW];                 // H1[row][k]
+    float w1[MLP_HID * MLP_IN], w3[MLP_OUT * MLP_HID], b1[MLP_HID], b2[MLP_HID], b3[MLP_OUT];
+    float xs[GR][MLP_IN];
+    float dy[GR][MLP_OUT];
+    float loss[GR * MLP_OUT];
+};
+
+template <int GR>
+__global__ void __launch_bounds__(8 * GR) k_mlp_grad(const float* __restrict__ params,
+                                                     const float* __restrict__ X,
+                                                     const float* __restrict__ Yt,
+                                                     const float* __restrict__ mask, int B, int rows,
+                                                     float norm, float* __restrict__ part) {
+    constexpr int GT = 8 * GR, LDR = GradSmem<GR>::LDR;
+    extern __shared__ __align__(16) unsigned char raw[];
+    GradSmem<GR>& s = *reinterpret_cast<GradSmem<GR>*>(raw);
+    const int t = threadIdx.x, ti = t % (GR / 2), tj = t / (GR / 2);  // rows 2 ti.., units 4 tj..
+    for (int e = t; e < MLP_HID * MLP_HID; e += GT) {
+        const float v = bf_round(params[OFF_W2 + e]);
+        s.w2[(e >> 6) * LDW + (e & 63)] = v;
+        s.w2t[(e & 63) * LDW + (e >> 6)] = v;
     }
-    for (int e = t; e < ROWS * MLP_IN; e += 64) {
-        const int rr = e / MLP_IN, k = e % MLP_IN;
-        xs[rr][k] = (r0 + rr < B) ? X[(size_t)(r0 + rr) * MLP_IN + k] : 0.0f;
+    for (int e = t; e < MLP_HID * MLP_IN; e += GT) s.w1[e] = bf_round(params[OFF_W1 + e]);
+    if (t < MLP_OUT * MLP_HID) s.w3[t] = bf_round(params[OFF_W3 + t]);
+    if (t < MLP_HID) {
+        s.b1[t] = bf_round(params[OFF_B1 + t]);
+        s.b2[t] = bf_round(params[OFF_B2 + t]);
     }
-    {
-        const int rr = t >> 1, o = t & 1;
-        float g = 0.0f, l = 0.0f;
-        if (r0 + rr < B) {
-            const size_t id = (size_t)(r0 + rr) * MLP_OUT + o;
-            const float diff = __fsub_rn(Y[id], Yt[id]);
-            const float mk = mask[id];
-            g = __fmul_rn(__fmul_rn(2.0f, mk), __fmul_rn(diff, norm));
-            l = __fmul_rn(mk, __fmul_rn(diff, diff));
+    if (t < MLP_OUT) s.b3[t] = bf_round(params[OFF_B3 + t]);
+    // W2's gradient: tiles of 4 rows and WC columns on the first 1024 / WC threads
+    constexpr int WC = GR == 32 ? 4 : 2, WT2 = 16 * (MLP_HID / WC);
+    const int wi = t % (MLP_HID / WC), wj = t / (MLP_HID / WC);
+    constexpr int N1 = GT >= 512 ? 1 : 2;  // W1 elements of a thread (t < 512 / N1)
+    const int q = t - (GT - 256);          // the last 256 threads: W3, b1, b2; b3 and the loss
+    float g2[4][WC] = {}, g1[N1] = {};
+    float g3 = 0.0f, gl = 0.0f;
+    const int r0 = blockIdx.x * rows, r1 = min(r0 + rows, B);
+    for (int base = r0; base < r1; base += GR) {
+        const int n = min(GR, r1 - base);
+        __syncthreads();
+        {
+            const int rr = t / MLP_IN;  // GR x 8 values, one per thread
+            s.xs[rr][t % MLP_IN] = rr < n ? X[(size_t)(base + rr) * MLP_IN + t % MLP_IN] : 0.0f;
         }
-        dY[rr][o] = g;
-        lossv[t] = l;
+        __syncthreads();
+        // H1: unit t & 63 of rows t >> 6, + GR / 8, ...; 0 in rows past the last
+        {
+            const int k = t & 63;
+            float w[MLP_IN];
+#pragma unroll
+            for (int c = 0; c < MLP_IN; ++c) w[c] = s.w1[k * MLP_IN + c];
+            const float bb = s.b1[k];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+                const int rr = (t >> 6) + GR / 8 * m;
+                float acc = 0.0f;
+#pragma unroll
+                for (int c = 0; c < MLP_IN; ++c) acc = __fmaf_rn(w[c], s.xs[rr][c], acc);
+                acc += bb;
+                const float h = acc > 0.0f && rr < n ? acc : 0.0f;
+                s.a1[rr * LDW + k] = h;
+                s.a1t[k * LDR + rr] = h;
+            }
+        }
+        __syncthreads();
+        // H2[j][row] = relu(sum_k W2[j][k] H1[k][row] + b2[j])
+        {
+            float acc[4][2] = {};
+#pragma unroll 8
+            for (int k = 0; k < MLP_HID; ++k) {
+                const float4 w = *reinterpret_cast<const float4*>(&s.w2t[k * LDW + 4 * tj]);
+                const float2 h = *reinterpret_cast<const float2*>(&s.a1t[k * LDR + 2 * ti]);
+                const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    acc[u][0] = __fmaf_rn(wv[u], h.x, acc[u][0]);
+                    acc[u][1] = __fmaf_rn(wv[u], h.y, acc[u][1]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float bb = s.b2[4 * tj + u];
+                float2 h;
+                h.x = 2 * ti + 0 < n ? fmaxf(acc[u][0] + bb, 0.0f) : 0.0f;
+                h.y = 2 * ti + 1 < n ? fmaxf(acc[u][1] + bb, 0.0f) : 0.0f;
+                *reinterpret_cast<float2*>(&s.a2t[(4 * tj + u) * LDR + 2 * ti]) = h;
+            }
+        }
+        __syncthreads();
+        // outputs, their errors and gradients: two threads per row
+        if (t < GR * MLP_OUT) {
+            const int rr = t >> 1, o = t & 1;
+            float acc = 0.0f;
+#pragma unroll 16
+            for (int j = 0; j < MLP_HID; ++j) acc = __fmaf_rn(s.w3[o * MLP_HID + j], s.a2t[j * LDR + rr], acc);
+            acc += s.b3[o];
+            float g = 0.0f, l = 0.0f;
+            if (rr < n) {
+                const size_t id = (size_t)(base + rr) * MLP_OUT + o;
+                const float diff = acc - Yt[id], mk = mask[id];
+                g = 2.0f * mk * (diff * norm);
+                l = mk * (diff * diff);
+            }
+            s.dy[rr][o] = g;
+            s.loss[t] = l;
+        }
+        __syncthreads();
+        // dH2 (unit t & 63 of rows t >> 6, + GR / 8, ...); zero past the last row (dY = 0)
+        {
+            const int j = t & 63;
+            const float w30 = s.w3[j], w31 = s.w3[MLP_HID + j];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+                const int rr = (t >> 6) + GR / 8 * m;
+                const float v = __fmaf_rn(s.dy[rr][1], w31, s.dy[rr][0] * w30);
+                const float d = s.a2t[j * LDR + rr] > 0.0f ? v : 0.0f;
+                s.d2t[j * LDR + rr] = d;
+                s.d2[rr * LDW + j] = d;
+            }
+        }
+        __syncthreads();
+        // dH1[k][row] = [H1 > 0] sum_j W2[j][k] dH2[j][row]; W2's gradient [j][k] += sum_row
+        {
+            float acc[4][2] = {};
+#pragma unroll 8
+            for (int j = 0; j < MLP_HID; ++j) {
+                const float4 w = *reinterpret_cast<const float4*>(&s.w2[j * LDW + 4 * tj]);
+                const float2 d = *reinterpret_cast<const float2*>(&s.d2t[j * LDR + 2 * ti]);
+                const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    acc[u][0] = __fmaf_rn(wv[u], d.x, acc[u][0]);
+                    acc[u][1] = __fmaf_rn(wv[u], d.y, acc[u][1]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int o = (4 * tj + u) * LDR + 2 * ti;
+                const float2 h = *reinterpret_cast<const float2*>(&s.a1t[o]);
+                float2 d;
+                d.x = h.x > 0.0f ? acc[u][0] : 0.0f;
+                d.y = h.y > 0.0f ? acc[u][1] : 0.0f;
+                *reinterpret_cast<float2*>(&s.d1t[o]) = d;
+            }
+        }
+        if (t < WT2) {
+#pragma unroll 8
+            for (int rr = 0; rr < GR; ++rr) {
+                const float4 d = *reinterpret_cast<const float4*>(&s.d2[rr * LDW + 4 * wj]);
+                const float dv[4] = {d.x, d.y, d.z, d.w};
+                float hv[WC];
+#pragma unroll
+                for (int c = 0; c < WC; c += 2) {
+                    const float2 h = *reinterpret_cast<const float2*>(&s.a1[rr * LDW + WC * wi + c]);
+                    hv[c] = h.x;
+                    hv[c + 1] = h.y;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int c = 0; c < WC; ++c) g2[u][c] = __fmaf_rn(dv[u], hv[c], g2[u][c]);
+            }
+        }
+        __syncthreads();
+        if (t < 512 / N1)
+#pragma unroll
+            for (int m = 0; m < N1; ++m) {
+                const int e = t + GT * m, j = e / MLP_IN, k = e % MLP_IN;
+                float acc = 0.0f;
+#pragma unroll 16
+                for (int rr = 0; rr < GR; ++rr) acc = __fmaf_rn(s.d1t[j * LDR + rr], s.xs[rr][k], acc);
+                g1[m] += acc;
+            }
+        if (q >= 0) {
+            float acc = 0.0f;
+            if (q < MLP_OUT * MLP_HID) {  // W3
+                const int o = q >> 6, j = q & 63;
+#pragma unroll 16
+                for (int rr = 0; rr < GR; ++rr) acc = __fmaf_rn(s.dy[rr][o], s.a2t[j * LDR + rr], acc);
+            } else {  // b1, b2
+                const int u = q - 128;
+                const float* row = u < 64 ? &s.d1t[u * LDR] : &s.d2t[(u - 64) * LDR];
+#pragma unroll 16
+                for (int rr = 0; rr < GR; ++rr) acc += row[rr];
+            }
+            g3 += acc;
+            if (q < 64) {  // two warps: b3 (lanes o, o + 2, ...) and the loss
+                float v = 0.0f;
+                const int l = q & 31;
+                if (q < 32) {
+                    for (int rr = l >> 1; rr < GR; rr += 16) v += s.dy[rr][l & 1];
+                } else {
+                    for (int e = l; e < GR * MLP_OUT; e += 32) v += s.loss[e];
+                    v += __shfl_xor_sync(0xffffffffu, v, 1);
+                }
+                for (int o = 16; o >= 2; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                gl += v;
+            }
+        }
     }
-    __syncthreads();
-    // dH2 (thread t = hidden unit j)
-    for (int rr = 0; rr < ROWS; ++rr) {
-        float acc = 0.0f;
-        for (int o = 0; o < MLP_OUT; ++o)
-            acc = __fadd_rn(acc, __fmul_rn(dY[rr][o], bf_round(params[OFF_W3 + o * MLP_HID + t])));
-        d2[rr][t] = a2[rr][t] > 0.0f ? acc : 0.0f;
-    }
-    __syncthreads();
-    // dH1 (thread t = hidden unit i)
-    for (int rr = 0; rr < ROWS; ++rr) {
-        float acc = 0.0f;
-        for (int j = 0; j < MLP_HID; ++j)
-            acc = __fadd_rn(acc, __fmul_rn(d2[rr][j], bf_round(params[OFF_W2 + j * MLP_HID + t])));
-        d1[rr][t] = a1[rr][t] > 0.0f ? acc : 0.0f;
-    }
-    __syncthreads();
     float* g = part + (size_t)blockIdx.x * (MLP_NPARAM + 1);
-    // W1 row t, b1[t]
-    for (int k = 0; k < MLP_IN; ++k) {
-        float acc = 0.0f;
-        for (int rr = 0; rr < ROWS; ++rr) acc = __fadd_rn(acc, __fmul_rn(d1[rr][t], xs[rr][k]));
-        g[OFF_W1 + t * MLP_IN + k] = acc;
-    }
-    {
-        float acc = 0.0f;
-        for (int rr = 0; rr < ROWS; ++rr) acc = __fadd_rn(acc, d1[rr][t]);
-        g[OFF_B1 + t] = acc;
-    }
-    // W2 row t (output unit t), b2[t]
-    for (int k = 0; k < MLP_HID; ++k) {
-        float acc = 0.0f;
-        for (int rr = 0; rr < ROWS; ++rr) acc = __fadd_rn(acc, __fmul_rn(d2[rr][t], a1[rr][k]));
-        g[OFF_W2 + t * MLP_HID + k] = acc;
-    }
-    {
-        float acc = 0.0f;
-        for (int rr = 0; rr < ROWS; ++rr) acc = __fadd_rn(acc, d2[rr][t]);
-        g[OFF_B2 + t] = acc;
-    }
-    // W3 column t, b3
-    for (int o = 0; o < MLP_OUT; ++o) {
-        float acc = 0.0f;
-        for (int rr = 0; rr < ROWS; ++rr) acc = __fadd_rn(acc, __fmul_rn(dY[rr][o], a2[rr][t]));
-        g[OFF_W3 + o * MLP_HID + t] = acc;
-    }
-    if (t < MLP_OUT) {
-        float acc = 0.0f;
-        for (int rr = 0; rr < ROWS; ++rr) acc = __fadd_rn(acc, dY[rr][t]);
-        g[OFF_B3 + t] = acc;
-    }
-    if (t == 0) {
-        float acc = 0.0f;
-        for (int q = 0; q < 64; ++q) acc = __fadd_rn(acc, lossv[q]);
-        g[MLP_NPARAM] = __fmul_rn(acc, norm);
+    if (t < WT2)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int c = 0; c < WC; ++c) g[OFF_W2 + (4 * wj + u) * MLP_HID + WC * wi + c] = g2[u][c];
+    if (t < 512 / N1)
+#pragma unroll
+        for (int m = 0; m < N1; ++m) g[OFF_W1 + t + GT * m] = g1[m];
+    if (q >= 0) {
+        g[q < 128 ? OFF_W3 + q : (q < 192 ? OFF_B1 - 128 : OFF_B2 - 192) + q] = g3;
+        if (q < MLP_OUT) g[OFF_B3 + q] = gl;
+        if (q == 32) g[MLP_NPARAM] = gl * norm;
     }
 }
 
-// fixed-order sum of the per-CTA partials
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nb, float* __restrict__ grads,
-                             float* __restrict__ loss) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > MLP_NPARAM) return;
+template <int GR>
+cudaError_t launch_grad(const float* params, const float* X, const float* Yt, const float* mask,
+                        int B, int rows, unsigned nb, float norm, float* part, cudaStream_t s) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_mlp_grad<GR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem<GR>));
+    if (e != cudaSuccess) return e;
+    k_mlp_grad<GR><<<nb, 8 * GR, sizeof(GradSmem<GR>), s>>>(params, X, Yt, mask, B, rows, norm, part);
+    return cudaGetLastError();
+}
+
+// fixed-order sum of the per-CTA parts: eight warps of a CTA take the parts b = w, w + 8,
+// ... of 32 parameters, then the eight sums in order
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ part, int nb,
+                                                    float* __restrict__ grads,
+                                                    float* __restrict__ loss) {
+    __shared__ float sh[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
     float acc = 0.0f;
-    for (int b = 0; b < nb; ++b) acc = __fadd_rn(acc, part[(size_t)b * (MLP_NPARAM + 1) + k]);
+    if (k <= MLP_NPARAM)
+#pragma unroll 8
+        for (int b = w; b < nb; b += 8) acc += part[(size_t)b * (MLP_NPARAM + 1) + k];
+    sh[w][lane] = acc;
+    __syncthreads();
+    if (w != 0 || k > MLP_NPARAM) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) acc += sh[q][lane];
     if (k < MLP_NPARAM) grads[k] = acc;
     else if (loss) *loss = acc;
 }
@@ -234,8 +391,7 @@ size_t pa_mlp_scratch_bytes(int32_t B) {
 pa_status pa_mlp_forward(const uint16_t* params_bf16, const float* X, int32_t B, float* Y,
                          void* cuda_stream) {
     if (!params_bf16 || !X || !Y || B <= 0) return PA_ERR_ARG;
-    k_mlp_fwd<false><<<(unsigned)mlp_blocks(B), 64, 0, (cudaStream_t)cuda_stream>>>(
-        params_bf16, X, B, nullptr, nullptr, Y);
+    k_mlp_fwd<<<(unsigned)mlp_blocks(B), 64, 0, (cudaStream_t)cuda_stream>>>(params_bf16, X, B, Y);
     return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
 }
 
@@ -245,15 +401,17 @@ pa_status pa_mlp_gradients(const float* params, const float* X, const float* Yt,
     if (!params || !X || !Yt || !mask || !grads || B <= 0 || !scratch) return PA_ERR_ARG;
     if (scratch_bytes < pa_mlp_scratch_bytes(B)) return PA_ERR_NOMEM;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    float* H1 = (float*)scratch;
-    float* H2 = H1 + (size_t)B * MLP_HID;
-    float* Y = H2 + (size_t)B * MLP_HID;
-    float* part = Y + (size_t)B * MLP_OUT;
-    const unsigned nb = (unsigned)mlp_blocks(B);
+    // one CTA per SM; the scratch holds a part per ROWS rows, which is never fewer
+    const int rows = std::max(ROWS, (B + 151) / 152);
+    const unsigned nb = (unsigned)((B + rows - 1) / rows);
+    float* part = (float*)scratch;
     const float norm = 1.0f / (float)(B * MLP_OUT);
-    k_mlp_fwd<true><<<nb, 64, 0, s>>>(params, X, B, H1, H2, Y);
-    k_mlp_bwd<<<nb, 64, 0, s>>>(params, X, Yt, mask, B, norm, H1, H2, Y, part);
-    k_mlp_reduce<<<(MLP_NPARAM + 256) / 256, 256, 0, s>>>(part, (int)nb, grads, loss);
+    const cudaError_t e =
+        rows <= 32   ? launch_grad<32>(params, X, Yt, mask, B, rows, nb, norm, part, s)
+        : rows <= 64 ? launch_grad<64>(params, X, Yt, mask, B, rows, nb, norm, part, s)
+                     : launch_grad<96>(params, X, Yt, mask, B, rows, nb, norm, part, s);
+    if (e != cudaSuccess) return PA_ERR_CUDA;
+    k_mlp_reduce<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, s>>>(part, (int)nb, grads, loss);
     return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
 }
 
