@@ -299,8 +299,8 @@ pa_status pa_set_wait_test(pa_ctx *ctx, int32_t on);
  *
  * Scratch: one statically allocated device array (about 1.3 MB) that every
  * GPU loading the library holds until the process exits.  Every call shares
- * it and it keeps the last call's contents (the call clears what must start
- * at zero), so calls whose kernels overlap on the GPU -- on different streams,
+ * it and leaves its counts at zero for the next (one launch up to 2048
+ * energies, two beyond), so calls whose kernels overlap on the GPU -- on different streams,
  * or from several host threads -- race and must be serialised by the caller.
  * Each call looks up the array's device address with the caller's device
  * current; the first call on a device loads the library's device code there,
