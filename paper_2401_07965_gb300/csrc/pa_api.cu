@@ -766,6 +766,13 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
     }
     p.nblk_total = blk0;
     p.ngrp_total = grp0;
+    uint32_t mostR = 0;
+    int mostl = 0;
+    for (const RunHost& h : ctx->runs) {
+        mostR = std::max(mostR, h.Rcap);
+        mostl = std::max(mostl, h.nlev);
+    }
+    p.pop = pop_ctas(mostR, mostl, M, p.method, &p.pop_threads, &p.pop_levels);
 
     // The sweep's launches: the 2D kernel when all runs have one of its sides; else the
     // column walk, one launch per distinct side (at most four), each over the CTAs of the

@@ -98,6 +98,19 @@ __device__ __forceinline__ void mulhilo(uint32_t a, uint32_t b, uint32_t& hi, ui
     lo = (uint32_t)p;
 }
 
+// floor(2^40 x / S), the quotient rounded to FP64 first, for 0 <= x < 2^24 S, y = 1 / S rounded.  Two residual corrections of x y give the rounded quotient (Markstein, IBM
+// J. Res. Dev. 34, 1990): 5 operations of the FP64 pipe instead of a division's 20.  Below
+// 2^-45 S the result is 0, and from there on no operation meets a subnormal unless S is tiny
+// (partial resampling alone: a level sum is at least 1).
+__device__ __forceinline__ uint64_t fixed_quotient(double x, double S, double y) {
+    if (S < 0x1p-900) return __double2ull_rz(__dmul_rn(__ddiv_rn(x, S), 0x1p40));
+    if (!(x >= __dmul_rn(S, 0x1p-45))) return 0ull;
+    double q = __dmul_rn(x, y);
+    q = __fma_rn(__fma_rn(-q, S, x), y, q);
+    q = __fma_rn(__fma_rn(-q, S, x), y, q);
+    return __double2ull_rz(__dmul_rn(q, 0x1p40));
+}
+
 // Device state shared by the kernels of a run (the runs' states stand side by side; a
 // cache line each).
 struct alignas(128) DevState {
@@ -115,7 +128,8 @@ struct alignas(128) DevState {
     uint32_t sweeps;   // learned schedule: sweeps spent so far
     int32_t resample;  // partial resampling: this step resamples
     int32_t wexp;      // partial resampling: exponent of the largest new weight
-    double S_new;      // partial resampling: sum of the new weights
+    double S_new;      // sum of the level weights (partial resampling: of the new weights)
+    double S_inv;      // 1 / S_new
     uint32_t epoch;    // resampling steps taken (tags the look-back descriptors)
     int32_t kmax;      // a Poisson inversion of this step hit its limit
     int32_t hlo, hhi;  // lowest / highest histogram level filled since the last reweighting
@@ -235,6 +249,8 @@ struct KParams {
     int g3mul;                 // 3D: sets of groups per CTA, the side's count times this (1 or 2)
     WalkPlan wplan[4];
     int G2, TG2;               // 2D kernel (nw = 0): groups per CTA (0: the general kernel), threads of each
+    int pop;                   // k_pop: CTAs per run (0: the general kernels),
+    int pop_threads, pop_levels;  // their threads, entries of their level arrays
     const uint32_t* wmap[4];   // CTA -> run of each launch
     uint32_t wcta[4];
 };
@@ -254,6 +270,9 @@ namespace pa {
 cudaError_t launch_init_spins(const KParams& p, const RunDesc* host_runs, cudaStream_t s);
 cudaError_t launch_measure(const KParams& p, int threads, cudaStream_t s);
 cudaError_t launch_resample(const KParams& p, cudaStream_t s, int64_t* launches);
+int pop_ctas(uint32_t most_R, int most_levels, int M, int method, int* threads,
+             int* levels);
+cudaError_t launch_pop(const KParams& p, cudaStream_t s);
 cudaError_t launch_partial_init(const KParams& p, cudaStream_t s);
 cudaError_t launch_sweep(const KParams& p, int threads, cudaStream_t s);
 cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int64_t* launches);

@@ -1,0 +1,349 @@
+// pa_pop.cu -- the whole resampling of a small population in one launch: weights, ln Q,
+// copy numbers, ancestors and families (pa_resample.cu's kernels, same results bit for bit).
+//
+// A run is one thread-block cluster of 1 to 16 CTAs, each with POP_CHUNK replicas, two per
+// thread.  Every CTA computes the level weights for itself; block totals, the multinomial
+// searches and their counts go through the cluster's shared memory, so the look-backs, the
+// prefix arrays and the launches between the phases are gone.
+// What bounds it: latency, 16 to 20 thousand cycles (9 to 11 us) of short phases: three block
+// scans with a cluster barrier each 6, the level weights 5, the draws or the copy numbers 3 to
+// 6, the scatter 2, the variance's tree 1.5.  Temperature steps with ten sweeps: 2D L = 16,
+// R = 1000, multinomial (four kernels before) 57 -> 42 us; L = 64, R = 3000, systematic, with
+// the learned schedule 60 -> 53; +-J L = 48, R = 20001, Poisson 231 -> 219.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "pa_counts.cuh"
+
+namespace pa {
+
+namespace cg = cooperative_groups;
+
+constexpr int POP_CTAS = 16;
+static_assert(SCAN_CHUNK == 2 * SCAN_THREADS && SCAN_THREADS == 256, "two adjacent replicas per thread");
+
+template <int POP_THREADS>
+__global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
+    constexpr int POP_CHUNK = 2 * POP_THREADS;  // replicas of a CTA
+    cg::cluster_group cl = cg::this_cluster();
+    const unsigned cs = cl.num_blocks(), rank = cl.block_rank();
+    const auto sync = [&] {  // one CTA needs no cluster barrier (1000 cycles)
+        if (cs == 1) __syncthreads();
+        else cl.sync();
+    };
+    DevState* st = p.runs[blockIdx.x / cs].st;
+    if (st->status != S_OK) return;  // written by this cluster alone, after its last barrier
+    cl.barrier_arrive();  // waited for before the first access to another CTA's shared memory
+    extern __shared__ __align__(16) unsigned char dyn[];
+    double* ta = reinterpret_cast<double*>(dyn);  // level tree; later the variance terms
+    double* tb = ta + p.pop_levels;               // level weights, then fixed-point weights
+    __shared__ __align__(16) RunDesc r;           // the run's pointers, a load away
+    __shared__ uint32_t cnt[POP_CHUNK], so[POP_CHUNK], sfam[POP_CHUNK];
+    __shared__ uint64_t sh[33], xf[POP_CTAS], xg[POP_CTAS], xc[POP_CTAS];
+    __shared__ double qsq[32], S_sh, rS_sh;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    static_assert(sizeof(RunDesc) % 8 == 0 && sizeof(RunDesc) / 8 <= 256, "one word per thread");
+    if (t < (int)(sizeof(RunDesc) / 8))
+        reinterpret_cast<uint64_t*>(&r)[t] = reinterpret_cast<const uint64_t*>(p.runs + blockIdx.x / cs)[t];
+    const int i = st->step + 1, method = p.method;
+    const uint32_t Rprev = st->R_cur;
+    const int lmin = st->hlo, hi = st->hhi;
+    __syncthreads();
+    const int dN = p.d * r.N;
+    const int K = hi >= lmin ? hi - lmin + 1 : 0;
+    const uint32_t j0 = rank * POP_CHUNK + 2 * t;
+    const int32_t* E = r.E[(i - 1) & 1];
+    const uint32_t* fam0 = r.fam[(i - 1) & 1];
+    int32_t Ej[2];
+    uint32_t fj[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const bool in = j0 + e < Rprev;
+        Ej[e] = in ? E[j0 + e] : 0;
+        fj[e] = in ? fam0[j0 + e] : 0u;
+    }
+    // ---- level weights: S = sum_k n_k w_k by the fixed pairwise tree, f_k (k_weights) ----
+    if (t == 0) {
+        const int nb = max(5, K > 1 ? 32 - __clz(K - 1) : 0);
+        double b = r.sq[i - 1];
+        for (int m = 0; m < nb; ++m) {
+            qsq[m] = b;
+            b = __dmul_rn(b, b);
+        }
+    }
+    int P = 1;
+    while (P < K) P <<= 1;
+    const uint32_t n0 = t < K ? r.hist[lmin + t] : 0u;
+    __syncthreads();
+    double wlow = 1.0;  // the low five bits of k are the lane's: pow_tab's product so far
+    if (warp * 32 < K) {
+#pragma unroll
+        for (int m = 0; m < 5; ++m)
+            if ((lane >> m) & 1) wlow = __dmul_rn(wlow, qsq[m]);
+    }
+    for (int k = t; k < P; k += POP_THREADS) {
+        double v = 0.0;
+        if (k < K) {
+            double w = wlow;
+            for (uint32_t m = 5, hk = (uint32_t)k >> 5; hk; ++m, hk >>= 1)
+                if (hk & 1u) w = __dmul_rn(w, qsq[m]);
+            tb[k] = w;
+            v = __dmul_rn((double)(k == t ? n0 : r.hist[lmin + k]), w);
+        }
+        ta[k] = v;
+    }
+    __syncthreads();
+    int h = P >> 1;
+    for (; h >= 32; h >>= 1) {
+        for (int k = t; k < h; k += POP_THREADS) ta[k] = __dadd_rn(ta[k], ta[k + h]);
+        __syncthreads();
+    }
+    if (warp == 0) {
+        const int live = h > 0 ? 2 * h : 1;
+        double v = lane < live ? ta[lane] : 0.0;
+        for (; h >= 1; h >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, h));
+        if (lane == 0) {
+            S_sh = v;
+            rS_sh = __ddiv_rn(1.0, v);
+        }
+    }
+    __syncthreads();
+    const double S = S_sh;
+    const double Rd = (double)r.R, rS = rS_sh;
+    uint64_t* fl = reinterpret_cast<uint64_t*>(tb);
+    for (int k = t; k < K; k += POP_THREADS) fl[k] = fixed_quotient(__dmul_rn(Rd, tb[k]), S, rS);
+    __syncthreads();
+    // ---- expected copies, their prefix and total over the cluster ----
+    constexpr uint64_t FMASK = (1ull << FRAC_BITS) - 1;
+    uint64_t f[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) f[e] = j0 + e < Rprev ? fl[level_of(Ej[e], dN) - lmin] : 0ull;
+    uint64_t tf, tg = 0ull, eg = 0ull;
+    const uint64_t ef = block_excl_scan(f[0] + f[1], sh, &tf);
+    if (method == M_RESIDUAL) eg = block_excl_scan((f[0] & FMASK) + (f[1] & FMASK), sh, &tg);
+    cl.barrier_wait();
+    if (t < (int)cs) {
+        cl.map_shared_rank(xf, t)[rank] = tf;
+        cl.map_shared_rank(xg, t)[rank] = tg;
+    }
+    sync();
+    uint64_t T = 0ull, G = 0ull, pf = 0ull, pg = 0ull;
+    for (unsigned q = 0; q < cs; ++q) {
+        if (q == rank) {
+            pf = T;
+            pg = G;
+        }
+        T += xf[q];
+        G += xg[q];
+    }
+    // ---- copy numbers ----
+    uint32_t rc[2] = {0u, 0u};
+    bool kmax = false;
+    if (method == M_MULTINOMIAL || method == M_RESIDUAL) {
+        const bool residual = method == M_RESIDUAL, useg = residual && G > 0;
+        // every CTA gets the whole population's prefix, over its level arrays (read by now):
+        // a search in another CTA's memory takes 250 cycles a step
+        uint64_t* box = reinterpret_cast<uint64_t*>(dyn);
+        const uint32_t nbox = cs * POP_CHUNK, me = rank * POP_CHUNK + 2 * t;
+        uint64_t c[2];
+        c[0] = (useg ? pg + eg : pf + ef) + (useg ? f[0] & FMASK : f[0]);
+        c[1] = c[0] + (useg ? f[1] & FMASK : f[1]);
+        for (unsigned q = 0; q < cs; ++q) {
+            uint64_t* bx = q == rank ? box : cl.map_shared_rank(box, q);
+            *reinterpret_cast<ulonglong2*>(bx + me) = make_ulonglong2(c[0], c[1]);
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) cnt[2 * t + e] = residual ? (uint32_t)(f[e] >> FRAC_BITS) : 0u;
+        sync();
+        const uint64_t n = residual ? (uint64_t)r.R - ((T - G) >> FRAC_BITS) : (uint64_t)r.R;
+        const uint64_t total = useg ? G : T;
+        const uint32_t rule = residual ? RULE_RESIDUAL : RULE_MULTINOMIAL;
+        for (uint64_t k = 2 * (rank * POP_THREADS + t); k < n; k += 2 * cs * POP_THREADS) {
+            // two draws of one Philox block; the first replica whose prefix exceeds each (the
+            // prefix is flat past the last replica, and the draws lie below its end)
+            const uint4x x = draw_block(p, r, i, k, rule);
+            const uint64_t p0 = __umul64hi(((uint64_t)x.y << 32) | x.x, total);
+            const uint64_t p1 = __umul64hi(((uint64_t)x.w << 32) | x.z, total);
+            uint32_t l0 = 0, l1 = 0;
+            for (uint32_t w = nbox / 2; w >= 1; w >>= 1) {
+                if (box[l0 + w - 1] <= p0) l0 += w;
+                if (box[l1 + w - 1] <= p1) l1 += w;
+            }
+            const unsigned q0 = l0 / POP_CHUNK, q1 = l1 / POP_CHUNK;
+            atomicAdd((q0 == rank ? cnt : cl.map_shared_rank(cnt, q0)) + l0 % POP_CHUNK, 1u);
+            if (k + 1 < n)
+                atomicAdd((q1 == rank ? cnt : cl.map_shared_rank(cnt, q1)) + l1 % POP_CHUNK, 1u);
+        }
+        sync();
+        rc[0] = cnt[2 * t];
+        rc[1] = cnt[2 * t + 1];
+    } else {
+        uint32_t usys = 0u;
+        uint64_t below = 0ull, cf = pf + ef;
+        if (method == M_SYSTEMATIC) {
+            usys = systematic_offset(p, r, i);
+            below = sys_below(cf, r.R, T, usys);
+        }
+#pragma unroll 1
+        for (int e = 0; e < 2; ++e) {
+            const uint32_t j = j0 + e;
+            if (j >= Rprev) continue;
+            const uint64_t fe = e ? f[1] : f[0];
+            uint32_t c;
+            if (method == M_NEAREST) {
+                c = nearest_count(p, r, i, j, fe);
+            } else if (method == M_SYSTEMATIC) {
+                cf += fe;
+                const uint64_t bn = sys_below(cf, r.R, T, usys);
+                c = (uint32_t)(bn - below);
+                below = bn;
+            } else {
+                c = poisson_count(p, r, i, j, fe, kmax);
+            }
+            if (e) rc[1] = c;
+            else rc[0] = c;
+        }
+    }
+    // ---- first slot of every replica over the cluster ----
+    uint64_t tot;
+    const uint64_t ex = block_excl_scan((uint64_t)rc[0] + rc[1], sh, &tot);
+    const int km = __syncthreads_or(kmax);
+    if (t < (int)cs) cl.map_shared_rank(xc, t)[rank] = tot | (km ? 1ull << 63 : 0ull);
+    sync();
+    uint64_t Ri = 0ull, pre = 0ull;
+    bool anyk = false;
+    for (unsigned q = 0; q < cs; ++q) {
+        if (q == rank) pre = Ri;
+        Ri += xc[q] & ~(1ull << 63);
+        anyk |= (xc[q] >> 63) != 0;
+    }
+    // ---- ancestors and families (slots past the capacity are not written), the variance ----
+    uint32_t* fam1 = r.fam[i & 1];
+    const uint64_t room = pre < (uint64_t)r.Rcap ? (uint64_t)r.Rcap - pre : 0ull;
+    const uint32_t nslot = (uint32_t)(tot < room ? tot : room);
+    uint32_t o = (uint32_t)(ex < 0xFFFFFFFFull ? ex : 0xFFFFFFFFull);
+    double sv = 0.0;
+    int skew = 0;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        so[2 * t + e] = o;
+        sfam[2 * t + e] = fj[e];
+        o += rc[e];
+        skew |= rc[e] > 4u;
+        if (j0 + e >= Rprev) continue;
+        r.counts[j0 + e] = rc[e];
+        const double dl = count_excess(rc[e], f[e]);
+        sv = __dadd_rn(sv, __dmul_rn(dl, dl));
+    }
+    ta[t] = sv;
+    if (!__syncthreads_or(skew)) {  // as in k_resample: at most four copies each, or by slots
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (uint32_t c = 0; c < 4u; ++c) {
+                const uint32_t q = so[2 * t + e] + c;
+                if (c < rc[e] && q < nslot) {
+                    r.anc[pre + q] = j0 + e;
+                    fam1[pre + q] = fj[e];
+                }
+            }
+    } else {
+        for (uint32_t q = t; q < nslot; q += POP_THREADS) {
+            int lo = 0;
+#pragma unroll
+            for (int w = POP_CHUNK / 2; w >= 1; w >>= 1)
+                if (so[lo + w] <= q) lo += w;
+            r.anc[pre + q] = rank * POP_CHUNK + lo;
+            fam1[pre + q] = sfam[lo];
+        }
+    }
+    // the scan blocks' partials, each over its SCAN_THREADS threads in the same pairs
+    const int u = t & (SCAN_THREADS - 1);
+    for (int w = SCAN_THREADS / 2; w >= 32; w >>= 1) {
+        if (u < w) ta[t] = __dadd_rn(ta[t], ta[t + w]);
+        __syncthreads();
+    }
+    if (u < 32) {
+        double v = ta[t];
+        for (int w = 16; w >= 1; w >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, w));
+        const int b = (int)(rank * (POP_CHUNK / SCAN_CHUNK)) + t / SCAN_THREADS;
+        if (u == 0 && b < r.nblk) r.partD[b] = __dmul_rn(v, 0x1p-80);
+    }
+    // the run's state, which every CTA of the cluster has read; ln Q is left to the kernel
+    // that closes the step
+    if (rank == 0) {
+        for (int k = t; k < K; k += POP_THREADS) r.hist[lmin + k] = 0u;
+        if (t == POP_THREADS - 1) {
+            st->step = i;  // the step's other kernels read its index here
+            st->epoch += 1u;
+            st->S_new = S;
+            st->R_prev = Rprev;
+            st->lmin = (uint32_t)lmin;
+            st->K = (uint32_t)K;
+            st->hlo = 0x7FFFFFFF;  // the histogram is empty again
+            st->hhi = -1;
+            TraceRow* tr = r.trace + i;
+            tr->c_ln_c = 0.0;
+            tr->sv_sum = 0.0;
+            tr->sumE = tr->sumE2 = tr->sumAbsM = tr->sumM2 = tr->sumC2 = tr->accepts = 0ull;
+            tr->R_prev = Rprev;
+            tr->R_i = 0;
+            // a population that outgrows its capacity, or dies out, stops the run
+            st->kmax = anyk;
+            if (anyk) st->status = S_KMAX;
+            else if (Ri > (uint64_t)r.Rcap || Ri == 0) st->status = S_CAPACITY;
+            else st->R_cur = (uint32_t)Ri;
+        }
+    }
+}
+
+// CTAs per run (a power of two), or 0 where the general kernels take the batch.  The fewest
+// threads per CTA that hold the population in POP_CTAS CTAs: an SM's FP64 pipe and its
+// shared-memory banks are what the phases share (2D L = 16 / 32, one sweep, us per step with
+// 256, 512 and 1024 threads: multinomial R = 2000 29, 31, 33, R = 4000 31, 36, 41; systematic
+// R = 4000 23, 25, 27, R = 8000 26, 27, 30).  General kernels for more than 32768 replicas,
+// for the drawn rules beyond 512 threads (R = 30000: 61 general, 80 here; residual 59, 64;
+// systematic 48, 44; Poisson 51, 47; nearest 47, 42), for more levels than shared memory
+// holds and for more runs than fit at a time.
+int pop_ctas(uint32_t most_R, int most_levels, int M, int method, int* threads, int* levels) {
+    const int most = method == M_MULTINOMIAL || method == M_RESIDUAL ? 512 : 1024;
+    int nt = 256, cs = 1;
+    while (nt < most && (uint64_t)POP_CTAS * 2 * nt < most_R) nt <<= 1;
+    while ((uint64_t)cs * 2 * nt < most_R) cs <<= 1;
+    int P = 1024;
+    while (P < most_levels) P <<= 1;
+    if (most == 512) P = std::max(P, cs * nt);  // two words per level hold a prefix per replica
+    *threads = nt;
+    *levels = P;
+    return cs <= POP_CTAS && P <= 8192 && (int64_t)M * cs <= 128 ? cs : 0;
+}
+
+template <int NT>
+static cudaError_t launch(const KParams& p, cudaStream_t s) {
+    const size_t sm = 2 * sizeof(double) * (size_t)p.pop_levels;
+    cudaError_t e = cudaFuncSetAttribute(k_pop<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e == cudaSuccess && p.pop > 8)
+        e = cudaFuncSetAttribute(k_pop<NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)p.pop;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)(p.M * p.pop));
+    c.blockDim = dim3(NT);
+    c.dynamicSmemBytes = sm;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k_pop<NT>, p);
+}
+
+cudaError_t launch_pop(const KParams& p, cudaStream_t s) {
+    return p.pop_threads == 256   ? launch<256>(p, s)
+           : p.pop_threads == 512 ? launch<512>(p, s)
+                                  : launch<1024>(p, s);
+}
+
+}  // namespace pa

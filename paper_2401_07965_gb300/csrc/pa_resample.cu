@@ -23,137 +23,9 @@
 // six kernels: 2D L = 64, R = 10^4, 200 steps 52.9 -> 40.4 ms).
 #include <climits>
 
-#include "pa_internal.cuh"
+#include "pa_counts.cuh"
 
 namespace pa {
-
-// q^k by binary powering from a table of the squares qsq[m] = q^(2^m), each the
-// rounded square of the one before (qsq[0] = q): the product of the squares of
-// the set bits of k, least significant first, every multiply rounded -- the
-// same value as squaring and multiplying in one loop, with popc(k) multiplies
-// on the dependent chain.
-__device__ __forceinline__ double pow_tab(const double* qsq, uint32_t k) {
-    double r = 1.0;
-    for (int m = 0; k; ++m, k >>= 1)
-        if (k & 1u) r = __dmul_rn(r, qsq[m]);
-    return r;
-}
-
-// exp(x) = 2^n sum_{k<=13} r^k / k!, x = n ln2 + r (Cody-Waite reduction),
-// every operation explicitly rounded.  Used for the Poisson rule, x in [-16, 0].
-__device__ __forceinline__ double exp_taylor(double x) {
-    const double INV_LN2 = 0x1.71547652b82fep+0;
-    const double LN2_HI = 0x1.62e42fefa3800p-1;
-    const double LN2_LO = 0x1.ef35793c76730p-45;
-    const double c[14] = {0x1.0000000000000p+0,  0x1.0000000000000p+0,  0x1.0000000000000p-1,
-                          0x1.5555555555555p-3,  0x1.5555555555555p-5,  0x1.1111111111111p-7,
-                          0x1.6c16c16c16c17p-10, 0x1.a01a01a01a01ap-13, 0x1.a01a01a01a01ap-16,
-                          0x1.71de3a556c734p-19, 0x1.27e4fb7789f5cp-22, 0x1.ae64567f544e4p-26,
-                          0x1.1eed8eff8d898p-29, 0x1.6124613a86d09p-33};
-    const double nd = floor(__dadd_rn(__dmul_rn(x, INV_LN2), 0.5));
-    const double r = __dsub_rn(__dsub_rn(x, __dmul_rn(nd, LN2_HI)), __dmul_rn(nd, LN2_LO));
-    double pp = c[13];
-#pragma unroll
-    for (int k = 12; k >= 0; --k) pp = __dadd_rn(__dmul_rn(pp, r), c[k]);
-    return scalbn(pp, (int)nd);
-}
-
-// Poisson draw of mean lc in [0, 16] by sequential inversion of the CDF: the first k with
-// u < P_k, u = bits >> 11 in 2^-53 units, P_k summed in explicitly rounded FP64.  The search
-// runs in FP32 first: its P_k is within 1e-5 of the FP64 one (k <= 64: each term carries at
-// most 2 + 2k roundings of 2^-24, the terms sum to 1), so u farther than 2e-5 from every
-// P_k it passes decides alike; the others (about 1e-4 of the draws) repeat it in FP64, whose
-// operations occupy the pipe for 16 cycles per warp (k_resample, +-J L = 48, R = 20001:
-// 34 -> 27 us).
-__device__ __forceinline__ uint32_t poisson_draw(double lc, uint64_t bits, bool& kmax) {
-    {
-        const float l = (float)lc, u = (float)(uint32_t)(bits >> 40) * 0x1p-24f;
-        float pr = expf(-l), Pc = pr;
-        uint32_t k = 0;
-        while (u - Pc > 2e-5f && k < 64u) {
-            k += 1;
-            pr = __fdividef(pr * l, (float)k);
-            Pc += pr;
-        }
-        if (u - Pc < -2e-5f) return k;
-    }
-    const double u = scalbn((double)(bits >> 11), -53);
-    double pr = exp_taylor(-lc);
-    double Pc = pr;
-    uint32_t k = 0;
-    while (u >= Pc) {
-        k += 1;
-        if (k > POISSON_KMAX) {
-            kmax = true;
-            break;
-        }
-        pr = __ddiv_rn(__dmul_rn(pr, lc), (double)k);
-        Pc = __dadd_rn(Pc, pr);
-    }
-    return k;
-}
-
-struct U128 {
-    uint64_t hi, lo;
-};
-__device__ __forceinline__ U128 mul128(uint64_t a, uint64_t b) { return {__umul64hi(a, b), a * b}; }
-__device__ __forceinline__ bool lt128(U128 a, U128 b) {
-    return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo);
-}
-__device__ __forceinline__ bool le128(U128 a, U128 b) { return !lt128(b, a); }
-
-// Systematic rule: number of labels (k + u/2^32) T/R, k in [0,R), below x:
-// with xR = aT + b, that is a + [b 2^32 > u T], at most R.
-__device__ uint64_t sys_below(uint64_t x, uint64_t R, uint64_t T, uint32_t u) {
-    const U128 P = mul128(x, R);
-    // a = floor(xR / T) <= R < 2^24: an FP32 estimate is within a few units (FP64 is
-    // slow on this part), and the 128-bit corrections below make it exact
-    uint64_t a = (uint64_t)__fdiv_rn(__fmul_rn((float)x, (float)R), (float)T);
-    for (int it = 0; it < 8 && lt128(P, mul128(a, T)); ++it) --a;
-    for (int it = 0; it < 8 && le128(mul128(a + 1, T), P); ++it) ++a;
-    const uint64_t b = P.lo - a * T;  // < T, exact in the low 64 bits
-    const U128 lhs = {b >> 32, b << 32};
-    const U128 rhs = mul128((uint64_t)u, T);
-    const uint64_t n = a + (lt128(rhs, lhs) ? 1u : 0u);
-    return n < R ? n : R;
-}
-
-__device__ __forceinline__ int level_of(int32_t E, int dN) {
-    return ((E + dN) >> 1) >> 1;  // U = (E + dN)/2, level = U >> 1
-}
-
-// --------------------------------------------------------------------------
-// block helpers
-// --------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ T warp_incl_scan(T v, int lane) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        T n = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += n;
-    }
-    return v;
-}
-
-// exclusive block scan of one value per thread (blockDim == SCAN_THREADS)
-template <typename T>
-__device__ __forceinline__ T block_excl_scan(T v, T* sh, T* total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    T incl = warp_incl_scan(v, lane);
-    if (lane == 31) sh[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        T w = (lane < (int)(blockDim.x >> 5)) ? sh[lane] : (T)0;
-        T wi = warp_incl_scan(w, lane);
-        sh[lane] = wi - w;
-        if (lane == 31) sh[32] = wi;
-    }
-    __syncthreads();
-    T res = sh[warp] + incl - v;
-    *total = sh[32];
-    __syncthreads();
-    return res;
-}
 
 // balanced binary tree sums (adjacent pairs first) in explicitly rounded FP64:
 // over 8 or 16 consecutive values, and over the threads of a CTA (thread t =
@@ -226,9 +98,8 @@ __device__ __forceinline__ double max_threads(double v, double* sh, int n = 1024
 // K3: weights, S, ln Q, f table (one CTA)
 //
 // One CTA of 1024 threads; its time is latency, not work, so the phases are
-// kept few: the level counts are read from global memory once (into shared
-// memory, while the occupied range is found), the logarithms of ln Q run on a
-// warp that has no level of its own while the others compute f.
+// kept few: the level counts are read from global memory once, and the logarithms of
+// ln Q are left to the kernel that closes the step (finish_run).
 // --------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_weights(KParams p) {
     const RunDesc& r = p.runs[blockIdx.x];
@@ -241,11 +112,10 @@ __global__ void __launch_bounds__(1024) k_weights(KParams p) {
     double* tsm = tw;
     double* wsm = tw + TREE_SMEM;
     uint32_t* hc = reinterpret_cast<uint32_t*>(tw);
-    __shared__ double qsq[32], S_sh, lnS_sh, lnR_sh;
+    __shared__ double qsq[32], S_sh, rS_sh;
     const int i = st->step + 1;
     const uint32_t Rprev = st->R_cur;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nwarps = (int)(blockDim.x >> 5);
     // the occupied level range, recorded by the kernels that filled the histogram
     // (the lowest and highest level any replica took)
     const int lo = st->hlo, hi = st->hhi;
@@ -341,25 +211,19 @@ __global__ void __launch_bounds__(1024) k_weights(KParams p) {
         const volatile double* t = in_smem ? tsm : r.tree;
         double v = lane < live ? t[lane] : 0.0;
         for (; h >= 1; h >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, h));
-        if (lane == 0) S_sh = v;
+        if (lane == 0) {
+            S_sh = v;
+            rS_sh = __ddiv_rn(1.0, v);
+        }
     }
     __syncthreads();
     const double S = S_sh;
-    // ln S and ln R_{i-1} on the last warp (lanes 0 and 1, one pass), before its levels
-    if (warp == nwarps - 1) {
-        const double lx = log(lane == 0 ? S : (double)Rprev);
-        if (lane == 0) lnS_sh = lx;
-        if (lane == 1) lnR_sh = lx;
-    }
-    const double Rd = (double)r.R;
+    const double Rd = (double)r.R, rS = rS_sh;
     // f_k, and the totals T = sum_j f_j = sum_k n_k f_k and of the fractional parts
     // (exact integer sums; the copy-count kernels need them before any scan)
     unsigned long long sT = 0, sTr = 0;
     for (int k = threadIdx.x, j = 0; k < K; k += blockDim.x, ++j) {
-        double a = __dmul_rn(Rd, in_smem ? wsm[k] : pow_tab(qsq, (uint32_t)k));
-        a = __ddiv_rn(a, S);
-        a = scalbn(a, FRAC_BITS);
-        const uint64_t f = (uint64_t)floor(a);
+        const uint64_t f = fixed_quotient(__dmul_rn(Rd, in_smem ? wsm[k] : pow_tab(qsq, (uint32_t)k)), S, rS);
         r.flev[k] = f;
         const uint64_t n = in_smem ? (j == 0 ? n0 : n1) : r.hist[lmin + k];
         sT += n * f;
@@ -385,19 +249,13 @@ __global__ void __launch_bounds__(1024) k_weights(KParams p) {
         st->Rres = (uint64_t)r.R - ((tsum[0] - tsum[1]) >> FRAC_BITS);
         st->epoch += 1u;
         st->kmax = 0;
-        const int32_t Umin = 2 * lmin + r.parity;
-        const int32_t Emin = 2 * Umin - p.d * r.N;
-        const double lnQ = __dsub_rn(__dsub_rn(lnS_sh, lnR_sh),
-                                     __dmul_rn(r.sdbeta[i - 1], (double)Emin));
+        st->S_new = S;
         st->R_prev = Rprev;
         st->lmin = (uint32_t)lmin;
         st->K = (uint32_t)K;
         st->hlo = 0x7FFFFFFF;  // the histogram is empty again
         st->hhi = -1;
-        st->sum_lnQ = __dadd_rn(st->sum_lnQ, lnQ);
         TraceRow* tr = r.trace + i;
-        tr->lnQ = lnQ;
-        tr->sum_lnQ = st->sum_lnQ;
         tr->c_ln_c = 0.0;
         tr->sv_sum = 0.0;
         tr->sumE = tr->sumE2 = tr->sumAbsM = tr->sumM2 = tr->sumC2 = tr->accepts = 0ull;
@@ -493,6 +351,7 @@ __global__ void __launch_bounds__(1024) k_pw_final(KParams p) {
         st->resample = res;
         st->wexp = e;
         st->S_new = S[1];
+        st->S_inv = __ddiv_rn(1.0, S[1]);
         st->T = st->Tres = 0ull;  // summed by k_fsum
         st->epoch += 1u;
         st->kmax = 0;
@@ -524,16 +383,14 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_fsum(KParams p) {
     if (st->status != S_OK || !st->resample) return;  // the population is kept
     __shared__ unsigned long long tot[2];
     const uint32_t Rprev = st->R_prev;
+    const double S = st->S_new, rS = st->S_inv;
     const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
     unsigned long long sf = 0, sg = 0;
 #pragma unroll
     for (int e = 0; e < SCAN_ITEMS; ++e) {
         const int j = j0 + e;
         if ((uint32_t)j < Rprev) {
-            double a = __dmul_rn((double)r.R, r.w[j]);
-            a = __ddiv_rn(a, st->S_new);
-            a = scalbn(a, FRAC_BITS);
-            const uint64_t f = (uint64_t)floor(a);
+            const uint64_t f = fixed_quotient(__dmul_rn((double)r.R, r.w[j]), S, rS);
             r.C[j] = f;
             sf += f;
             sg += f & ((1ull << FRAC_BITS) - 1);
@@ -591,8 +448,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_draws(KParams p) {
     }
     const uint64_t stride = (uint64_t)r.nblk * SCAN_THREADS;
     for (uint64_t k = (uint64_t)b * SCAN_THREADS + threadIdx.x; k < n; k += stride) {
-        const uint4x x = philox((uint32_t)(k >> 1), DOM_RESAMPLE | (r.run << 8) | rule, (uint32_t)i,
-                                0u, p.k0, p.k1);
+        const uint4x x = draw_block(p, r, i, k, rule);
         const uint64_t u = (k & 1) ? (((uint64_t)x.w << 32) | x.z) : (((uint64_t)x.y << 32) | x.x);
         const uint64_t pos = __umul64hi(u, total);
         uint32_t lo = 0, hi = Rprev;
@@ -766,12 +622,19 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
     finish_run<PARTIAL>(p, r, st, mode, fa, fb, sd);
 }
 
-// fixed-order sums of the run's per-block partials, close the step (one CTA of
+// fixed-order sums of the run's per-block partials and ln Q (its logarithms cost 2000 cycles
+// each on this part: here they run beside the sweep), close the step (one CTA of
 // SCAN_THREADS threads; a, b, ws: shared arrays of SCAN_THREADS doubles)
 template <bool PARTIAL>
 __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int mode, double* a,
                            double* b, double* ws) {
     const int i = st->step;
+    __shared__ double lg[2];
+    if (!PARTIAL && mode == 0 && threadIdx.x >= SCAN_THREADS - 32) {  // beside the sums
+        const int lane = threadIdx.x & 31;
+        const double lx = log(lane == 0 ? st->S_new : (double)st->R_prev);
+        if (lane < 2) lg[lane] = lx;
+    }
     const int nb_sv = (mode == 0) ? (int)((st->R_prev + SCAN_CHUNK - 1) / SCAN_CHUNK) : 0;
     const int nb_f = (int)((st->R_cur + SCAN_CHUNK - 1) / SCAN_CHUNK);
     double sa = 0.0, sb = 0.0;
@@ -821,6 +684,16 @@ __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int
     }
     if (threadIdx.x == 0) {
         TraceRow* tr = r.trace + i;
+        if (!PARTIAL && mode == 0) {
+            const int32_t Umin = 2 * (int32_t)st->lmin + r.parity;
+            const int32_t Emin = 2 * Umin - p.d * r.N;
+            const double lnQ = __dsub_rn(__dsub_rn(lg[0], lg[1]),
+                                         __dmul_rn(r.sdbeta[i - 1], (double)Emin));
+            const double sum = __dadd_rn(st->sum_lnQ, lnQ);
+            st->sum_lnQ = sum;
+            tr->lnQ = lnQ;
+            tr->sum_lnQ = sum;
+        }
         tr->sv_sum = a[0];
         tr->c_ln_c = b[0];
         tr->R_i = st->R_cur;
@@ -974,8 +847,7 @@ __device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDe
         o += rc[e];
         skew |= rc[e] > 4u;
         if (!in) continue;
-        const double tau = scalbn((double)fv[e], -FRAC_BITS);
-        const double dl = __dsub_rn((double)rc[e], tau);
+        const double dl = count_excess(rc[e], fv[e]);
         sv = __dadd_rn(sv, __dmul_rn(dl, dl));
     }
     // Parents of at most four copies write their slots themselves; a block with a larger
@@ -1011,7 +883,7 @@ __device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDe
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        r.partD[b] = sd[0];
+        r.partD[b] = __dmul_rn(sd[0], 0x1p-80);
         if (b == r.nblk - 1) {
             const uint64_t Ri = pre + tot;
             // a population that outgrows its capacity, or dies out, stops the run
@@ -1085,9 +957,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
     }
     uint64_t cf = pre[0] + ef, cg = pre[1] + eg;
     const int method = p.method;
-    uint32_t usys = 0;
-    if (method == M_SYSTEMATIC)
-        usys = philox(0u, DOM_RESAMPLE | (r.run << 8) | RULE_SYSTEMATIC, (uint32_t)i, 0u, p.k0, p.k1).x;
+    const uint32_t usys = method == M_SYSTEMATIC ? systematic_offset(p, r, i) : 0u;
     bool kmax = false;
     uint32_t rc[SCAN_ITEMS];
     // systematic: labels below the running boundary, carried from item to item
@@ -1101,11 +971,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
         cg += f[e] & ((1ull << FRAC_BITS) - 1);
         uint32_t cnt = 0;
         if (method == M_NEAREST) {
-            const uint4x x = philox((uint32_t)j, DOM_RESAMPLE | (r.run << 8) | RULE_NEAREST, (uint32_t)i, 0u,
-                                    p.k0, p.k1);
-            const uint64_t u40 = (((uint64_t)x.y << 32) | x.x) >> 24;
-            cnt = (uint32_t)(f[e] >> FRAC_BITS) +
-                  (u40 < (f[e] & ((1ull << FRAC_BITS) - 1)) ? 1u : 0u);
+            cnt = nearest_count(p, r, i, (uint32_t)j, f[e]);
         } else if (method == M_SYSTEMATIC) {
             const uint64_t bn = sys_below(cf, r.R, T, usys);
             cnt = (uint32_t)(bn - below);
@@ -1116,19 +982,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
             cnt = (uint32_t)(f[e] >> FRAC_BITS);
         } else if (method == M_MULTINOMIAL) {
             r.C[j] = cf;
-        } else {  // Poisson
-            // sequential inversion per chunk of mean lc <= 16; poisson_draw decides in FP32
-            // where that is certain
-            const double lam = scalbn((double)f[e], -FRAC_BITS);
-            const uint32_t M = (uint32_t)(f[e] >> 44) + 1u;
-            const double lc = M == 1u ? lam : __ddiv_rn(lam, (double)M);
-            uint32_t total = 0;
-            for (uint32_t m = 0; m < M; ++m) {
-                const uint4x x = philox((uint32_t)j, DOM_RESAMPLE | (r.run << 8) | RULE_POISSON, (uint32_t)i, m,
-                                        p.k0, p.k1);
-                total += poisson_draw(lc, ((uint64_t)x.y << 32) | x.x, kmax);
-            }
-            cnt = total;
+        } else {
+            cnt = poisson_count(p, r, i, (uint32_t)j, f[e], kmax);
         }
         rc[e] = cnt;
         r.counts[j] = cnt;
@@ -1169,6 +1024,10 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_cscan(KParams p) {
 
 // --------------------------------------------------------------------------
 cudaError_t launch_resample(const KParams& p, cudaStream_t s, int64_t* launches) {
+    if (p.pop && p.alpha < 0.0 && !p.lb_hold) {
+        if (launches) *launches += 1;
+        return launch_pop(p, s);
+    }
     k_weights<<<p.M, 1024, 0, s>>>(p);
     int n = 1;
     if (p.alpha >= 0.0) {

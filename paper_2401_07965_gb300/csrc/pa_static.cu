@@ -51,7 +51,7 @@ k_static_weights(StaticScratch* sc, const int32_t* __restrict__ E, uint32_t R_pr
                  int d, int N, int parity, double dbeta, double q, double* lnQ_out,
                  uint64_t* f_out) {
     extern __shared__ __align__(16) uint32_t sh[];  // counts of the nlev levels; then the tree
-    __shared__ double qsq[32], S_sh, lnS_sh, lnR_sh;
+    __shared__ double qsq[32], S_sh, rS_sh, lnS_sh, lnR_sh;
     __shared__ int s_lo, s_hi, s_bad, s_last;
     const int nlev = d * N / 2 + 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -154,7 +154,10 @@ k_static_weights(StaticScratch* sc, const int32_t* __restrict__ E, uint32_t R_pr
         double v = 0.0;
         if (lane < live) v = tree_sh ? ts[lane] : tg[lane];
         for (; h >= 1; h >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, h));
-        if (lane == 0) S_sh = v;
+        if (lane == 0) {
+            S_sh = v;
+            rS_sh = __ddiv_rn(1.0, v);
+        }
     }
     __syncthreads();
     const double S = S_sh;
@@ -163,12 +166,9 @@ k_static_weights(StaticScratch* sc, const int32_t* __restrict__ E, uint32_t R_pr
         if (lane == 0) lnS_sh = lx;
         if (lane == 1) lnR_sh = lx;
     }
-    const double Rd = (double)R;
+    const double Rd = (double)R, rS = rS_sh;
     for (int k = threadIdx.x; k < K; k += STATIC_THREADS) {
-        double a = __dmul_rn(Rd, pow_sq(qsq, (uint32_t)k));
-        a = __ddiv_rn(a, S);
-        a = scalbn(a, pa::FRAC_BITS);
-        sc->flev[k] = (uint64_t)floor(a);
+        sc->flev[k] = pa::fixed_quotient(__dmul_rn(Rd, pow_sq(qsq, (uint32_t)k)), S, rS);
     }
     __threadfence_block();
     __syncthreads();
