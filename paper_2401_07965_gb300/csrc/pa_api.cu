@@ -222,7 +222,7 @@ Layout make_layout(const std::vector<RunHost>& runs, int n_steps) {
         rs[R_OP] = (size_t)h.nblk * 5 * 8;
         rs[R_TRACE] = (size_t)(n_steps + 1) * sizeof(TraceRow);
         rs[R_LB1] = rs[R_LB2] = (size_t)h.nblk * sizeof(LBDesc);
-        rs[R_TICK] = 2 * sizeof(uint32_t);
+        rs[R_TICK] = 3 * sizeof(uint32_t);
         // the run's own step tables (used under the learned schedule)
         rs[R_SB] = (size_t)(n_steps + 1) * 8;
         rs[R_SDB] = rs[R_SQ] = (size_t)n_steps * 8;
@@ -326,7 +326,7 @@ pa_status map_dev_status(int s) {
 cudaError_t clear_lookback(const RunDesc& r, const RunHost& h, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(r.lb1, 0, (size_t)h.nblk * sizeof(LBDesc), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(r.lb2, 0, (size_t)h.nblk * sizeof(LBDesc), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r.tick, 0, 2 * sizeof(uint32_t), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(r.tick, 0, 3 * sizeof(uint32_t), s);
     return e;
 }
 
@@ -334,6 +334,8 @@ pa_status enqueue_measure(pa_ctx* ctx) {
     PA_CUDA(launch_measure(ctx->kp, ctx->threads, ctx->stream));
     ctx->launches += 1;
     PA_CUDA(launch_family_finish(ctx->kp, 1, ctx->stream, &ctx->launches));
+    if (ctx->kp.alpha >= 0.0)
+        PA_CUDA(launch_weighted_sums(ctx->kp, 1, ctx->stream, &ctx->launches));
     return PA_OK;
 }
 
@@ -462,16 +464,13 @@ pa_status grow_event_pool(pa_ctx* ctx, size_t n) {
 // weighted sums of the sweep's energies and follow it.
 pa_status enqueue_step(pa_ctx* ctx, int64_t* launches, cudaStream_t stream,
                        cudaStream_t side) {
-    const bool partial = ctx->kp.alpha >= 0.0;
     PA_CUDA(launch_resample(ctx->kp, stream, launches));
-    if (!partial) {
-        if (side) {
-            PA_CUDA(cudaEventRecord(ctx->ev_fork, stream));
-            PA_CUDA(cudaStreamWaitEvent(side, ctx->ev_fork, 0));
-        }
-        PA_CUDA(launch_family_finish(ctx->kp, 0, side ? side : stream, launches));
-        if (side) PA_CUDA(cudaEventRecord(ctx->ev_join, side));
+    if (side) {
+        PA_CUDA(cudaEventRecord(ctx->ev_fork, stream));
+        PA_CUDA(cudaStreamWaitEvent(side, ctx->ev_fork, 0));
     }
+    PA_CUDA(launch_family_finish(ctx->kp, 0, side ? side : stream, launches));
+    if (side) PA_CUDA(cudaEventRecord(ctx->ev_join, side));
     const bool timed = ctx->timing && !side;
     if (timed) {
         if (ctx->ev_used == ctx->ev_start.size()) {
@@ -483,8 +482,8 @@ pa_status enqueue_step(pa_ctx* ctx, int64_t* launches, cudaStream_t stream,
     PA_CUDA(launch_sweep(ctx->kp, ctx->threads, stream));
     if (launches) *launches += 1;
     if (timed) PA_CUDA(cudaEventRecord(ctx->ev_stop[ctx->ev_used++], stream));
-    if (partial) PA_CUDA(launch_family_finish(ctx->kp, 0, stream, launches));
-    else if (side) PA_CUDA(cudaStreamWaitEvent(stream, ctx->ev_join, 0));
+    if (ctx->kp.alpha >= 0.0) PA_CUDA(launch_weighted_sums(ctx->kp, 0, stream, launches));
+    if (side) PA_CUDA(cudaStreamWaitEvent(stream, ctx->ev_join, 0));
     if (ctx->kp.ctl) {
         PA_CUDA(launch_control(ctx->kp, stream));
         if (launches) *launches += 1;

@@ -34,13 +34,13 @@ __device__ __forceinline__ float bf_round(float v) {
 // now run beside the sweep and the decision has to wait for both (learned schedule, L = 64,
 // R = 3000: 24.6 -> 22.5 ms for 240 steps).
 // --------------------------------------------------------------------------
-__global__ void __launch_bounds__(64) k_control(KParams p) {
+__global__ void __launch_bounds__(32 * MLP_IN) k_control(KParams p) {
     const RunDesc& r = p.runs[blockIdx.x];  // one CTA per run of the batch
     control_after_step(p, r, r.st);
 }
 
 cudaError_t launch_control(const KParams& p, cudaStream_t s) {
-    k_control<<<p.M, 64, 0, s>>>(p);
+    k_control<<<p.M, 32 * MLP_IN, 0, s>>>(p);
     return cudaGetLastError();
 }
 

@@ -27,12 +27,12 @@ __device__ __forceinline__ float bf(uint16_t v) {
 // --------------------------------------------------------------------------
 // controller step
 //
-// Called by every thread of one CTA of at least 64 threads per run (threads
-// 0-63 work, the others only take part in the barriers).  Its time is latency:
+// Called by every thread of one CTA of at least 256 threads per run (threads 0-63 work,
+// and the first lane of each of eight warps; the others only take part in the barriers).  Its time is latency:
 // a dependent FP64 operation costs tens of cycles on this part and a logarithm
 // about 2000, so the work is spread and the chains kept short.  Each weight
 // row is loaded into the registers of the thread that uses it at entry; the
-// features are formed by threads 0-7 at once, with products by 1/R_i in place
+// features are formed by eight warps at once, with products by 1/R_i in place
 // of divisions and ln R_i from the host's ln R (equal to the direct formulas to
 // an FP64 rounding or two, below the FP32 rounding of the features); the
 // step-table entries of every admissible step size are prefetched while the
@@ -86,40 +86,42 @@ __device__ __forceinline__ void control_after_step(const KParams& p, const RunDe
     const float b1 = bf(w[OFF_B1 + t]), b2 = bf(w[OFF_B2 + t]);
     const float b3 = t < MLP_OUT ? bf(w[OFF_B3 + t]) : 0.0f;
 
-    // features (R22), one per thread (threads 0-7).  The FP64 divisions and
+    // features (R22), one per warp (eight lanes of one warp took their branches one after
+    // the other: 11 -> 6.7 us from cold caches).  The FP64 divisions and
     // logarithms of this part have long dependent chains (a logarithm takes about
     // 2000 cycles), so each thread's chain is kept short: 1/R_i once, products
     // after it, and ln R_i = ln R + log1p((R_i - R) / R) from the host's ln R
     // (R_i = R for the fixed-size rules) with the small correction in FP32.
-    if (act && t < MLP_IN) {
+    if ((threadIdx.x & 31u) == 0u && threadIdx.x < 32u * MLP_IN) {
+        const int f = (int)(threadIdx.x >> 5);
         const double Ri = (double)tr->R_i, N = (double)r.N;
         const double invR = 1.0 / Ri;
         float v;
-        if (t == 0) {
+        if (f == 0) {
             v = (float)r.sbeta[i];
-        } else if (t == 1 || t == 2) {
+        } else if (f == 1 || f == 2) {
             const double mE = (double)(long long)tr->sumE * invR;
-            if (t == 1) {
+            if (f == 1) {
                 v = (float)(mE / N);
             } else {
                 const double var = ((double)(long long)tr->sumE2 * invR - mE * mE) / N;
                 v = (float)(var * 0.1);
             }
-        } else if (t == 3) {
+        } else if (f == 3) {
             v = (float)(tr->lnQ / N * 10.0);
-        } else if (t == 4) {
+        } else if (f == 4) {
             v = (float)((double)(long long)tr->sumC2 * invR * invR);
-        } else if (t == 5) {
+        } else if (f == 5) {
             const float dR = __fdiv_rn((float)((long long)tr->R_i - (long long)r.R), (float)r.R);
             const double lnRi = r.lnR + (double)log1pf(dR);
             v = (float)((lnRi - tr->c_ln_c * invR) / r.lnR);
-        } else if (t == 6) {
+        } else if (f == 6) {
             const double th = i > 0 ? (double)r.stheta[i - 1] : 0.0;
             v = th > 0 ? (float)((double)tr->accepts * invR / (th * N)) : 0.0f;
         } else {
             v = (float)r.L / 64.0f;
         }
-        x[t] = v;
+        x[f] = v;
     }
     // the step tables of the admissible next steps u = 1 .. CTL_UMAX (k + u <= K)
     if (act && t >= 16 && t < 16 + CTL_UMAX) {

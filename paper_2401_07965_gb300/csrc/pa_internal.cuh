@@ -130,6 +130,7 @@ struct alignas(128) DevState {
     int32_t wexp;      // partial resampling: exponent of the largest new weight
     double S_new;      // sum of the level weights (partial resampling: of the new weights)
     double S_inv;      // 1 / S_new
+    double S_old;      // sum of the weights before the step (the population size, mostly)
     uint32_t epoch;    // resampling steps taken (tags the look-back descriptors)
     int32_t kmax;      // a Poisson inversion of this step hit its limit
     int32_t hlo, hhi;  // lowest / highest histogram level filled since the last reweighting
@@ -205,7 +206,7 @@ struct RunDesc {
     uint32_t* stheta;
     LBDesc* lb1;             // look-back descriptors: prefix of the expected copies
     LBDesc* lb2;             // and of the copy numbers
-    uint32_t* tick;          // [0] scan-block tickets, [1] family-block tickets
+    uint32_t* tick;          // tickets of the scan blocks [0], family blocks [1], k_wsums blocks [2]
 };
 
 // Geometry of a launch of the column-walk sweep kernel (one side L).
@@ -273,6 +274,8 @@ cudaError_t launch_resample(const KParams& p, cudaStream_t s, int64_t* launches)
 int pop_ctas(uint32_t most_R, int most_levels, int M, int method, int* threads,
              int* levels);
 cudaError_t launch_pop(const KParams& p, cudaStream_t s);
+inline bool pop_takes(const KParams& p) { return p.pop && !p.lb_hold; }
+cudaError_t launch_weighted_sums(const KParams& p, int mode, cudaStream_t s, int64_t* launches);
 cudaError_t launch_partial_init(const KParams& p, cudaStream_t s);
 cudaError_t launch_sweep(const KParams& p, int threads, cudaStream_t s);
 cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int64_t* launches);

@@ -1,5 +1,5 @@
-// pa_pop.cu -- the whole resampling of a small population in one launch: weights, ln Q,
-// copy numbers, ancestors and families (pa_resample.cu's kernels, same results bit for bit).
+// pa_pop.cu -- the whole resampling of a small population in one launch: weights, copy numbers,
+// (partial resampling: effective size and decision), ancestors and families (pa_resample.cu's kernels, same results bit for bit).
 //
 // A run is one thread-block cluster of 1 to 16 CTAs, each with POP_CHUNK replicas, two per
 // thread.  Every CTA computes the level weights for itself; block totals, the multinomial
@@ -9,7 +9,9 @@
 // scans with a cluster barrier each 6, the level weights 5, the draws or the copy numbers 3 to
 // 6, the scatter 2, the variance's tree 1.5.  Temperature steps with ten sweeps: 2D L = 16,
 // R = 1000, multinomial (four kernels before) 57 -> 42 us; L = 64, R = 3000, systematic, with
-// the learned schedule 60 -> 53; +-J L = 48, R = 20001, Poisson 231 -> 219.
+// the learned schedule 60 -> 53; +-J L = 48, R = 20001, Poisson 231 -> 219; L = 64,
+// R = 10^4, systematic, partial resampling (seven kernels, the family statistics after the
+// sweep) 202 -> 185.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -23,7 +25,29 @@ namespace cg = cooperative_groups;
 constexpr int POP_CTAS = 16;
 static_assert(SCAN_CHUNK == 2 * SCAN_THREADS && SCAN_THREADS == 256, "two adjacent replicas per thread");
 
-template <int POP_THREADS>
+// the run's state and trace row after its weights (threads t < n of one CTA)
+__device__ __forceinline__ void close_step(const RunDesc& r, DevState* st, int i, uint32_t Rprev,
+                                           int lmin, int K, double S, double S_old, int t, int n) {
+    for (int k = t; k < K; k += n) r.hist[lmin + k] = 0u;
+    if (t != n - 1) return;
+    st->step = i;  // the step's other kernels read its index here
+    st->epoch += 1u;
+    st->S_new = S;
+    st->S_old = S_old;
+    st->R_prev = Rprev;
+    st->lmin = (uint32_t)lmin;
+    st->K = (uint32_t)K;
+    st->hlo = 0x7FFFFFFF;  // the histogram is empty again
+    st->hhi = -1;
+    TraceRow* tr = r.trace + i;
+    tr->c_ln_c = 0.0;
+    tr->sv_sum = 0.0;
+    tr->sumE = tr->sumE2 = tr->sumAbsM = tr->sumM2 = tr->sumC2 = tr->accepts = 0ull;
+    tr->R_prev = Rprev;
+    tr->R_i = 0;
+}
+
+template <int POP_THREADS, bool PARTIAL>
 __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
     constexpr int POP_CHUNK = 2 * POP_THREADS;  // replicas of a CTA
     cg::cluster_group cl = cg::this_cluster();
@@ -42,6 +66,9 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
     __shared__ uint32_t cnt[POP_CHUNK], so[POP_CHUNK], sfam[POP_CHUNK];
     __shared__ uint64_t sh[33], xf[POP_CTAS], xg[POP_CTAS], xc[POP_CTAS];
     __shared__ double qsq[32], S_sh, rS_sh;
+    __shared__ double pw[PARTIAL ? 3 : 1][33], xw[PARTIAL ? 3 : 1][POP_CTAS * 4];
+    __shared__ unsigned long long pm[32], xm[POP_CTAS];
+    __shared__ int wexp_sh;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     static_assert(sizeof(RunDesc) % 8 == 0 && sizeof(RunDesc) / 8 <= 256, "one word per thread");
     if (t < (int)(sizeof(RunDesc) / 8))
@@ -74,7 +101,12 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
     }
     int P = 1;
     while (P < K) P <<= 1;
-    const uint32_t n0 = t < K ? r.hist[lmin + t] : 0u;
+    const uint32_t n0 = !PARTIAL && t < K ? r.hist[lmin + t] : 0u;
+    double wj[2];
+    if (PARTIAL) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) wj[e] = j0 + e < Rprev ? r.w[j0 + e] : 0.0;
+    }
     __syncthreads();
     double wlow = 1.0;  // the low five bits of k are the lane's: pow_tab's product so far
     if (warp * 32 < K) {
@@ -89,40 +121,144 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
             for (uint32_t m = 5, hk = (uint32_t)k >> 5; hk; ++m, hk >>= 1)
                 if (hk & 1u) w = __dmul_rn(w, qsq[m]);
             tb[k] = w;
-            v = __dmul_rn((double)(k == t ? n0 : r.hist[lmin + k]), w);
+            if (!PARTIAL) v = __dmul_rn((double)(k == t ? n0 : r.hist[lmin + k]), w);
         }
-        ta[k] = v;
+        if (!PARTIAL) ta[k] = v;
     }
     __syncthreads();
-    int h = P >> 1;
-    for (; h >= 32; h >>= 1) {
-        for (int k = t; k < h; k += POP_THREADS) ta[k] = __dadd_rn(ta[k], ta[k + h]);
-        __syncthreads();
-    }
-    if (warp == 0) {
-        const int live = h > 0 ? 2 * h : 1;
-        double v = lane < live ? ta[lane] : 0.0;
-        for (; h >= 1; h >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, h));
+    double S, S_old = (double)Rprev;
+    uint64_t f[2];
+    if constexpr (PARTIAL) {
+        // ---- new weights, their tree sums (blocks of SCAN_CHUNK, then the blocks: k_pw_update
+        // and k_pw_final), effective size, decision ----
+        double wn[2], v[3], mx;
+        {
+            double wo[2], w2[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool in = j0 + e < Rprev;
+                wo[e] = in ? wj[e] : 0.0;
+                wn[e] = in ? __dmul_rn(wo[e], tb[level_of(Ej[e], dN) - lmin]) : 0.0;
+                w2[e] = __dmul_rn(wn[e], wn[e]);
+            }
+            v[0] = __dadd_rn(wo[0], wo[1]);
+            v[1] = __dadd_rn(wn[0], wn[1]);
+            v[2] = __dadd_rn(w2[0], w2[1]);
+            mx = fmax(wn[0], wn[1]);
+        }
+#pragma unroll
+        for (int w = 1; w < 32; w <<= 1) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v[q] = __dadd_rn(v[q], __shfl_down_sync(0xffffffffu, v[q], w));
+        }
+        // the bit patterns of non-negative doubles are ordered like the values
+        unsigned long long um = (unsigned long long)__double_as_longlong(mx);
+        for (int w = 16; w >= 1; w >>= 1) {
+            const unsigned long long o = __shfl_xor_sync(0xffffffffu, um, w);
+            um = o > um ? o : um;
+        }
         if (lane == 0) {
-            S_sh = v;
-            rS_sh = __ddiv_rn(1.0, v);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) pw[q][warp] = v[q];
+            pm[warp] = um;
         }
+        __syncthreads();
+        cl.barrier_wait();
+        constexpr int NW = POP_THREADS / 32, BW = SCAN_THREADS / 32;
+        if (warp < 3) {  // the blocks' roots, to every CTA
+            double u = lane < NW ? pw[warp][lane] : 0.0;
+            for (int w = 1; w < BW; w <<= 1) u = __dadd_rn(u, __shfl_down_sync(0xffffffffu, u, w));
+            if (lane < NW && lane % BW == 0)
+                for (unsigned q = 0; q < cs; ++q)
+                    cl.map_shared_rank(&xw[warp][0], q)[rank * (NW / BW) + lane / BW] = u;
+        } else if (warp == 3) {
+            unsigned long long u = lane < NW ? pm[lane] : 0ull;
+            for (int w = 16; w >= 1; w >>= 1) {
+                const unsigned long long o = __shfl_xor_sync(0xffffffffu, u, w);
+                u = o > u ? o : u;
+            }
+            if (lane < (int)cs) cl.map_shared_rank(xm, lane)[rank] = u;
+        }
+        sync();
+        if (warp < 3) {  // up to 64 blocks, the rest of the tree's leaves are zeros
+            const int nb = (int)cs * (NW / BW);
+            double u = __dadd_rn(2 * lane < nb ? xw[warp][2 * lane] : 0.0,
+                                 2 * lane + 1 < nb ? xw[warp][2 * lane + 1] : 0.0);
+            for (int w = 1; w < 32; w <<= 1) u = __dadd_rn(u, __shfl_down_sync(0xffffffffu, u, w));
+            if (lane == 0) {
+                pw[warp][0] = u;
+                if (warp == 1) rS_sh = __ddiv_rn(1.0, u);
+            }
+        } else if (warp == 3) {
+            unsigned long long u = lane < (int)cs ? xm[lane] : 0ull;
+            for (int w = 16; w >= 1; w >>= 1) {
+                const unsigned long long o = __shfl_xor_sync(0xffffffffu, u, w);
+                u = o > u ? o : u;
+            }
+            int e = 0;
+            frexp(__longlong_as_double((long long)u), &e);
+            if (lane == 0) wexp_sh = e;
+        }
+        __syncthreads();
+        S_old = pw[0][0];
+        S = pw[1][0];
+        const double ess = __ddiv_rn(__dmul_rn(S, S), pw[2][0]);
+        const bool res = ess < __dmul_rn(p.alpha, (double)Rprev);
+        if (rank == 0 && t == 0) {
+            st->resample = res;
+            st->wexp = wexp_sh;
+            r.trace[i].ess = ess;
+            r.trace[i].resampled = res;
+        }
+        if (!res) {  // every replica is kept once, with its weight rescaled by a power of two
+            const int we = wexp_sh;
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                if (j0 + e < Rprev) {
+                    r.w[j0 + e] = scalbn(wn[e], -we);
+                    r.counts[j0 + e] = 1u;
+                    r.anc[j0 + e] = j0 + e;
+                    r.fam[i & 1][j0 + e] = fj[e];
+                }
+            const int b = (int)(rank * (POP_CHUNK / SCAN_CHUNK)) + t / SCAN_THREADS;
+            if (t % SCAN_THREADS == 0 && b < r.nblk) r.partD[b] = 0.0;
+            if (rank == 0) close_step(r, st, i, Rprev, lmin, K, S, S_old, t, POP_THREADS);
+            return;
+        }
+        const double rS = rS_sh;
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            f[e] = j0 + e < Rprev ? fixed_quotient(__dmul_rn((double)r.R, wn[e]), S, rS) : 0ull;
+    } else {
+        int h = P >> 1;
+        for (; h >= 32; h >>= 1) {
+            for (int k = t; k < h; k += POP_THREADS) ta[k] = __dadd_rn(ta[k], ta[k + h]);
+            __syncthreads();
+        }
+        if (warp == 0) {
+            const int live = h > 0 ? 2 * h : 1;
+            double v = lane < live ? ta[lane] : 0.0;
+            for (; h >= 1; h >>= 1) v = __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, h));
+            if (lane == 0) {
+                S_sh = v;
+                rS_sh = __ddiv_rn(1.0, v);
+            }
+        }
+        __syncthreads();
+        S = S_sh;
+        const double Rd = (double)r.R, rS = rS_sh;
+        uint64_t* fl = reinterpret_cast<uint64_t*>(tb);
+        for (int k = t; k < K; k += POP_THREADS) fl[k] = fixed_quotient(__dmul_rn(Rd, tb[k]), S, rS);
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < 2; ++e) f[e] = j0 + e < Rprev ? fl[level_of(Ej[e], dN) - lmin] : 0ull;
     }
-    __syncthreads();
-    const double S = S_sh;
-    const double Rd = (double)r.R, rS = rS_sh;
-    uint64_t* fl = reinterpret_cast<uint64_t*>(tb);
-    for (int k = t; k < K; k += POP_THREADS) fl[k] = fixed_quotient(__dmul_rn(Rd, tb[k]), S, rS);
-    __syncthreads();
     // ---- expected copies, their prefix and total over the cluster ----
     constexpr uint64_t FMASK = (1ull << FRAC_BITS) - 1;
-    uint64_t f[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) f[e] = j0 + e < Rprev ? fl[level_of(Ej[e], dN) - lmin] : 0ull;
     uint64_t tf, tg = 0ull, eg = 0ull;
     const uint64_t ef = block_excl_scan(f[0] + f[1], sh, &tf);
     if (method == M_RESIDUAL) eg = block_excl_scan((f[0] & FMASK) + (f[1] & FMASK), sh, &tg);
-    cl.barrier_wait();
+    if (!PARTIAL) cl.barrier_wait();
     if (t < (int)cs) {
         cl.map_shared_rank(xf, t)[rank] = tf;
         cl.map_shared_rank(xg, t)[rank] = tg;
@@ -246,6 +382,7 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
                 if (c < rc[e] && q < nslot) {
                     r.anc[pre + q] = j0 + e;
                     fam1[pre + q] = fj[e];
+                    if (PARTIAL) r.w[pre + q] = 1.0;
                 }
             }
     } else {
@@ -256,6 +393,7 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
                 if (so[lo + w] <= q) lo += w;
             r.anc[pre + q] = rank * POP_CHUNK + lo;
             fam1[pre + q] = sfam[lo];
+            if (PARTIAL) r.w[pre + q] = 1.0;
         }
     }
     // the scan blocks' partials, each over its SCAN_THREADS threads in the same pairs
@@ -273,22 +411,8 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
     // the run's state, which every CTA of the cluster has read; ln Q is left to the kernel
     // that closes the step
     if (rank == 0) {
-        for (int k = t; k < K; k += POP_THREADS) r.hist[lmin + k] = 0u;
+        close_step(r, st, i, Rprev, lmin, K, S, S_old, t, POP_THREADS);
         if (t == POP_THREADS - 1) {
-            st->step = i;  // the step's other kernels read its index here
-            st->epoch += 1u;
-            st->S_new = S;
-            st->R_prev = Rprev;
-            st->lmin = (uint32_t)lmin;
-            st->K = (uint32_t)K;
-            st->hlo = 0x7FFFFFFF;  // the histogram is empty again
-            st->hhi = -1;
-            TraceRow* tr = r.trace + i;
-            tr->c_ln_c = 0.0;
-            tr->sv_sum = 0.0;
-            tr->sumE = tr->sumE2 = tr->sumAbsM = tr->sumM2 = tr->sumC2 = tr->accepts = 0ull;
-            tr->R_prev = Rprev;
-            tr->R_i = 0;
             // a population that outgrows its capacity, or dies out, stops the run
             st->kmax = anyk;
             if (anyk) st->status = S_KMAX;
@@ -319,12 +443,12 @@ int pop_ctas(uint32_t most_R, int most_levels, int M, int method, int* threads, 
     return cs <= POP_CTAS && P <= 8192 && (int64_t)M * cs <= 128 ? cs : 0;
 }
 
-template <int NT>
+template <int NT, bool PARTIAL>
 static cudaError_t launch(const KParams& p, cudaStream_t s) {
     const size_t sm = 2 * sizeof(double) * (size_t)p.pop_levels;
-    cudaError_t e = cudaFuncSetAttribute(k_pop<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute(k_pop<NT, PARTIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e == cudaSuccess && p.pop > 8)
-        e = cudaFuncSetAttribute(k_pop<NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        e = cudaFuncSetAttribute(k_pop<NT, PARTIAL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
@@ -337,13 +461,18 @@ static cudaError_t launch(const KParams& p, cudaStream_t s) {
     c.stream = s;
     c.attrs = &at;
     c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, k_pop<NT>, p);
+    return cudaLaunchKernelEx(&c, k_pop<NT, PARTIAL>, p);
+}
+
+template <bool PARTIAL>
+static cudaError_t launch(const KParams& p, cudaStream_t s) {
+    return p.pop_threads == 256   ? launch<256, PARTIAL>(p, s)
+           : p.pop_threads == 512 ? launch<512, PARTIAL>(p, s)
+                                  : launch<1024, PARTIAL>(p, s);
 }
 
 cudaError_t launch_pop(const KParams& p, cudaStream_t s) {
-    return p.pop_threads == 256   ? launch<256>(p, s)
-           : p.pop_threads == 512 ? launch<512>(p, s)
-                                  : launch<1024>(p, s);
+    return p.alpha >= 0.0 ? launch<true>(p, s) : launch<false>(p, s);
 }
 
 }  // namespace pa

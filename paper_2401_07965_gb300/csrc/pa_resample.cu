@@ -10,7 +10,8 @@
 //   S = fixed pairwise tree sum of n_k w_k over a power-of-two array,
 //   ln Q = (ln S - ln R_{i-1}) - dbeta E_min,
 //   f_k = floor(2^40 * ((R w_k) / S))  (tau-hat of Eq. taus in 2^-40 units).
-// The copy counts are exact integer functions of f and of Philox draws.
+// The copy counts are exact integer functions of f and of Philox draws.  Small populations
+// take one kernel for all of it (pa_pop.cu); the kernels here take the others.
 //
 // Partial resampling (alpha >= 0): replicas carry weights w_j.  The step
 // multiplies them by the level factors q^(l_j - l_min) (k_pw_update), sums
@@ -18,7 +19,7 @@
 // replica index (blocks of SCAN_CHUNK aligned replicas, then the blocks:
 // k_pw_final), and resamples with f_j = floor(2^40 (R wn_j) / S_new) only if
 // (sum wn)^2 / sum wn^2 < alpha R_{i-1}; otherwise every replica is kept once
-// and its weight is rescaled by a power of two (k_family).  The f_j and their total come
+// and its weight is rescaled by a power of two (k_wsums).  The f_j and their total come
 // from k_fsum, the rest from the kernels of the plain step (its look-back scans replaced
 // six kernels: 2D L = 64, R = 10^4, 200 steps 52.9 -> 40.4 ms).
 #include <climits>
@@ -250,6 +251,7 @@ __global__ void __launch_bounds__(1024) k_weights(KParams p) {
         st->epoch += 1u;
         st->kmax = 0;
         st->S_new = S;
+        st->S_old = (double)Rprev;
         st->R_prev = Rprev;
         st->lmin = (uint32_t)lmin;
         st->K = (uint32_t)K;
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(1024) k_pw_final(KParams p) {
     const RunDesc& r = p.runs[blockIdx.x];
     DevState* st = r.st;
     if (st->status != S_OK) return;
-    __shared__ double sh[3 * 33], lg[2];
+    __shared__ double sh[3 * 33];
     const int i = st->step;
     const int nb = r.nblk;  // <= PARTIAL_MAX_BLOCKS = LEAVES leaves x 1024 threads
     constexpr int LEAVES = PARTIAL_MAX_BLOCKS / 1024;
@@ -336,29 +338,21 @@ __global__ void __launch_bounds__(1024) k_pw_final(KParams p) {
     for (int bb = threadIdx.x; bb < nb; bb += blockDim.x) mx = fmax(mx, r.wpart[4 * bb + 3]);
     tree_threads(S, sh, nb <= 1024 ? nb : 1024);
     mx = max_threads(mx, sh, nb);
-    if (threadIdx.x < 2) lg[threadIdx.x] = log(S[threadIdx.x]);  // two lanes, one pass
-    __syncwarp();
     if (threadIdx.x == 0) {
         const uint32_t Rprev = st->R_prev;
-        const int32_t Umin = 2 * (int32_t)st->lmin + r.parity;
-        const int32_t Emin = 2 * Umin - p.d * r.N;
-        const double lnQ = __dsub_rn(__dsub_rn(lg[1], lg[0]),
-                                     __dmul_rn(r.sdbeta[i - 1], (double)Emin));
         const double ess = __ddiv_rn(__dmul_rn(S[1], S[1]), S[2]);
         const int res = ess < __dmul_rn(p.alpha, (double)Rprev) ? 1 : 0;
         int e = 0;
         frexp(mx, &e);
         st->resample = res;
         st->wexp = e;
+        st->S_old = S[0];
         st->S_new = S[1];
         st->S_inv = __ddiv_rn(1.0, S[1]);
         st->T = st->Tres = 0ull;  // summed by k_fsum
         st->epoch += 1u;
         st->kmax = 0;
-        st->sum_lnQ = __dadd_rn(st->sum_lnQ, lnQ);
         TraceRow* tr = r.trace + i;
-        tr->lnQ = lnQ;
-        tr->sum_lnQ = st->sum_lnQ;
         tr->ess = ess;
         tr->resampled = res;
     }
@@ -464,14 +458,11 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_draws(KParams p) {
 // --------------------------------------------------------------------------
 // family statistics of the new population (families stay sorted by slot)
 // --------------------------------------------------------------------------
-template <bool PARTIAL>
 __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int mode, double* a,
-                           double* b, double* ws);
+                           double* b);
 
-// Without partial resampling everything here is known once the ancestors are, so the
-// kernel runs beside the step's sweep (a branch of the captured step).  PARTIAL: partial
-// resampling, after the sweep (weighted sums of its energies).
-template <bool PARTIAL>
+// Everything here is known once the ancestors are, so the kernel runs beside the step's
+// sweep (a branch of the captured step).
 __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
     const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
     const uint32_t b = blockIdx.x - r.blk0;
@@ -576,40 +567,6 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
         r.partCL[b] = sd[0];
         if (sc2) atomicAdd(&r.trace[i].sumC2, sc2);
     }
-    if (PARTIAL) {
-        // partial resampling: the new population's weights (1 after a
-        // resampling, else the kept weight rescaled by 2^-wexp), then the
-        // block's tree sums of w, w E, w E^2, w |M|, w M^2
-        __syncthreads();
-        const int32_t* Ec = r.E[i & 1];
-        double v[5][SCAN_ITEMS];
-#pragma unroll
-        for (int e = 0; e < SCAN_ITEMS; ++e) {
-            const uint32_t d = (uint32_t)(j0 + e);
-            double w = 0.0, E = 0.0, M = 0.0;
-            if (d < Ri) {
-                w = r.w[d];
-                if (mode == 0) {
-                    w = st->resample ? 1.0 : scalbn(w, -st->wexp);
-                    r.w[d] = w;
-                }
-                E = (double)Ec[d];
-                M = (double)r.M[d];
-            }
-            v[0][e] = w;
-            v[1][e] = __dmul_rn(w, E);
-            v[2][e] = __dmul_rn(w, __dmul_rn(E, E));
-            v[3][e] = __dmul_rn(w, fabs(M));
-            v[4][e] = __dmul_rn(w, __dmul_rn(M, M));
-        }
-        double t5[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) t5[q] = tree_regs<SCAN_ITEMS>(v[q]);
-        tree_threads(t5, sd);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int q = 0; q < 5; ++q) r.opart[5 * b + q] = t5[q];
-    }
     // the run's last family block to finish closes the step: its ticket says every
     // other block's partials are written (each fenced them before its ticket)
     __threadfence();
@@ -619,20 +576,19 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_family(KParams p, int mode) {
     if (!last) return;
     if (threadIdx.x == 0) r.tick[1] = 0u;
     __threadfence();
-    finish_run<PARTIAL>(p, r, st, mode, fa, fb, sd);
+    finish_run(p, r, st, mode, fa, fb);
 }
 
 // fixed-order sums of the run's per-block partials and ln Q (its logarithms cost 2000 cycles
 // each on this part: here they run beside the sweep), close the step (one CTA of
-// SCAN_THREADS threads; a, b, ws: shared arrays of SCAN_THREADS doubles)
-template <bool PARTIAL>
+// SCAN_THREADS threads; a, b: shared arrays of SCAN_THREADS doubles)
 __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int mode, double* a,
-                           double* b, double* ws) {
+                           double* b) {
     const int i = st->step;
     __shared__ double lg[2];
-    if (!PARTIAL && mode == 0 && threadIdx.x >= SCAN_THREADS - 32) {  // beside the sums
+    if (mode == 0 && threadIdx.x >= SCAN_THREADS - 32) {  // beside the sums
         const int lane = threadIdx.x & 31;
-        const double lx = log(lane == 0 ? st->S_new : (double)st->R_prev);
+        const double lx = log(lane == 0 ? st->S_new : st->S_old);
         if (lane < 2) lg[lane] = lx;
     }
     const int nb_sv = (mode == 0) ? (int)((st->R_prev + SCAN_CHUNK - 1) / SCAN_CHUNK) : 0;
@@ -650,41 +606,9 @@ __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int
         }
         __syncthreads();
     }
-    if (PARTIAL) {
-        // partial resampling: tree over the blocks' weighted sums
-        // (PARTIAL_MAX_BLOCKS leaves in all, zero past the run's blocks)
-        const int nb = r.nblk;
-        constexpr int LEAVES = PARTIAL_MAX_BLOCKS / 256;
-        double t5[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            if (nb <= 256) {  // a leaf per thread; the leaves past it are zeros
-                t5[q] = (int)threadIdx.x < nb ? __ldcg(&r.opart[5 * threadIdx.x + q]) : 0.0;
-            } else {  // the thread's LEAVES leaves as a tree, in eighths
-                double x8[8];
-                for (int h = 0; h < 8; ++h) {
-                    double x[LEAVES / 8];
-#pragma unroll
-                    for (int k = 0; k < LEAVES / 8; ++k) {
-                        const int bb = LEAVES * threadIdx.x + LEAVES / 8 * h + k;
-                        x[k] = bb < nb ? __ldcg(&r.opart[5 * bb + q]) : 0.0;
-                    }
-                    x8[h] = tree_regs<LEAVES / 8>(x);
-                }
-                t5[q] = tree_regs<8>(x8);
-            }
-        }
-        tree_threads(t5, ws, nb <= 256 ? nb : 256);
-        if (threadIdx.x == 0) {
-            TraceRow* tr = r.trace + i;
-            double* dst[5] = {&tr->wsum, &tr->wE, &tr->wE2, &tr->wAM, &tr->wM2};
-#pragma unroll
-            for (int q = 0; q < 5; ++q) *dst[q] = t5[q];
-        }
-    }
     if (threadIdx.x == 0) {
         TraceRow* tr = r.trace + i;
-        if (!PARTIAL && mode == 0) {
+        if (mode == 0) {
             const int32_t Umin = 2 * (int32_t)st->lmin + r.parity;
             const int32_t Emin = 2 * Umin - p.d * r.N;
             const double lnQ = __dsub_rn(__dsub_rn(lg[0], lg[1]),
@@ -698,6 +622,86 @@ __device__ void finish_run(const KParams& p, const RunDesc& r, DevState* st, int
         tr->c_ln_c = b[0];
         tr->R_i = st->R_cur;
         if (mode != 0) tr->R_prev = st->R_cur;
+    }
+}
+
+// Partial resampling, after the sweep: the new population's weighted sums of 1, E, E^2, |M|
+// and M^2.  rescale: the weights are still those of the old population (k_pop leaves the new
+// ones).  What bounds it: the FP64 pipe (some 55 operations a thread of the CTA's SM).
+__global__ void __launch_bounds__(SCAN_THREADS) k_wsums(KParams p, int rescale) {
+    const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
+    const uint32_t b = blockIdx.x - r.blk0;
+    DevState* st = r.st;
+    if (st->status != S_OK) return;
+    __shared__ double sd[5 * 33];
+    __shared__ int last;
+    const int i = st->step;
+    const uint32_t Ri = st->R_cur;
+    const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
+    // the weights are 1 after a resampling, else the kept ones rescaled by 2^-wexp
+    const int32_t* Ec = r.E[i & 1];
+    double v[5][SCAN_ITEMS];
+#pragma unroll
+    for (int e = 0; e < SCAN_ITEMS; ++e) {
+        const uint32_t d = (uint32_t)(j0 + e);
+        double w = 0.0, E = 0.0, M = 0.0;
+        if (d < Ri) {
+            w = r.w[d];
+            if (rescale) {
+                w = st->resample ? 1.0 : scalbn(w, -st->wexp);
+                r.w[d] = w;
+            }
+            E = (double)Ec[d];
+            M = (double)r.M[d];
+        }
+        v[0][e] = w;
+        v[1][e] = __dmul_rn(w, E);
+        v[2][e] = __dmul_rn(w, __dmul_rn(E, E));
+        v[3][e] = __dmul_rn(w, fabs(M));
+        v[4][e] = __dmul_rn(w, __dmul_rn(M, M));
+    }
+    double t5[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) t5[q] = tree_regs<SCAN_ITEMS>(v[q]);
+    tree_threads(t5, sd);
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int q = 0; q < 5; ++q) r.opart[5 * b + q] = t5[q];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = (atomicAdd(&r.tick[2], 1u) == (uint32_t)r.nblk - 1u);
+    __syncthreads();
+    if (!last) return;
+    if (threadIdx.x == 0) r.tick[2] = 0u;
+    __threadfence();
+    // the run's last block: tree over the blocks' sums (PARTIAL_MAX_BLOCKS leaves in all, zero
+    // past the run's blocks)
+    const int nb = r.nblk;
+    constexpr int LEAVES = PARTIAL_MAX_BLOCKS / 256;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        if (nb <= 256) {  // a leaf per thread; the leaves past it are zeros
+            t5[q] = (int)threadIdx.x < nb ? __ldcg(&r.opart[5 * threadIdx.x + q]) : 0.0;
+        } else {  // the thread's LEAVES leaves as a tree, in eighths
+            double x8[8];
+            for (int h = 0; h < 8; ++h) {
+                double x[LEAVES / 8];
+#pragma unroll
+                for (int k = 0; k < LEAVES / 8; ++k) {
+                    const int bb = LEAVES * threadIdx.x + LEAVES / 8 * h + k;
+                    x[k] = bb < nb ? __ldcg(&r.opart[5 * bb + q]) : 0.0;
+                }
+                x8[h] = tree_regs<LEAVES / 8>(x);
+            }
+            t5[q] = tree_regs<8>(x8);
+        }
+    }
+    tree_threads(t5, sd, nb <= 256 ? nb : 256);
+    if (threadIdx.x == 0) {
+        TraceRow* tr = r.trace + i;
+        double* dst[5] = {&tr->wsum, &tr->wE, &tr->wE2, &tr->wAM, &tr->wM2};
+#pragma unroll
+        for (int q = 0; q < 5; ++q) *dst[q] = t5[q];
     }
 }
 
@@ -1024,7 +1028,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_cscan(KParams p) {
 
 // --------------------------------------------------------------------------
 cudaError_t launch_resample(const KParams& p, cudaStream_t s, int64_t* launches) {
-    if (p.pop && p.alpha < 0.0 && !p.lb_hold) {
+    if (pop_takes(p)) {
         if (launches) *launches += 1;
         return launch_pop(p, s);
     }
@@ -1057,8 +1061,13 @@ cudaError_t launch_partial_init(const KParams& p, cudaStream_t s) {
 }
 
 cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int64_t* launches) {
-    if (p.alpha >= 0.0) k_family<true><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode);
-    else k_family<false><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode);
+    k_family<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode);
+    if (launches) *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_weighted_sums(const KParams& p, int mode, cudaStream_t s, int64_t* launches) {
+    k_wsums<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode == 0 && !pop_takes(p));
     if (launches) *launches += 1;
     return cudaGetLastError();
 }

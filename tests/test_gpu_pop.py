@@ -73,3 +73,29 @@ def test_uneven_batch(rule, graph):
             assert np.array_equal(b.array(m, pa.PA_ARRAY_FAMILY), o.families()), (m, i)
             assert np.array_equal(b.array(m, pa.PA_ARRAY_ENERGY), o.energies()), (m, i)
     b.close()
+
+
+@pytest.mark.parametrize("rule,alpha", [("systematic", 0.6), ("poisson", 0.9), ("residual", 0.6),
+                                        ("multinomial", 1.0), ("nearest", 0.3)])
+@pytest.mark.parametrize("R", [1, 513, 2049, 4097, 9000, 16385, 20000, 33000])
+def test_partial_sizes(rule, alpha, R):
+    d, L = 2, 8
+    betas = np.array([0.0, 0.05, 0.08, 0.5, 0.52, 0.56])
+    n = len(betas) - 1
+    th = np.full(n, 1, np.uint32)
+    cap = pa.default_capacity(R, rule) + 200
+    g = pa.Population(d, L, R, betas, th, rule, 5, R_cap=cap)
+    g.set_partial_resampling(alpha)
+    o = O.Run(d, L, O.ferro_couplings(d, L), R, betas, th, O.RESAMPLERS[rule], 5, R_cap=cap,
+              alpha=alpha)
+    for i in range(n):
+        g.step(1)
+        assert o.step() == 0
+        go, oo = g.observables(), o.obs()
+        _same(go, oo, i)
+        assert go["ess"] == oo["ess"] and go["resampled"] == oo["resampled"], i
+        assert np.array_equal(g.weights(), o.weights()), i
+        assert np.array_equal(g.families(), o.families()), i
+        assert np.array_equal(g.energies(), o.energies()), i
+        assert math.isclose(go["e"], oo["wE"] / (oo["wsum"] * o.N), rel_tol=1e-12), i
+    g.close()
