@@ -132,19 +132,15 @@ struct alignas(128) DevState {
     double S_inv;      // 1 / S_new
     double S_old;      // sum of the weights before the step (the population size, mostly)
     uint32_t epoch;    // resampling steps taken (tags the look-back descriptors)
-    int32_t kmax;      // a Poisson inversion of this step hit its limit
     int32_t hlo, hhi;  // lowest / highest histogram level filled since the last reweighting
 };
 
-// Look-back descriptor of one scan block (single-pass scans of the resampling
-// step): the block's aggregate, then its inclusive prefix, published with a
-// flag tagged by the step's epoch (2e+1: aggregate, 2e+2: inclusive prefix).
-struct LBDesc {
-    uint32_t flag;
-    uint32_t pad;
-    unsigned long long agg[2];
-    unsigned long long inc[2];
-    unsigned long long pad2;
+// Look-back descriptor of one scan block (single-pass scans of the resampling step): the
+// block's aggregates, then its inclusive prefixes in their place.  A 64-bit value is two words
+// of 32 bits under a 32-bit tag of the step's epoch (2e+1: aggregate, 2e+2: inclusive prefix),
+// so one load gives a value and says what it is, without fences.
+struct alignas(32) LBDesc {
+    unsigned long long w[4];
 };
 
 // Per-step accumulators, device-resident (row i = after temperature step i).

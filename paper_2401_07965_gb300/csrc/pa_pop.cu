@@ -1,13 +1,15 @@
-// pa_pop.cu -- the whole resampling of a small population in one launch: weights, copy numbers,
-// (partial resampling: effective size and decision), ancestors and families (pa_resample.cu's kernels, same results bit for bit).
+// pa_pop.cu -- the whole resampling of a small population in one launch: weights, (partial
+// resampling: effective size and decision), copy numbers, ancestors and families
+// (pa_resample.cu's kernels, same results bit for bit).
 //
 // A run is one thread-block cluster of 1 to 16 CTAs, each with POP_CHUNK replicas, two per
 // thread.  Every CTA computes the level weights for itself; block totals, the multinomial
 // searches and their counts go through the cluster's shared memory, so the look-backs, the
 // prefix arrays and the launches between the phases are gone.
-// What bounds it: latency, 16 to 20 thousand cycles (9 to 11 us) of short phases: three block
-// scans with a cluster barrier each 6, the level weights 5, the draws or the copy numbers 3 to
-// 6, the scatter 2, the variance's tree 1.5.  Temperature steps with ten sweeps: 2D L = 16,
+// What bounds it: latency, 14 to 20 thousand cycles (8 to 11 us) of short phases: a block scan
+// with its cluster barrier 2 (one for the rules that need one prefix, three for the drawn
+// ones), the level weights 5, the draws or the copy numbers 3 to 6, the scatter 2, the
+// variance's tree 1.5.  Temperature steps with ten sweeps: 2D L = 16,
 // R = 1000, multinomial (four kernels before) 57 -> 42 us; L = 64, R = 3000, systematic, with
 // the learned schedule 60 -> 53; +-J L = 48, R = 20001, Poisson 231 -> 219; L = 64,
 // R = 10^4, systematic, partial resampling (seven kernels, the family statistics after the
@@ -255,27 +257,31 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
     }
     // ---- expected copies, their prefix and total over the cluster ----
     constexpr uint64_t FMASK = (1ull << FRAC_BITS) - 1;
-    uint64_t tf, tg = 0ull, eg = 0ull;
-    const uint64_t ef = block_excl_scan(f[0] + f[1], sh, &tf);
-    if (method == M_RESIDUAL) eg = block_excl_scan((f[0] & FMASK) + (f[1] & FMASK), sh, &tg);
+    const bool local = method == M_NEAREST || method == M_POISSON;  // no prefix needed
+    uint64_t tg = 0ull, ef = 0ull, eg = 0ull, T = 0ull, G = 0ull, pf = 0ull, pg = 0ull;
     if (!PARTIAL) cl.barrier_wait();
-    if (t < (int)cs) {
-        cl.map_shared_rank(xf, t)[rank] = tf;
-        cl.map_shared_rank(xg, t)[rank] = tg;
-    }
-    sync();
-    uint64_t T = 0ull, G = 0ull, pf = 0ull, pg = 0ull;
-    for (unsigned q = 0; q < cs; ++q) {
-        if (q == rank) {
-            pf = T;
-            pg = G;
+    if (!local) {
+        uint64_t tf;
+        ef = block_excl_scan(f[0] + f[1], sh, &tf);
+        if (method == M_RESIDUAL) eg = block_excl_scan((f[0] & FMASK) + (f[1] & FMASK), sh, &tg);
+        if (t < (int)cs) {
+            cl.map_shared_rank(xf, t)[rank] = tf;
+            cl.map_shared_rank(xg, t)[rank] = tg;
         }
-        T += xf[q];
-        G += xg[q];
+        sync();
+        for (unsigned q = 0; q < cs; ++q) {
+            if (q == rank) {
+                pf = T;
+                pg = G;
+            }
+            T += xf[q];
+            G += xg[q];
+        }
     }
     // ---- copy numbers ----
     uint32_t rc[2] = {0u, 0u};
     bool kmax = false;
+    uint64_t first = 0ull, below = 0ull;  // systematic: labels below the thread's replicas, through them
     if (method == M_MULTINOMIAL || method == M_RESIDUAL) {
         const bool residual = method == M_RESIDUAL, useg = residual && G > 0;
         // every CTA gets the whole population's prefix, over its level arrays (read by now):
@@ -316,10 +322,10 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
         rc[1] = cnt[2 * t + 1];
     } else {
         uint32_t usys = 0u;
-        uint64_t below = 0ull, cf = pf + ef;
+        uint64_t cf = pf + ef;
         if (method == M_SYSTEMATIC) {
             usys = systematic_offset(p, r, i);
-            below = sys_below(cf, r.R, T, usys);
+            first = below = sys_below(cf, r.R, T, usys);
         }
 #pragma unroll 1
         for (int e = 0; e < 2; ++e) {
@@ -342,17 +348,26 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
         }
     }
     // ---- first slot of every replica over the cluster ----
-    uint64_t tot;
-    const uint64_t ex = block_excl_scan((uint64_t)rc[0] + rc[1], sh, &tot);
-    const int km = __syncthreads_or(kmax);
-    if (t < (int)cs) cl.map_shared_rank(xc, t)[rank] = tot | (km ? 1ull << 63 : 0ull);
-    sync();
-    uint64_t Ri = 0ull, pre = 0ull;
+    uint64_t tot, ex, Ri = r.R, pre = 0ull;
     bool anyk = false;
-    for (unsigned q = 0; q < cs; ++q) {
-        if (q == rank) pre = Ri;
-        Ri += xc[q] & ~(1ull << 63);
-        anyk |= (xc[q] >> 63) != 0;
+    if (method == M_SYSTEMATIC) {  // the labels below its lower boundary
+        if (t == 0) sh[0] = first;
+        if (t == POP_THREADS - 1) sh[1] = below;
+        __syncthreads();
+        pre = sh[0];
+        ex = first - pre;
+        tot = sh[1] - pre;
+    } else {
+        ex = block_excl_scan((uint64_t)rc[0] + rc[1], sh, &tot);
+        const int km = __syncthreads_or(kmax);
+        if (t < (int)cs) cl.map_shared_rank(xc, t)[rank] = tot | (km ? 1ull << 63 : 0ull);
+        sync();
+        Ri = 0ull;
+        for (unsigned q = 0; q < cs; ++q) {
+            if (q == rank) pre = Ri;
+            Ri += xc[q] & ~(1ull << 63);
+            anyk |= (xc[q] >> 63) != 0;
+        }
     }
     // ---- ancestors and families (slots past the capacity are not written), the variance ----
     uint32_t* fam1 = r.fam[i & 1];
@@ -414,7 +429,6 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
         close_step(r, st, i, Rprev, lmin, K, S, S_old, t, POP_THREADS);
         if (t == POP_THREADS - 1) {
             // a population that outgrows its capacity, or dies out, stops the run
-            st->kmax = anyk;
             if (anyk) st->status = S_KMAX;
             else if (Ri > (uint64_t)r.Rcap || Ri == 0) st->status = S_CAPACITY;
             else st->R_cur = (uint32_t)Ri;

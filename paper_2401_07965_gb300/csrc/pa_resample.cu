@@ -249,7 +249,6 @@ __global__ void __launch_bounds__(1024) k_weights(KParams p) {
         st->Tres = tsum[1];
         st->Rres = (uint64_t)r.R - ((tsum[0] - tsum[1]) >> FRAC_BITS);
         st->epoch += 1u;
-        st->kmax = 0;
         st->S_new = S;
         st->S_old = (double)Rprev;
         st->R_prev = Rprev;
@@ -351,7 +350,6 @@ __global__ void __launch_bounds__(1024) k_pw_final(KParams p) {
         st->S_inv = __ddiv_rn(1.0, S[1]);
         st->T = st->Tres = 0ull;  // summed by k_fsum
         st->epoch += 1u;
-        st->kmax = 0;
         TraceRow* tr = r.trace + i;
         tr->ess = ess;
         tr->resampled = res;
@@ -715,13 +713,20 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_wsums(KParams p, int rescale) 
 // --------------------------------------------------------------------------
 constexpr uint32_t LB_SPIN_LIMIT = 1u << 22;
 
-__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* a) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
-    return v;
+// a value of a descriptor: its words are written and read one by one, each with its tag
+__device__ __forceinline__ void put_tagged(unsigned long long* w, unsigned long long v, uint32_t tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(w), "l"(t | (v & 0xFFFFFFFFull)),
+                 "l"(t | (v >> 32))
+                 : "memory");
 }
-__device__ __forceinline__ void st_release(uint32_t* a, uint32_t v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
+__device__ __forceinline__ bool get_tagged(const unsigned long long* w, unsigned long long& v,
+                                           uint32_t& tag) {
+    unsigned long long x, y;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(w) : "memory");
+    v = (x & 0xFFFFFFFFull) | (y << 32);
+    tag = (uint32_t)(x >> 32);
+    return tag == (uint32_t)(y >> 32);
 }
 
 __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
@@ -729,69 +734,70 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
     return v;
 }
 
-// Called by the 32 lanes of warp 0.  Publishes (a0, a1) of block b and returns in
-// (p0, p1) the sums over blocks 0..b-1 (every lane); false if a wait gave up.
-// publish = false (a test of the bounded waits) leaves block b's descriptor unset.
-__device__ bool look_back(LBDesc* d, int b, unsigned long long a0, unsigned long long a1,
-                          uint32_t ep, unsigned long long& p0, unsigned long long& p1,
-                          bool publish = true) {
-    const int lane = threadIdx.x & 31;
+// Called by the whole block.  Publishes the NV values a of block b and returns in pre their
+// sums over blocks 0..b-1 (every thread); false if a wait gave up.  A thread waits for one
+// predecessor, SCAN_THREADS of them in one round.  publish = false (a test of the bounded
+// waits) leaves block b's descriptor unset.  One warp looking back over 32 flags at a time,
+// with a fence and a second load for the value, took 8 to 10 k cycles of a block; with two of
+// them per block k_resample took 93 us for 24 runs of R = 50000 (systematic), now 54, and the
+// residual rule at R = 1024000 103 us in its two scans, now 74.
+template <int NV>
+__device__ bool look_back(LBDesc* d, int b, const unsigned long long (&a)[NV], uint32_t ep,
+                          unsigned long long (&pre)[NV], bool publish = true) {
+    constexpr int NW = SCAN_THREADS / 32;
+    __shared__ unsigned long long part[NV][NW];
+    __shared__ int first[NW];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t FA = 2u * ep + 1u, FI = 2u * ep + 2u;
-    if (lane == 0 && publish) {
-        d[b].agg[0] = a0;
-        d[b].agg[1] = a1;
-        if (b == 0) {
-            d[0].inc[0] = a0;
-            d[0].inc[1] = a1;
-        }
-        st_release(&d[b].flag, b == 0 ? FI : FA);
-    }
-    p0 = p1 = 0ull;
-    bool ok = true;
-    if (b > 0) {
-        int j0 = b - 1;
-        uint32_t spins = 0;
-        while (true) {
-            const int j = j0 - lane;
-            const uint32_t f = (j >= 0) ? ld_acquire(&d[j].flag) : FI;
-            const uint32_t valid = __ballot_sync(0xffffffffu, f == FA || f == FI);
-            const uint32_t incl = __ballot_sync(0xffffffffu, f == FI);
-            // lanes 0..m-1 (blocks j0, j0-1, ...) have published
-            const int m = (valid == 0xffffffffu) ? 32 : __ffs(~valid) - 1;
-            const uint32_t usable = incl & (m == 32 ? 0xffffffffu : ((1u << m) - 1u));
-            if (usable) {
-                const int k = __ffs(usable) - 1;
-                unsigned long long v0 = 0ull, v1 = 0ull;
-                if (lane < k) {
-                    v0 = __ldcg(&d[j].agg[0]);
-                    v1 = __ldcg(&d[j].agg[1]);
-                } else if (lane == k && j >= 0) {
-                    v0 = __ldcg(&d[j].inc[0]);
-                    v1 = __ldcg(&d[j].inc[1]);
+    if (threadIdx.x < NV && publish) put_tagged(&d[b].w[2 * threadIdx.x], a[threadIdx.x & (NV - 1)], b == 0 ? FI : FA);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) pre[q] = 0ull;
+    for (int j0 = b - 1; j0 >= 0; j0 -= SCAN_THREADS) {
+        const int j = j0 - (int)threadIdx.x;
+        uint32_t f = FI;  // before block 0: nothing
+        unsigned long long v[NV] = {};
+        bool ok = true;
+        if (j >= 0) {
+            uint32_t spins = 0;
+            while (true) {
+                bool got = get_tagged(&d[j].w[0], v[0], f) && (f == FA || f == FI);
+                if (NV == 2) {
+                    uint32_t f1;
+                    got = get_tagged(&d[j].w[2], v[NV - 1], f1) && f1 == f && got;
                 }
-                p0 += warp_sum_u64(v0);
-                p1 += warp_sum_u64(v1);
-                break;
+                if (got) break;
+                if (++spins > LB_SPIN_LIMIT) {
+                    ok = false;
+                    break;
+                }
+                __nanosleep(32);
             }
-            if (m == 32) {  // 32 aggregates, none inclusive: take them and look further
-                p0 += warp_sum_u64(__ldcg(&d[j].agg[0]));
-                p1 += warp_sum_u64(__ldcg(&d[j].agg[1]));
-                j0 -= 32;
-                continue;
-            }
-            if (++spins > LB_SPIN_LIMIT) {
-                ok = false;
-                break;
-            }
-            __nanosleep(64);
         }
-        if (lane == 0 && ok && publish) {
-            d[b].inc[0] = p0 + a0;
-            d[b].inc[1] = p1 + a1;
-            st_release(&d[b].flag, FI);
+        const uint32_t incl = __ballot_sync(0xffffffffu, f == FI);
+        if (lane == 0) first[warp] = incl ? warp * 32 + __ffs(incl) - 1 : SCAN_THREADS;
+        if (!__syncthreads_and(ok)) return false;
+        int k = SCAN_THREADS;  // the nearest block with its inclusive prefix
+#pragma unroll
+        for (int w = 0; w < NW; ++w) k = min(k, first[w]);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const unsigned long long u = warp_sum_u64((int)threadIdx.x <= k ? v[q] : 0ull);
+            if (lane == 0) part[q][warp] = u;
         }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < NV; ++q)
+#pragma unroll
+            for (int w = 0; w < NW; ++w) pre[q] += part[q][w];
+        if (k < SCAN_THREADS) break;
+        __syncthreads();
     }
-    return __all_sync(0xffffffffu, ok);
+    if (threadIdx.x < NV && b > 0 && publish) {
+        const int q = threadIdx.x & (NV - 1);
+        put_tagged(&d[b].w[2 * q], pre[q] + a[q], FI);
+    }
+    __syncthreads();  // the shared arrays are free again
+    return true;
 }
 
 // the block's ticket: its logical index within the run
@@ -801,36 +807,16 @@ __device__ __forceinline__ int take_ticket(uint32_t* tick, int* sb) {
     return *sb;
 }
 
-// Copy numbers' exclusive scan (look-back over lb2), the ancestor scatter and the
-// block's sampling-variance partial; the last block sets the new population size
+// The ancestor scatter of a block whose slots are [pre, pre + tot), ex of them before the
+// thread's, and its sampling-variance partial; the last block sets the new population size
 // (or the capacity error) and resets the tickets.
-__device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDesc& r,
-                                                   DevState* st, int b,
-                                                   const uint32_t (&rc)[SCAN_ITEMS], uint64_t* sh,
-                                                   double* sd, int* flag_sh,
-                                                   const uint64_t (&fv)[SCAN_ITEMS]) {
+__device__ __forceinline__ void scatter(const KParams& p, const RunDesc& r, DevState* st, int b,
+                                        const uint32_t (&rc)[SCAN_ITEMS], uint64_t ex, uint64_t pre,
+                                        uint64_t tot, double* sd, const uint64_t (&fv)[SCAN_ITEMS],
+                                        bool kmax = false) {
     const int i = st->step;
     const uint32_t Rprev = st->R_prev;
     const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
-    uint64_t sum = 0;
-#pragma unroll
-    for (int e = 0; e < SCAN_ITEMS; ++e) sum += rc[e];
-    uint64_t tot;
-    const uint64_t ex = block_excl_scan(sum, sh, &tot);
-    __shared__ unsigned long long pre;
-    if (threadIdx.x < 32) {
-        unsigned long long p0, p1;
-        const bool ok = look_back(r.lb2, b, tot, 0ull, st->epoch, p0, p1);
-        if (threadIdx.x == 0) {
-            pre = p0;
-            *flag_sh = ok;
-        }
-    }
-    __syncthreads();
-    if (!*flag_sh) {
-        if (threadIdx.x == 0) atomicCAS(&st->status, S_OK, S_TIMEOUT);
-        return;
-    }
     // The block's slots [pre, pre + tot): the total over blocks is known only to the last
     // block, so slots past the capacity are not written (the last block then stops the run
     // with the capacity error).
@@ -891,7 +877,7 @@ __device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDe
         if (b == r.nblk - 1) {
             const uint64_t Ri = pre + tot;
             // a population that outgrows its capacity, or dies out, stops the run
-            if (st->kmax) st->status = S_KMAX;
+            if (kmax) st->status = S_KMAX;
             else if (Ri > (uint64_t)r.Rcap || Ri == 0) st->status = S_CAPACITY;
             else st->R_cur = (uint32_t)Ri;
             r.tick[0] = 0u;
@@ -899,10 +885,34 @@ __device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDe
     }
 }
 
-// Expected copies f_j, their prefix C (and that of the fractional parts, G) by
-// look-back over lb1, and the copy numbers of the rules that need no search.
-// FULL (nearest, systematic, Poisson): then the count scan and the scatter too.
-template <bool FULL>
+// Copy numbers' exclusive scan (look-back over lb2) and the scatter.
+__device__ __forceinline__ void count_scan_scatter(const KParams& p, const RunDesc& r, DevState* st,
+                                                   int b, const uint32_t (&rc)[SCAN_ITEMS],
+                                                   uint64_t* sh, double* sd,
+                                                   const uint64_t (&fv)[SCAN_ITEMS],
+                                                   bool kmax = false, bool publish = true) {
+    uint64_t sum = 0;
+#pragma unroll
+    for (int e = 0; e < SCAN_ITEMS; ++e) sum += rc[e];
+    uint64_t tot;
+    const uint64_t ex = block_excl_scan(sum, sh, &tot);
+    // the second value counts the blocks with a Poisson inversion at its limit
+    const unsigned long long own[2] = {tot, (unsigned long long)(__syncthreads_or(kmax) != 0)};
+    unsigned long long pre[2];
+    if (!look_back(r.lb2, b, own, st->epoch, pre, publish)) {
+        if (threadIdx.x == 0) atomicCAS(&st->status, S_OK, S_TIMEOUT);
+        return;
+    }
+    scatter(p, r, st, b, rc, ex, pre[0], tot, sd, fv, pre[1] + own[1] != 0);
+}
+
+// Expected copies f_j and the copy numbers of the rules that need no search.  A rule needs one
+// look-back here (5 us of waiting each): PREFIX (multinomial, residual) stores the prefix C of
+// the f_j (and G of their fractional parts) for k_draws, by lb1; SYSTEMATIC has the number of
+// labels below C_j for first slots, by lb1; LOCAL (nearest, Poisson) needs no prefix of the
+// f_j, and scans its counts by lb2.
+enum { PREFIX, SYSTEMATIC, LOCAL };
+template <int RULE>
 __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
     const RunDesc& r = p.runs[p.blk2run[blockIdx.x]];
     DevState* st = r.st;
@@ -923,14 +933,12 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
     }
     __shared__ uint64_t sh[33];
     __shared__ double sd[SCAN_THREADS];
-    __shared__ int sb, okf;
-    __shared__ unsigned long long pre[2];
+    __shared__ int sb;
     const int b = take_ticket(&r.tick[0], &sb);
     const int i = st->step;
     const int32_t* E = r.E[(i - 1) & 1];
     const int dN = p.d * r.N;
     const uint32_t Rprev = st->R_prev, lmin = st->lmin;
-    const uint64_t T = st->T;
     const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
     uint64_t f[SCAN_ITEMS];
     uint64_t sf = 0, sg = 0;
@@ -942,65 +950,69 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4) k_resample(KParams p) {
         sf += f[e];
         sg += f[e] & ((1ull << FRAC_BITS) - 1);
     }
-    uint64_t tf, tg;
-    const uint64_t ef = block_excl_scan(sf, sh, &tf);
-    const uint64_t eg = block_excl_scan(sg, sh, &tg);
-    if (threadIdx.x < 32) {
-        unsigned long long p0, p1;
-        const bool ok = look_back(r.lb1, b, tf, tg, st->epoch, p0, p1, !(p.lb_hold && b == 0));
-        if (threadIdx.x == 0) {
-            pre[0] = p0;
-            pre[1] = p1;
-            okf = ok;
+    const int method = p.method;
+    uint32_t rc[SCAN_ITEMS];
+    if constexpr (RULE == LOCAL) {
+        bool kmax = false;
+#pragma unroll 1
+        for (int e = 0; e < SCAN_ITEMS; ++e) {
+            const uint32_t j = (uint32_t)(j0 + e);
+            rc[e] = 0u;
+            if (j >= Rprev) continue;
+            rc[e] = method == M_NEAREST ? nearest_count(p, r, i, j, f[e])
+                                        : poisson_count(p, r, i, j, f[e], kmax);
+            r.counts[j] = rc[e];
         }
+        count_scan_scatter(p, r, st, b, rc, sh, sd, f, kmax, !(p.lb_hold && b == 0));
+        return;
     }
-    __syncthreads();
-    if (!okf) {
+    const uint64_t T = st->T;
+    uint64_t tf, tg = 0ull, eg = 0ull;
+    const uint64_t ef = block_excl_scan(sf, sh, &tf);
+    if (RULE == PREFIX) eg = block_excl_scan(sg, sh, &tg);
+    constexpr int NV = RULE == PREFIX ? 2 : 1;
+    unsigned long long own[NV], pr[NV];
+    own[0] = tf;
+    if (NV == 2) own[NV - 1] = tg;
+    if (!look_back(r.lb1, b, own, st->epoch, pr, !(p.lb_hold && b == 0))) {
         if (threadIdx.x == 0) atomicCAS(&st->status, S_OK, S_TIMEOUT);
         return;
     }
-    uint64_t cf = pre[0] + ef, cg = pre[1] + eg;
-    const int method = p.method;
-    const uint32_t usys = method == M_SYSTEMATIC ? systematic_offset(p, r, i) : 0u;
-    bool kmax = false;
-    uint32_t rc[SCAN_ITEMS];
-    // systematic: labels below the running boundary, carried from item to item
-    uint64_t below = method == M_SYSTEMATIC ? sys_below(cf, r.R, T, usys) : 0ull;
-#pragma unroll 1
-    for (int e = 0; e < SCAN_ITEMS; ++e) {
-        const int j = j0 + e;
-        rc[e] = 0u;
-        if ((uint32_t)j >= Rprev) continue;
-        cf += f[e];
-        cg += f[e] & ((1ull << FRAC_BITS) - 1);
-        uint32_t cnt = 0;
-        if (method == M_NEAREST) {
-            cnt = nearest_count(p, r, i, (uint32_t)j, f[e]);
-        } else if (method == M_SYSTEMATIC) {
-            const uint64_t bn = sys_below(cf, r.R, T, usys);
-            cnt = (uint32_t)(bn - below);
-            below = bn;
-        } else if (method == M_RESIDUAL) {
+    uint64_t cf = pr[0] + ef, cg = pr[NV - 1] + eg;
+    if constexpr (RULE == PREFIX) {
+#pragma unroll
+        for (int e = 0; e < SCAN_ITEMS; ++e) {
+            const int j = j0 + e;
+            if ((uint32_t)j >= Rprev) continue;
+            cf += f[e];
+            cg += f[e] & ((1ull << FRAC_BITS) - 1);
             r.C[j] = cf;
-            r.G[j] = cg;
-            cnt = (uint32_t)(f[e] >> FRAC_BITS);
-        } else if (method == M_MULTINOMIAL) {
-            r.C[j] = cf;
-        } else {
-            cnt = poisson_count(p, r, i, (uint32_t)j, f[e], kmax);
+            if (method == M_RESIDUAL) r.G[j] = cg;
+            r.counts[j] = method == M_RESIDUAL ? (uint32_t)(f[e] >> FRAC_BITS) : 0u;
         }
-        rc[e] = cnt;
-        r.counts[j] = cnt;
-    }
-    if (kmax) {  // promoted to the status word by the scan's last block
-        atomicOr(&st->kmax, 1);
-        __threadfence();
-    }
-    if (!FULL) {
         if (threadIdx.x == 0 && b == r.nblk - 1) r.tick[0] = 0u;
-        return;
+    } else {
+        // labels below the running boundary, carried from item to item: the first slots
+        const uint32_t usys = systematic_offset(p, r, i);
+        const uint64_t first = sys_below(cf, r.R, T, usys);
+        uint64_t below = first;
+#pragma unroll 1
+        for (int e = 0; e < SCAN_ITEMS; ++e) {
+            const int j = j0 + e;
+            rc[e] = 0u;
+            if ((uint32_t)j >= Rprev) continue;
+            cf += f[e];
+            const uint64_t bn = sys_below(cf, r.R, T, usys);
+            rc[e] = (uint32_t)(bn - below);
+            below = bn;
+            r.counts[j] = rc[e];
+        }
+        if (threadIdx.x == 0) sh[0] = first;
+        if (threadIdx.x == SCAN_THREADS - 1) sh[1] = below;
+        __syncthreads();
+        const uint64_t pre = sh[0];
+        scatter(p, r, st, b, rc, first - pre, pre, sh[1] - pre, sd, f);
     }
-    count_scan_scatter(p, r, st, b, rc, sh, sd, &okf, f);
 }
 
 // multinomial / residual: the copy numbers are complete after k_draws
@@ -1010,7 +1022,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_cscan(KParams p) {
     if (st->status != S_OK || (p.alpha >= 0.0 && !st->resample)) return;
     __shared__ uint64_t sh[33];
     __shared__ double sd[SCAN_THREADS];
-    __shared__ int sb, okf;
+    __shared__ int sb;
     const int b = take_ticket(&r.tick[0], &sb);
     const uint32_t Rprev = st->R_prev;
     const int j0 = b * SCAN_CHUNK + threadIdx.x * SCAN_ITEMS;
@@ -1023,7 +1035,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_cscan(KParams p) {
         rc[e] = in ? r.counts[j] : 0u;
         f[e] = in ? r.C[j] - (j > 0 ? r.C[j - 1] : 0ull) : 0ull;
     }
-    count_scan_scatter(p, r, st, b, rc, sh, sd, &okf, f);
+    count_scan_scatter(p, r, st, b, rc, sh, sd, f);
 }
 
 // --------------------------------------------------------------------------
@@ -1043,12 +1055,13 @@ cudaError_t launch_resample(const KParams& p, cudaStream_t s, int64_t* launches)
         n += 3;
     }
     if (p.method == M_MULTINOMIAL || p.method == M_RESIDUAL) {
-        k_resample<false><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
+        k_resample<PREFIX><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
         k_draws<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
         k_cscan<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
         n += 3;
     } else {
-        k_resample<true><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
+        if (p.method == M_SYSTEMATIC) k_resample<SYSTEMATIC><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
+        else k_resample<LOCAL><<<p.nblk_total, SCAN_THREADS, 0, s>>>(p);
         n += 1;
     }
     if (launches) *launches += n;
