@@ -465,7 +465,8 @@ double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT) {
     const double er = rows >= 16 ? 1.0 : rows >= 12 ? 0.97 : rows >= 8 ? 0.93 : rows >= 6 ? 0.9
                       : rows >= 4 ? 0.85 : rows >= 2 ? 0.65 : 0.45;
     const int G = GP * CPT, nt = std::max(32, (GP * tg + 31) / 32 * 32);
-    const int hold = std::max(1, std::min(32, 65536 / (nt * regs))) * G;  // groups an SM holds
+    // groups an SM holds: each of its four schedulers has registers for whole warps
+    const int hold = std::max(1, 4 * (16384 / (32 * regs)) / (nt / 32)) * G;
     const int ncta = (int)((ngrp + G - 1) / G);
     const int most = std::min<int>((ncta + 151) / 152 * G, (int)ngrp);
     auto round = [&](double n) { return n > 0.0 ? n + 1.6 * 128.0 * CPT / tg : 0.0; };  // n at once

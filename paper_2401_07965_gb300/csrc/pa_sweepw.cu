@@ -29,7 +29,7 @@
 //
 // What bounds it: as in pa_sweep2d.cu the issue of logic operations and wide multiplies
 // (L = 8: about 150 of them per site word, 171 with the halo layout and its site tables).
-// +-J, theta = 10, beta 0 -> 3, updates/ns, before -> now: 64 runs of L = 4 2676 -> 3008,
+// +-J, theta = 10, beta 0 -> 3, updates/ns, before -> now: 64 runs of L = 4 2676 -> 3240,
 // 32 of L = 6 3225 -> 3526, 16 of L = 8 3474 -> 3742 (R = 50000 each), 4 of L = 16,
 // R = 20000 2643 -> 3514; one run of L = 6, R = 10^5 1798 -> 2497 (its level counts and
 // sums now leave the CTA once); ferromagnet L = 20, 4 runs of R = 10^4 2558 -> 2689.
@@ -99,7 +99,13 @@ __host__ __device__ inline WalkSmem walk_smem(const WalkPlan& g, int D, bool ea)
     const int G = g.GP * g.CPT;
     int o = (G * g.GS * 4 + 15) & ~15;
     m.lists = o;  // undecided sites; after the sweeps the per-replica sums sU, sNup
-    o += ((g.NT / 32) * 32 * g.span * g.CPT * 8 > G * 64 * 4 ? (g.NT / 32) * 32 * g.span * g.CPT * 8 : G * 64 * 4);
+    // ... and the CTA's level counts where the lattice is small (L = 4, 8 runs of R = 50000,
+    // four groups per CTA, where the lists leave no room: 150 us a step of ten sweeps with
+    // every replica counted in global memory, 126 with room)
+    const int nlev = D * (D == 3 ? g.L * g.L * g.L : g.L * g.L) / 2 + 1;
+    const int list = (g.NT / 32) * 32 * g.span * g.CPT * 8;
+    const int sums = G * 64 * 4 + (nlev <= 1024 ? nlev * 4 : 0);
+    o += ((list > sums ? list : sums) + 15) & ~15;
     m.jt = o;
     if (ea) o += 2 * g.CS;
     o = (o + 15) & ~15;
