@@ -210,7 +210,7 @@ def _sweep_traffic(kernel_src_hash):
 
 def _src_hash():
     h = hashlib.sha256()
-    for f in ("pa_sweep2d.cu", "pa_sweep_common.cuh", "pa_internal.cuh"):
+    for f in ("pa_sweep2d.cu", "pa_walk.cuh", "pa_sweep_common.cuh", "pa_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2401_07965_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -457,7 +457,7 @@ def run_ours(args):
         p3, h3 = mean_pipes(3, ea3d["timed_betas"])
         ea3d["roofline"] = roofline_record(p3, ea3d["sweep_updates_per_ns"], nsm, f_hz)
         ea3d["roofline"]["zero_class_steps"] = {str(z): c for z, c in sorted(h3.items())}
-        ea3d["roofline"]["kernel"] = "k_sweep3d<L,true> (L = 4, 6, 8; grouped replicas)"
+        ea3d["roofline"]["kernel"] = "k_walk<3,L,true> (L = 4, 6, 8; column walks)"
     cpu = cpu_mt = None
     if not args.no_cpu_baseline and world == 1:
         cpu = oracle_baseline(64, 5, parallel=False)

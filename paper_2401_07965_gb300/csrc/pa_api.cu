@@ -460,8 +460,8 @@ pa_status grow_event_pool(pa_ctx* ctx, size_t n) {
 
 // All kernels of one temperature step (and the controller's choice of the next).  The
 // family statistics need the ancestors only: while a step is captured they go to a
-// branch beside the sweep (side != nullptr).  Under partial resampling they carry
-// weighted sums of the sweep's energies and follow it.
+// branch beside the sweep (side != nullptr).  The weighted sums of partial resampling
+// take the sweep's energies and follow it.
 pa_status enqueue_step(pa_ctx* ctx, int64_t* launches, cudaStream_t stream,
                        cudaStream_t side) {
     PA_CUDA(launch_resample(ctx->kp, stream, launches));

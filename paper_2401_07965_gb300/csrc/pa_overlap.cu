@@ -17,7 +17,8 @@
 // pass is needed.  The kernel is bound by HBM: 2 Wp words per replica pair are
 // read once.
 //
-// k_overlap_P: the weighted estimate over pairs, one thread per k,
+// k_overlap_P: the weighted estimate over pairs, one thread per k, the pairs' weights
+// formed once per CTA,
 //   P(k) = sum_p omega_p hist_p[k] / n_p,  omega_p ∝ (R_i^a Zhat_a)(R_i^b Zhat_b),
 // the product of the two populations' weights of Eq. (weighted-averages)
 // (independent populations: the joint weight factorises), pairs summed in

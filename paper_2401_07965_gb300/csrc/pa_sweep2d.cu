@@ -25,9 +25,8 @@
 //
 // Undecided sites.  After two unconditional plane blocks (eight bits of the
 // uniforms) a site flips the replicas that are decided; a site with undecided
-// ones (12% at most) keeps their mask in a slot of its own and sets the site's bit
-// in the thread's register, both under a predicate.  After its rows the warp
-// lists the set bits (one prefix sum over the lanes) and finishes the listed sites
+// ones (12% at most) goes to the warp's list with their mask (a shared-memory
+// atomic under a predicate).  After its rows the warp finishes the listed sites
 // one per lane, from plane block 2 on; the undecided replicas have not flipped, so
 // their classes come from the site again.
 //
