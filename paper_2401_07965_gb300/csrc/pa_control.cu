@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(64) k_mlp_fwd(const uint16_t* __restrict__ par
 // What bounds it: shared-memory latency on one CTA per SM (30 k flops per row).  GR = 32, 64
 // or 96, the least that takes the rows of one of 152 CTAs in one pass: 12040 rows are 151
 // CTAs of 80 rows; two passes of 64 with 256 threads took 33 us, one pass 22 us (the whole
-// update of 12040 rows: 66 us with the forward pass stored and read back, now 30).
+// update of 12040 rows: 66 us with the forward pass stored and read back, 31 with one kernel,
+// 29 with the reduction chained to it).
 // --------------------------------------------------------------------------
 constexpr int LDW = MLP_HID + 4;  // padded rows of units: 16-byte aligned
 
@@ -126,6 +127,7 @@ __global__ void __launch_bounds__(8 * GR) k_mlp_grad(const float* __restrict__ p
     extern __shared__ __align__(16) unsigned char raw[];
     GradSmem<GR>& s = *reinterpret_cast<GradSmem<GR>*>(raw);
     const int t = threadIdx.x, ti = t % (GR / 2), tj = t / (GR / 2);  // rows 2 ti.., units 4 tj..
+    chain_next();
     for (int e = t; e < MLP_HID * MLP_HID; e += GT) {
         const float v = bf_round(params[OFF_W2 + e]);
         s.w2[(e >> 6) * LDW + (e & 63)] = v;
@@ -337,12 +339,11 @@ cudaError_t launch_grad(const float* params, const float* X, const float* Yt, co
 
 // fixed-order sum of the per-CTA parts: eight warps of a CTA take the parts b = w, w + 8,
 // ... of 32 parameters, then the eight sums in order
-__global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ part, int nb,
-                                                    float* __restrict__ grads,
-                                                    float* __restrict__ loss) {
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float* part, int nb, float* grads, float* loss) {
     __shared__ float sh[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
     float acc = 0.0f;
+    chain_wait();
     if (k <= MLP_NPARAM)
 #pragma unroll 8
         for (int b = w; b < nb; b += 8) acc += part[(size_t)b * (MLP_NPARAM + 1) + k];
@@ -411,8 +412,10 @@ pa_status pa_mlp_gradients(const float* params, const float* X, const float* Yt,
         : rows <= 64 ? launch_grad<64>(params, X, Yt, mask, B, rows, nb, norm, part, s)
                      : launch_grad<96>(params, X, Yt, mask, B, rows, nb, norm, part, s);
     if (e != cudaSuccess) return PA_ERR_CUDA;
-    k_mlp_reduce<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, s>>>(part, (int)nb, grads, loss);
-    return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
+    return launch_chained(k_mlp_reduce, (MLP_NPARAM + 1 + 31) / 32, 256u, 0, s, part, (int)nb, grads,
+                          loss) == cudaSuccess
+               ? PA_OK
+               : PA_ERR_CUDA;
 }
 
 pa_status pa_mlp_adam(float* params, const float* grads, float* m, float* v, uint16_t* params_bf16,

@@ -10,7 +10,7 @@
 // with its cluster barrier 2 (one for the rules that need one prefix, three for the drawn
 // ones), the level weights 5, the draws or the copy numbers 3 to 6, the scatter 2, the
 // variance's tree 1.5.  Temperature steps with ten sweeps: 2D L = 16,
-// R = 1000, multinomial (four kernels before) 57 -> 42 us; L = 64, R = 3000, systematic, with
+// R = 1000, multinomial (four kernels before) 57 -> 42 us, 41 with the sweep chained to it; L = 64, R = 3000, systematic, with
 // the learned schedule 60 -> 53; +-J L = 48, R = 20001, Poisson 231 -> 219; L = 64,
 // R = 10^4, systematic, partial resampling (seven kernels, the family statistics after the
 // sweep) 202 -> 185.
@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(POP_THREADS, 1) k_pop(KParams p) {
     constexpr int POP_CHUNK = 2 * POP_THREADS;  // replicas of a CTA
     cg::cluster_group cl = cg::this_cluster();
     const unsigned cs = cl.num_blocks(), rank = cl.block_rank();
+    chain_next();  // the sweep's CTAs
     const auto sync = [&] {  // one CTA needs no cluster barrier (1000 cycles)
         if (cs == 1) __syncthreads();
         else cl.sync();

@@ -55,6 +55,7 @@ k_static_weights(StaticScratch* sc, const int32_t* __restrict__ E, uint32_t R_pr
     __shared__ int s_lo, s_hi, s_bad, s_last;
     const int nlev = d * N / 2 + 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pa::chain_next();
     for (int l = threadIdx.x; l < nlev; l += STATIC_THREADS) sh[l] = 0u;
     if (threadIdx.x == 0) {
         s_lo = nlev;
@@ -185,12 +186,19 @@ k_static_weights(StaticScratch* sc, const int32_t* __restrict__ E, uint32_t R_pr
 
 // f_j of every replica from the level table (a launch of its own: every CTA needs it)
 __global__ void __launch_bounds__(256)
-k_static_f(const StaticScratch* __restrict__ sc, const int32_t* __restrict__ E, uint32_t R_prev,
-           int dN, uint64_t* __restrict__ f_out) {
+k_static_f(const StaticScratch* sc, const int32_t* E, uint32_t R_prev, int dN, uint64_t* f_out) {
+    uint64_t j = (uint64_t)blockIdx.x * 256u + threadIdx.x;
+    int32_t Ej = j < R_prev ? E[j] : 0;  // not written by the kernel before
+    pa::chain_wait();
     if (!sc->ok) return;
     const int lmin = sc->lmin;
-    for (uint64_t j = (uint64_t)blockIdx.x * 256u + threadIdx.x; j < R_prev; j += gridDim.x * 256u)
-        f_out[j] = sc->flev[((E[j] + dN) >> 2) - lmin];
+    while (j < R_prev) {
+        const uint64_t next = j + gridDim.x * 256u;
+        const int32_t En = next < R_prev ? E[next] : 0;
+        f_out[j] = sc->flev[((Ej + dN) >> 2) - lmin];
+        j = next;
+        Ej = En;
+    }
 }
 
 }  // namespace
@@ -227,6 +235,7 @@ extern "C" pa_status pa_weights_static(const int32_t* E, uint32_t R_prev, uint32
                                                      lnQ, na == 1 ? f : nullptr);
     if (na == 1) return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
     const unsigned nf = (unsigned)std::min<uint64_t>(((uint64_t)R_prev + 1023u) / 1024u, 152u * 8u);
-    k_static_f<<<nf, 256, 0, st>>>(sc, E, R_prev, dim * (int)N, f);
-    return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
+    return pa::launch_chained(k_static_f, nf, 256u, 0, st, sc, E, R_prev, dim * (int)N, f) == cudaSuccess
+               ? PA_OK
+               : PA_ERR_CUDA;
 }

@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
 
     const RunDesc& r = p.runs[cta2run[blockIdx.x]];
     const DevState* st = r.st;
+    chain_wait();
     if (st->status != S_OK) return;
     const int i = st->step;
     const uint32_t R = st->R_cur;
@@ -409,9 +410,8 @@ cudaError_t launch2d(const KParams& p, const uint32_t* cta2run, uint32_t ncta, c
         attr_set = true;
     }
     if (attr_only || ncta == 0) return cudaSuccess;
-    k_sweep2d<L, NT, G, EA, MINB>
-        <<<ncta, NT, spread_smem(sm, ncta, NT, NT == 512 ? 128 : 96), s>>>(p, cta2run);
-    return cudaGetLastError();
+    return launch_chained(k_sweep2d<L, NT, G, EA, MINB>, ncta, (unsigned)NT,
+                          spread_smem(sm, ncta, NT, NT == 512 ? 128 : 96), s, p, cta2run);
 }
 
 template <int L, int NT, int G>

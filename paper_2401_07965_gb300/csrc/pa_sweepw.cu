@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
 
     const RunDesc& r = p.runs[cta2run[blockIdx.x]];
     const DevState* st = r.st;
+    chain_wait();
     if (st->status != S_OK) return;
     const int i = st->step;
     const uint32_t R = st->R_cur;
@@ -573,8 +574,7 @@ cudaError_t launch_walk_t(const KParams& p, const WalkPlan& g, const uint32_t* c
     }
     if (attr_only || ncta == 0) return cudaSuccess;
     const size_t sm = spread_smem((size_t)walk_smem(g, D, EA).total, ncta, g.NT, 96);
-    k_walk<D, LT, EA><<<ncta, g.NT, sm, s>>>(p, g, cta2run);
-    return cudaGetLastError();
+    return launch_chained(k_walk<D, LT, EA>, ncta, (unsigned)g.NT, sm, s, p, g, cta2run);
 }
 
 template <bool EA>
