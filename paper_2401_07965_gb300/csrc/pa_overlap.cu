@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(256) k_overlap_hist(KParams p, const int32_t* 
                                                       uint32_t* tickets) {
     extern __shared__ uint32_t sh[];
     __shared__ int last_cta;
+    chain_next();  // k_overlap_P
     const int pair = blockIdx.y;
     const RunDesc& ra = p.runs[pairs[2 * pair]];
     const RunDesc& rb = p.runs[pairs[2 * pair + 1]];
@@ -97,7 +98,8 @@ __global__ void __launch_bounds__(256) k_overlap_hist(KParams p, const int32_t* 
 
 // The pairs' weights once per CTA (a logarithm takes about 2000 cycles here, so a thread
 // takes one pair's), then a thread sums its k over the pairs in index order.  With every
-// thread forming every pair's weight twice, 16 pairs took 133 us.
+// thread forming every pair's weight twice, 16 pairs took 133 us.  The kernel is chained to
+// k_overlap_hist and forms the weights before it waits: a call of 16 pairs 192 -> 184 us.
 constexpr int OVP_T = 128;
 __global__ void __launch_bounds__(OVP_T) k_overlap_P(KParams p, const int32_t* pairs, int n_pairs,
                                                      int bins, const uint32_t* hist, double* P) {
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(OVP_T) k_overlap_P(KParams p, const int32_t* p
     }
     __syncthreads();
     lmax = smax;
+    chain_wait();  // the weights come from the runs' traces, the counts from k_overlap_hist
     double S = 0.0, acc = 0.0;
     for (int q0 = 0; q0 < n_pairs; q0 += OVP_T) {
         const int q = q0 + threadIdx.x;
@@ -168,8 +171,8 @@ cudaError_t launch_overlap(const KParams& p, const int32_t* pairs, int n_pairs, 
         k_overlap_hist<false><<<grid, 256, 0, s>>>(p, pairs, G, bins, hist, acc, tickets);
     e = cudaGetLastError();
     if (e != cudaSuccess || !P) return e;
-    k_overlap_P<<<(bins + OVP_T - 1) / OVP_T, OVP_T, 0, s>>>(p, pairs, n_pairs, bins, hist, P);
-    return cudaGetLastError();
+    return launch_chained(k_overlap_P, (unsigned)((bins + OVP_T - 1) / OVP_T), (unsigned)OVP_T, 0, s, p,
+                          pairs, n_pairs, bins, (const uint32_t*)hist, P);
 }
 
 }  // namespace pa
