@@ -76,9 +76,9 @@ struct pa_ctx {
     pa_status sticky = PA_OK;
     bool timing = false;
     bool use_graph = true;
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph[2] = {};          // one captured step, GRAPH_STEPS of them
     int graph_threads = 0;
-    int64_t graph_kernels = 0;
+    int64_t graph_kernels[2] = {};
     cudaStream_t cap = nullptr, side = nullptr;  // the captured step and its branch
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::vector<cudaEvent_t> ev_start, ev_stop;  // pool of timing events, reused
@@ -425,6 +425,19 @@ void plan_sweep(pa_ctx* ctx, int gm, uint32_t* map, std::vector<uint32_t>& c3) {
     }
 }
 
+// Steps of the larger captured graph.  Between two graph launches the GPU stands idle
+// longer than between two kernels of one: 2D L = 16, R = 1000, 100 steps 4078 -> 3940 us, the
+// learned schedule at R = 3000 18.7 -> 18.2 ms; capturing eight steps instead of one takes
+// some 20 us, so the graph is built where a call has at least two of them to run.
+constexpr int GRAPH_STEPS = 8;
+
+void drop_graphs(pa_ctx* ctx) {
+    for (cudaGraphExec_t& g : ctx->graph) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+}
+
 // rebuild the plan (after a change of threads or of the group multiple): no step in
 // flight may read the old one
 pa_status replan(pa_ctx* ctx, int gm) {
@@ -435,10 +448,7 @@ pa_status replan(pa_ctx* ctx, int gm) {
         PA_CUDA(cudaMemcpy(ctx->d_cta, c3.data(), c3.size() * 4, cudaMemcpyHostToDevice));
     PA_CUDA(cudaMemcpy((void*)ctx->kp.runs, ctx->desc.data(), sizeof(RunDesc) * ctx->desc.size(),
                        cudaMemcpyHostToDevice));
-    if (ctx->graph) {  // the captured step holds the old launch configuration
-        cudaGraphExecDestroy(ctx->graph);
-        ctx->graph = nullptr;
-    }
+    drop_graphs(ctx);  // the captured step holds the old launch configuration
     return PA_OK;
 }
 
@@ -524,13 +534,9 @@ uint32_t run_theta(const pa_ctx* ctx, int run, int i) {
     return ctx->controlled ? ctx->rtheta[run][i] : ctx->theta[i];
 }
 
-// capture one temperature step; every kernel reads the step index and the
-// population sizes from device memory, so the same graph serves every step
-pa_status build_graph(pa_ctx* ctx) {
-    if (ctx->graph) {
-        cudaGraphExecDestroy(ctx->graph);
-        ctx->graph = nullptr;
-    }
+// capture one temperature step (many = 0) or GRAPH_STEPS of them; every kernel reads the
+// step index and the population sizes from device memory, so the same graph serves every step
+pa_status build_graph(pa_ctx* ctx, int many) {
     PA_CUDA(prepare_sweep(ctx->kp, ctx->threads));
     if (!ctx->side) {
         int least = 0, greatest = 0;
@@ -546,7 +552,9 @@ pa_status build_graph(pa_ctx* ctx) {
     // take their places on some SMs and leave the sweep unevenly spread
     PA_CUDA(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
     int64_t n = 0;
-    const pa_status s = enqueue_step(ctx, &n, ctx->cap, ctx->side);
+    pa_status s = PA_OK;
+    for (int k = many ? GRAPH_STEPS : 1; k > 0 && s == PA_OK; --k)
+        s = enqueue_step(ctx, &n, ctx->cap, ctx->side);
     const cudaError_t e = cudaStreamEndCapture(ctx->cap, &g);
     if (s != PA_OK) {
         if (g) cudaGraphDestroy(g);
@@ -556,15 +564,15 @@ pa_status build_graph(pa_ctx* ctx) {
         ctx->sticky = PA_ERR_CUDA;
         return PA_ERR_CUDA;
     }
-    const cudaError_t ei = cudaGraphInstantiate(&ctx->graph, g, 0);
+    const cudaError_t ei = cudaGraphInstantiate(&ctx->graph[many], g, 0);
     cudaGraphDestroy(g);
     if (ei != cudaSuccess) {
-        ctx->graph = nullptr;
+        ctx->graph[many] = nullptr;
         ctx->sticky = PA_ERR_CUDA;
         return PA_ERR_CUDA;
     }
     ctx->graph_threads = ctx->threads;
-    ctx->graph_kernels = n;
+    ctx->graph_kernels[many] = n;
     return PA_OK;
 }
 
@@ -884,21 +892,25 @@ pa_status pa_step(pa_ctx* ctx, int32_t n) {
     }
     if (ctx->host_step + n > ctx->n_steps) return PA_ERR_DONE;
     const bool graph = ctx->use_graph && !ctx->timing && ctx->stream != nullptr;
-    if (graph && n > 0 && (!ctx->graph || ctx->graph_threads != ctx->threads)) {
-        const pa_status s = build_graph(ctx);
-        if (s != PA_OK) return s;
-    }
-    for (int k = 0; k < n; ++k) {
-        const int i = ctx->host_step + 1;
+    if (graph && ctx->graph_threads != ctx->threads) drop_graphs(ctx);
+    while (n > 0) {
+        int took = 1;
         if (graph) {
-            PA_CUDA(cudaGraphLaunch(ctx->graph, ctx->stream));
-            ctx->launches += ctx->graph_kernels;
+            const int many = n >= 2 * GRAPH_STEPS || (n >= GRAPH_STEPS && ctx->graph[1]);
+            if (!ctx->graph[many]) {
+                const pa_status s = build_graph(ctx, many);
+                if (s != PA_OK) return s;
+            }
+            PA_CUDA(cudaGraphLaunch(ctx->graph[many], ctx->stream));
+            ctx->launches += ctx->graph_kernels[many];
+            if (many) took = GRAPH_STEPS;
         } else {
-            if (ctx->timing) ctx->timed_steps.push_back(i);
+            if (ctx->timing) ctx->timed_steps.push_back(ctx->host_step + 1);
             const pa_status s = enqueue_step(ctx, &ctx->launches, ctx->stream, nullptr);
             if (s != PA_OK) return s;
         }
-        ctx->host_step = i;
+        ctx->host_step += took;
+        n -= took;
     }
     return PA_OK;
 }
@@ -1171,10 +1183,7 @@ pa_status pa_set_partial_resampling(pa_ctx* ctx, double alpha) {
         t.wM2 = (double)(long long)t.sumM2;
         PA_CUDA(cudaMemcpy(ctx->desc[m].trace, &t, sizeof(t), cudaMemcpyHostToDevice));
     }
-    if (ctx->graph) {  // the step graph must now include the weight kernels
-        cudaGraphExecDestroy(ctx->graph);
-        ctx->graph = nullptr;
-    }
+    drop_graphs(ctx);  // the step graph must now include the weight kernels
     return pa_sync(ctx);
 }
 
@@ -1254,10 +1263,7 @@ pa_status pa_set_controller(pa_ctx* ctx, const pa_controller* cfg) {
     ctx->rdone.assign(ctx->M, 0);
     ctx->kp.ctl = ctx->d_ctl;
     ctx->controlled = true;
-    if (ctx->graph) {  // the step graph must now include the controller
-        cudaGraphExecDestroy(ctx->graph);
-        ctx->graph = nullptr;
-    }
+    drop_graphs(ctx);  // the step graph must now include the controller
     // choose the first step from the initial population
     PA_CUDA(launch_control(ctx->kp, ctx->stream));
     ctx->launches += 1;
@@ -1355,20 +1361,14 @@ int32_t pa_get_sweep_threads(const pa_ctx* ctx) { return ctx ? ctx->threads : 0;
 pa_status pa_set_sweep_queue(pa_ctx* ctx, int32_t cap) {
     if (!ctx || cap < -1) return PA_ERR_ARG;
     ctx->kp.qcap_limit = cap;
-    if (ctx->graph) {  // the captured step holds the old kernel parameters
-        cudaGraphExecDestroy(ctx->graph);
-        ctx->graph = nullptr;
-    }
+    drop_graphs(ctx);  // the captured step holds the old kernel parameters
     return PA_OK;
 }
 
 pa_status pa_set_wait_test(pa_ctx* ctx, int32_t on) {
     if (!ctx || (on != 0 && on != 1)) return PA_ERR_ARG;
     ctx->kp.lb_hold = on;
-    if (ctx->graph) {  // the captured step holds the old kernel parameters
-        cudaGraphExecDestroy(ctx->graph);
-        ctx->graph = nullptr;
-    }
+    drop_graphs(ctx);  // the captured step holds the old kernel parameters
     return PA_OK;
 }
 
@@ -1378,7 +1378,7 @@ pa_status pa_destroy(pa_ctx* ctx) {
         cudaEventDestroy(ctx->ev_start[k]);
         cudaEventDestroy(ctx->ev_stop[k]);
     }
-    if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
+    drop_graphs(ctx);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
     if (ctx->cap) cudaStreamDestroy(ctx->cap);
