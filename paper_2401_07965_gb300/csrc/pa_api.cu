@@ -427,8 +427,8 @@ void plan_sweep(pa_ctx* ctx, int gm, uint32_t* map, std::vector<uint32_t>& c3) {
 
 // Steps of the larger captured graph.  Between two graph launches the GPU stands idle
 // longer than between two kernels of one: 2D L = 16, R = 1000, 100 steps 4078 -> 3940 us, the
-// learned schedule at R = 3000 18.7 -> 18.2 ms; capturing eight steps instead of one takes
-// some 20 us, so the graph is built where a call has at least two of them to run.
+// learned schedule at R = 3000 18.7 -> 18.2 ms (each run captures its graphs anew).  The graph
+// is built where a call has at least two of them to run, so that its capture pays.
 constexpr int GRAPH_STEPS = 8;
 
 void drop_graphs(pa_ctx* ctx) {
