@@ -205,7 +205,7 @@ __host__ __device__ __forceinline__ int queue_capacity(int N) {
 // mode 1: measurement of the current population only (init / restore).
 // ---------------------------------------------------------------------------
 template <int D, bool EA, int NT>
-__global__ void __launch_bounds__(NT) k_group(KParams p, int mode) {
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_group(KParams p, int mode) {
     extern __shared__ __align__(16) uint32_t smem[];
     // the CTA's run and its replica group within the run; the flattened CTA
     // index is the global replica group of the sweep draws
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(NT) k_group(KParams p, int mode) {
         for (int s = threadIdx.x; s < N; s += blockDim.x) jb[s] = r.jbits[s];
     __syncthreads();
 
-    uint32_t acc = 0;
+    unsigned long long acc = 0;
     if (mode == 0) {
         const uint32_t theta = r.stheta[i - 1];
         uint32_t thr[4];
@@ -408,8 +408,7 @@ __global__ void __launch_bounds__(NT) k_group(KParams p, int mode) {
     atomicAdd(&sU[lane], U);
     atomicAdd(&sNup[lane], nup);
     // accepted flips of the CTA
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0 && acc) atomicAdd(&sAcc, (unsigned long long)acc);
+    add_accepts(&sAcc, acc, lane);
     __syncthreads();
 
     if (warp == 0) {

@@ -191,8 +191,9 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
     const int span = p.qcap_limit >= 0 && p.qcap_limit < S2::QW ? U : H;
     __syncthreads();
 
-    uint32_t acc = 0;
+    unsigned long long accepts = 0;
     for (uint32_t h = 0; h < nh; ++h) {
+        uint32_t acc = 0;
         const uint32_t colour = h & 1u;
         if (h + 1 < nh) build_keys(h + 1);
         uint32_t* own = lat + gl * GS + colour * CS + y0 * S + xi;
@@ -316,6 +317,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
             }
             __syncwarp();
         }
+        accepts += acc;
         if constexpr (TG > 32) __syncthreads();
     }
     __syncthreads();
@@ -368,8 +370,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
         atomicAdd(&sU[g][lane], Uw);
         atomicAdd(&sNup[g][lane], nup);
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0 && acc) atomicAdd(&sums.acc, (unsigned long long)acc);
+    add_accepts(&sums.acc, accepts, lane);
     __syncthreads();
 
     if (G == 1 && warp > 0) return;  // one group: its warp adds to the trace itself

@@ -423,8 +423,9 @@ __global__ void __launch_bounds__(NT3, 6) k_sweep3d(KParams p, const uint32_t* c
     __syncthreads();
 
     const uint32_t lml = (1u << lane) - 1u;
-    uint32_t acc = 0;
+    unsigned long long accepts = 0;
     for (uint32_t h = 0; h < nh; ++h) {
+        uint32_t acc = 0;
         const int colour = (int)(h & 1u);
         if (h + 1 < nh) build_tables(h + 1);
         const uint2* ct = stab + colour * H;
@@ -509,6 +510,7 @@ __global__ void __launch_bounds__(NT3, 6) k_sweep3d(KParams p, const uint32_t* c
             __syncwarp();
             if (k == S::ITERS) break;
         }
+        accepts += acc;
         __syncthreads();
     }
 
@@ -554,8 +556,7 @@ __global__ void __launch_bounds__(NT3, 6) k_sweep3d(KParams p, const uint32_t* c
         atomicAdd(&sU[g][lane], U);
         atomicAdd(&sNup[g][lane], nup);
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0 && acc) atomicAdd(&sAcc, (unsigned long long)acc);
+    add_accepts(&sAcc, accepts, lane);
     __syncthreads();
 
     for (int g = warp; g < G; g += NW) {

@@ -15,6 +15,13 @@ __device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
     return d;
 }
 
+// Accepted flips of a CTA, from its threads' 64-bit counts (the walks count a half-sweep in 32
+// bits and add it up in 64: a step may have 2^24 sweeps).  Called by whole warps.
+__device__ __forceinline__ void add_accepts(unsigned long long* sum, unsigned long long a, int lane) {
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0 && a) atomicAdd(sum, a);
+}
+
 __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
     // lane i holds row i (bit c = element (i, c)); returns column `lane`
     const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};

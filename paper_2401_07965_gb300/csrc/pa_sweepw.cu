@@ -279,8 +279,9 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
     if (nh > 0) build_keys(0u);
     __syncthreads();
 
-    uint32_t acc = 0;
+    unsigned long long accepts = 0;
     for (uint32_t h = 0; h < nh; ++h) {
+        uint32_t acc = 0;
         const uint32_t colour = h & 1u;
         if (h + 1 < nh) build_keys(h + 1);
         const uint32_t par = ((uint32_t)yy + colour) & 1u;  // x parity of the column's first site
@@ -421,6 +422,7 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
             }
             __syncwarp();
         }
+        accepts += acc;
         if (local) __syncwarp();
         else __syncthreads();
     }
@@ -533,8 +535,7 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
                 make_uint4(out[0], out[1], out[2], out[3]);
         atomicAdd(&sNup[32 * g + lane], nup);
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0 && acc) atomicAdd(&sums.acc, (unsigned long long)acc);
+    add_accepts(&sums.acc, accepts, lane);
     __syncthreads();
 
     // a small lattice's levels are counted in the CTA first
