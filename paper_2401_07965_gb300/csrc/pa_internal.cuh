@@ -219,6 +219,15 @@ struct WalkPlan {
     int flat;         // nonzero: a side of pa_sweep3d.cu, GP groups per CTA
 };
 
+// The group (index within the CTA) whose block keys are entry q of a builder that has gpw
+// groups from `first` on in each of the plan's sets, or -1 for an entry past the set's last
+// group: the next set's first groups may belong to another warp, which no barrier orders.
+__host__ __device__ inline int walk_key_group(const WalkPlan& g, int gpw, int first, int q) {
+    const int c = q / gpw;
+    const int u = first + q - c * gpw;
+    return u < g.GP ? c * g.GP + u : -1;
+}
+
 // Batch-wide parameters, passed by value to every kernel.
 struct KParams {
     int d, ea, method, n_steps, M;

@@ -270,9 +270,8 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
             if (k < 8) {
                 bpart[8 * (hh & 1u) + k] = bp;
             } else {
-                const int q = (k - 8) >> 1, c = q / gpw;
-                const int g = c * GP + (local ? warp * gpw : 0) + q - c * gpw;
-                if (g < G) keys[2 * G * (hh & 1u) + 2 * g + b] = block_key_of(p, bp, sL0a[g]);
+                const int g = walk_key_group(pl, gpw, local ? warp * gpw : 0, (k - 8) >> 1);
+                if (g >= 0) keys[2 * G * (hh & 1u) + 2 * g + b] = block_key_of(p, bp, sL0a[g]);
             }
         }
     };
