@@ -25,6 +25,7 @@ namespace pa {
 namespace cg = cooperative_groups;
 
 constexpr int POP_CTAS = 16;
+constexpr int POP_LEVELS = 8192;  // entries of the level arrays, at most
 static_assert(SCAN_CHUNK == 2 * SCAN_THREADS && SCAN_THREADS == 256, "two adjacent replicas per thread");
 
 // the run's state and trace row after its weights (threads t < n of one CTA)
@@ -455,13 +456,16 @@ int pop_ctas(uint32_t most_R, int most_levels, int M, int method, int* threads, 
     if (most == 512) P = std::max(P, cs * nt);  // two words per level hold a prefix per replica
     *threads = nt;
     *levels = P;
-    return cs <= POP_CTAS && P <= 8192 && (int64_t)M * cs <= 128 ? cs : 0;
+    return cs <= POP_CTAS && P <= POP_LEVELS && (int64_t)M * cs <= 128 ? cs : 0;
 }
 
 template <int NT, bool PARTIAL>
 static cudaError_t launch(const KParams& p, cudaStream_t s) {
     const size_t sm = 2 * sizeof(double) * (size_t)p.pop_levels;
-    cudaError_t e = cudaFuncSetAttribute(k_pop<NT, PARTIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // the limit is the kernel's, whoever launches it: always the largest, so that a context on
+    // another thread never lowers it between this call and the launch
+    cudaError_t e = cudaFuncSetAttribute(k_pop<NT, PARTIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         2 * (int)sizeof(double) * POP_LEVELS);
     if (e == cudaSuccess && p.pop > 8)
         e = cudaFuncSetAttribute(k_pop<NT, PARTIAL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;

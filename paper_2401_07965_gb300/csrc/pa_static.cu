@@ -41,6 +41,7 @@ __device__ __forceinline__ double pow_sq(const double* qsq, uint32_t k) {
 
 constexpr int STATIC_SMEM_TREE = 2048;  // tree entries that fit the smallest shared array
 constexpr int STATIC_SMEM_MIN = STATIC_SMEM_TREE * 8;
+constexpr int STATIC_SMEM_MAX = (3 * 32768 / 2 + 1) * 4;  // the counts of the most levels (3D, N = 32768)
 
 // Level counts over all CTAs; the last CTA to finish (a ticket) turns them into S, ln Q
 // and the fixed-point weights of the levels and leaves the counts at zero.  With one CTA
@@ -227,9 +228,10 @@ extern "C" pa_status pa_weights_static(const int32_t* E, uint32_t R_prev, uint32
     const uint32_t per = 4 * STATIC_THREADS;
     const unsigned na = (unsigned)std::min<uint64_t>(((uint64_t)R_prev + per - 1) / per, 152u);
     const int sm = std::max(STATIC_SMEM_MIN, (int)(dim * N / 2 + 1) * 4);  // at most 197 KB
+    // (always the largest limit: another thread's call must not lower it before this launch)
     if (sm > 48 * 1024 - 512 &&
-        cudaFuncSetAttribute(k_static_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, sm) !=
-            cudaSuccess)
+        cudaFuncSetAttribute(k_static_weights, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             STATIC_SMEM_MAX) != cudaSuccess)
         return PA_ERR_CUDA;
     k_static_weights<<<na, STATIC_THREADS, sm, st>>>(sc, E, R_prev, R, dim, (int)N, parity, dbeta, q,
                                                      lnQ, na == 1 ? f : nullptr);

@@ -1,0 +1,56 @@
+"""What the library's host code asks the CUDA runtime for, on a stand-in for it (no GPU)."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from tests import fake_runtime
+
+
+@pytest.fixture
+def pa():
+    return fake_runtime.load()
+
+
+def _run(pa, L, R, rule="systematic", dim=2, priority=0, steps=40, graph=True):
+    return pa.Batch([{"dim": dim, "L": L, "R": R}], np.linspace(0.0, 1.0, steps + 1),
+                    np.full(steps, 2, np.uint32), rule, 1, graph=graph, use_torch_memory=False,
+                    stream=fake_runtime.Stream(pa._lib, priority))
+
+
+@pytest.mark.parametrize("small,large", [((16, 500), (64, 500)), ((16, 500), (16, 8000))])
+def test_one_launch_resampling_beside_another_context(pa, small, large):
+    """Two contexts on two host threads: a step of one comes between the other's attribute calls
+    and its launch, at every one of them."""
+    a, b = _run(pa, *large, rule="multinomial", graph=False), _run(pa, *small, rule="multinomial",
+                                                                   graph=False)
+    inside = []
+
+    @C.CFUNCTYPE(None)
+    def other_thread():
+        if not inside:
+            inside.append(1)
+            b.step(1)
+            inside.pop()
+
+    pa._lib.fake_attr_hook(other_thread)
+    a.step(1)
+    pa._lib.fake_attr_hook(None)
+    names = [x["name"] for x in fake_runtime.launches(pa._lib)]
+    assert sum("k_pop" in n for n in names) > 1
+
+
+def test_static_weights_beside_another_call(pa):
+    buf = np.zeros(64, np.int64).ctypes.data
+    inside = []
+
+    @C.CFUNCTYPE(None)
+    def other_thread():
+        if not inside:
+            inside.append(1)
+            pa.pa_weights_static(buf, 10, 10, 2, 114, 0, 0.01, buf, buf, 0)
+            inside.pop()
+
+    pa._lib.fake_attr_hook(other_thread)
+    pa.pa_weights_static(buf, 10, 10, 3, 32, 0, 0.01, buf, buf, 0)
+    pa._lib.fake_attr_hook(None)
