@@ -507,15 +507,8 @@ static size_t group_smem(const KParams& p) {
 
 template <int D, bool EA, int NT>
 static cudaError_t prepare_nt() {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_group<D, EA, NT>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             200 * 1024);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    return cudaSuccess;
+    return cudaFuncSetAttribute(k_group<D, EA, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                200 * 1024);
 }
 
 template <int D, bool EA, int NT>
@@ -555,7 +548,8 @@ static cudaError_t prepare_t(int threads) {
     }
 }
 
-// one-time function attributes, outside any stream capture
+// The function attributes, before a stream capture.  Every launch sets its kernel's as well:
+// they belong to the device that is current, and the same constants are set each time.
 cudaError_t prepare_sweep(const KParams& p, int threads) {
     bool done = false;
     cudaError_t e = launch_sweep2d(p, nullptr, true, &done);

@@ -402,15 +402,10 @@ cudaError_t launch2d(const KParams& p, const uint32_t* cta2run, uint32_t ncta, c
     constexpr size_t sm = Shape2<L, NT, G, EA>::SMEM;
     static_assert(sm <= smem2d_max(G), "2D sweep shared memory");
     constexpr int MINB = 65536 / (NT * 96);
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_sweep2d<L, NT, G, EA, MINB>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem2d_max(G));
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    if (attr_only || ncta == 0) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(k_sweep2d<L, NT, G, EA, MINB>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem2d_max(G));
+    if (e != cudaSuccess || attr_only || ncta == 0) return e;
     return launch_chained(k_sweep2d<L, NT, G, EA, MINB>, ncta, (unsigned)NT,
                           spread_smem(sm, ncta, NT, NT == 512 ? 128 : 96), s, p, cta2run);
 }

@@ -609,15 +609,10 @@ size_t smem3d() {
 template <int L, bool EA, int GM>
 cudaError_t launch3d(const KParams& p, const uint32_t* cta2run, uint32_t ncta, cudaStream_t s,
                      bool attr_only) {
-    static bool attr_set = false;
     const size_t sm = smem3d<L, EA, GM>();
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_sweep3d<L, EA, GM>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    if (attr_only || ncta == 0) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_sweep3d<L, EA, GM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess || attr_only || ncta == 0) return e;
     k_sweep3d<L, EA, GM><<<ncta, NT3, sm, s>>>(p, cta2run);
     return cudaGetLastError();
 }

@@ -565,14 +565,9 @@ constexpr int WALK_SMEM_MAX = 227 * 1024 - 1024;
 template <int D, int LT, bool EA>
 cudaError_t launch_walk_t(const KParams& p, const WalkPlan& g, const uint32_t* cta2run,
                           uint32_t ncta, cudaStream_t s, bool attr_only) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(
-            k_walk<D, LT, EA>, cudaFuncAttributeMaxDynamicSharedMemorySize, WALK_SMEM_MAX);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
-    if (attr_only || ncta == 0) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_walk<D, LT, EA>, cudaFuncAttributeMaxDynamicSharedMemorySize, WALK_SMEM_MAX);
+    if (e != cudaSuccess || attr_only || ncta == 0) return e;
     const size_t sm = spread_smem((size_t)walk_smem(g, D, EA).total, ncta, g.NT, 96);
     return launch_chained(k_walk<D, LT, EA>, ncta, (unsigned)g.NT, sm, s, p, g, cta2run);
 }

@@ -54,3 +54,23 @@ def test_static_weights_beside_another_call(pa):
     pa._lib.fake_attr_hook(other_thread)
     pa.pa_weights_static(buf, 10, 10, 3, 32, 0, 0.01, buf, buf, 0)
     pa._lib.fake_attr_hook(None)
+
+
+@pytest.mark.parametrize("dim,L,R,ea", [(2, 16, 1000, False), (2, 64, 3000, True),
+                                        (2, 24, 1000, False), (3, 6, 1000, True),
+                                        (3, 10, 1000, True), (2, [4, 6, 8, 10, 100], 100, True)])
+def test_every_device_of_a_process(pa, dim, L, R, ea):
+    """A run on a second device, after one of the same shape on the first: function attributes
+    are a device's own."""
+    pa._lib.fake_reset(2)
+    sides = L if isinstance(L, list) else [L]
+    for dev in (0, 1, 0):
+        pa._lib.fake_set_device(dev)
+        first = pa._lib.fake_launches()
+        b = pa.Batch([{"dim": dim, "L": s, "R": R, "couplings": ("ea", 3, 1) if ea else ("ferro",)}
+                      for s in sides], np.linspace(0.0, 1.0, 5), np.full(4, 2, np.uint32),
+                     "systematic", 1, use_torch_memory=False, stream=fake_runtime.Stream(pa._lib))
+        b.step(2)
+        new = fake_runtime.launches(pa._lib, first)
+        assert len(new) >= 4 and all(x["device"] == dev for x in new)
+        b.close()
