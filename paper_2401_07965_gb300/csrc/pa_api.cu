@@ -79,6 +79,7 @@ struct pa_ctx {
     cudaGraphExec_t graph[2] = {};          // one captured step, GRAPH_STEPS of them
     int graph_threads = 0;
     int64_t graph_kernels[2] = {};
+    int device = 0;                         // current at pa_init; the captures' too
     cudaStream_t cap = nullptr, side = nullptr;  // the captured step and its branch
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::vector<cudaEvent_t> ev_start, ev_stop;  // pool of timing events, reused
@@ -534,9 +535,22 @@ uint32_t run_theta(const pa_ctx* ctx, int run, int i) {
     return ctx->controlled ? ctx->rtheta[run][i] : ctx->theta[i];
 }
 
-// capture one temperature step (many = 0) or GRAPH_STEPS of them; every kernel reads the
-// step index and the population sizes from device memory, so the same graph serves every step
+// Capture one temperature step (many = 0) or GRAPH_STEPS of them; every kernel reads the
+// step index and the population sizes from device memory, so the same graph serves every step.
+// The context's device is current meanwhile: a graph is launched whatever device is.
+struct DeviceScope {
+    int before = 0;
+    cudaError_t e;
+    explicit DeviceScope(int device) {
+        e = cudaGetDevice(&before);
+        if (e == cudaSuccess && before != device) e = cudaSetDevice(device);
+    }
+    ~DeviceScope() { cudaSetDevice(before); }
+};
+
 pa_status build_graph(pa_ctx* ctx, int many) {
+    const DeviceScope scope(ctx->device);
+    PA_CUDA(scope.e);
     PA_CUDA(prepare_sweep(ctx->kp, ctx->threads));
     if (!ctx->side) {
         int least = 0, greatest = 0;
@@ -635,6 +649,7 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
     ctx->method = (int)resampler;
     ctx->seed = seed;
     ctx->stream = (cudaStream_t)cuda_stream;
+    cudaGetDevice(&ctx->device);
     ctx->beta.assign(sched->beta, sched->beta + n + 1);
     ctx->theta.assign(sched->theta, sched->theta + n);
     int maxN = 0;

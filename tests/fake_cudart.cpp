@@ -72,6 +72,7 @@ void fake_reset(int n_devices) {  // the attributes stay, as a process keeps the
     attr_hook = nullptr;
 }
 void fake_set_device(int d) { device = d; }
+int fake_device() { return device; }
 void fake_static_smem(const char* part, int bytes) { static_smem[part] = bytes; }
 void fake_clusters_fit(int n) { clusters_fit = n; }
 void fake_attr_hook(void (*f)()) { attr_hook = f; }

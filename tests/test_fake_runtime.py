@@ -74,3 +74,18 @@ def test_every_device_of_a_process(pa, dim, L, R, ea):
         new = fake_runtime.launches(pa._lib, first)
         assert len(new) >= 4 and all(x["device"] == dev for x in new)
         b.close()
+
+
+@pytest.mark.parametrize("n", [1, 16])
+def test_steps_with_another_device_current(pa, n):
+    """A captured step is launched whatever device is current; a longer call, which captures
+    several steps, must not need the context's own one either."""
+    pa._lib.fake_reset(2)
+    pa._lib.fake_set_device(0)
+    b = _run(pa, 16, 1000)
+    b.step(1)
+    pa._lib.fake_set_device(1)
+    first = pa._lib.fake_launches()
+    b.step(n)
+    assert all(x["device"] == 0 for x in fake_runtime.launches(pa._lib, first))
+    assert pa._lib.fake_device() == 1
