@@ -317,7 +317,8 @@ cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int
 cudaError_t prepare_sweep(const KParams& p, int threads);
 cudaError_t launch_sweep2d(const KParams& p, cudaStream_t s, bool attr_only, bool* done);
 double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT);
-size_t spread_smem(size_t sm, uint32_t ncta, int nt, int regs);
+size_t spread_smem(const void* kernel, size_t sm, uint32_t ncta, int nt, int regs);
+cudaError_t family_attributes(cudaFuncAttributes* a);
 int sweep3d_groups(int L, int gm);
 cudaError_t launch_sweep3d(const KParams& p, int L, int G, const uint32_t* cta2run, uint32_t ncta,
                            cudaStream_t s, bool attr_only);

@@ -476,16 +476,23 @@ double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT) {
 }
 
 // Dynamic shared memory for a sweep launch of ncta CTAs of nt threads (regs registers each)
-// that need sm bytes.  A launch that the 152 SMs hold at once ends with its fullest SM, and
-// beside another kernel (the family branch) its CTAs are not spread evenly: it asks for so
-// much that no SM takes more than its share (+-J L = 48, 626 CTAs where 7 fit an SM: the
-// step 249 us without, 227 us with the limit), less 8 KB for the other kernel.
-size_t spread_smem(size_t sm, uint32_t ncta, int nt, int regs) {
-    constexpr size_t SM_BYTES = 227 * 1024, FIXED = 2560;  // static part and the system's
-    const size_t fit = std::min<size_t>(65536 / (size_t)(nt * regs), SM_BYTES / (sm + FIXED));
-    const size_t want = (ncta + 151) / 152;
-    if (want == 0 || want >= fit) return sm;
-    return std::max(sm, std::min<size_t>((SM_BYTES - 8192) / want - FIXED, SM_BYTES - 8192 - FIXED));
+// of `kernel` that need sm bytes.  A launch that the 152 SMs hold at once ends with its fullest
+// SM, and beside another kernel (the family branch) its CTAs are not spread evenly: it asks for
+// so much that no SM takes more than its share (+-J L = 48, 626 CTAs where 7 fit an SM: the
+// step 249 us without, 227 us with the limit), less the room of a CTA of the family kernel.
+// The share must still fit: a CTA takes the kernel's static part and 1 KB of the system's, too.
+// (want + 1 CTAs with their needs fit an SM and want + 1 < 22, so the share is never below sm.)
+size_t spread_smem(const void* kernel, size_t sm, uint32_t ncta, int nt, int regs) {
+    constexpr size_t SM_BYTES = 228 * 1024, SYSTEM = 1024;
+    cudaFuncAttributes at, family;
+    const size_t want = (ncta + 151) / 152, by_regs = 65536 / (size_t)(nt * regs);
+    if (want == 0 || want >= by_regs || cudaFuncGetAttributes(&at, kernel) != cudaSuccess ||
+        family_attributes(&family) != cudaSuccess)
+        return sm;
+    const size_t fixed = at.sharedSizeBytes + SYSTEM;
+    if (want >= SM_BYTES / (sm + fixed)) return sm;
+    const size_t share = (SM_BYTES - family.sharedSizeBytes - SYSTEM) / want & ~(size_t)127;
+    return std::max(sm, std::min(share - fixed, (size_t)at.maxDynamicSharedSizeBytes));
 }
 
 int sweep_threads(int N) {

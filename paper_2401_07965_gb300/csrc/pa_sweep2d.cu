@@ -407,7 +407,9 @@ cudaError_t launch2d(const KParams& p, const uint32_t* cta2run, uint32_t ncta, c
                                                (int)smem2d_max(G));
     if (e != cudaSuccess || attr_only || ncta == 0) return e;
     return launch_chained(k_sweep2d<L, NT, G, EA, MINB>, ncta, (unsigned)NT,
-                          spread_smem(sm, ncta, NT, NT == 512 ? 128 : 96), s, p, cta2run);
+                          spread_smem((const void*)k_sweep2d<L, NT, G, EA, MINB>, sm, ncta, NT,
+                                      NT == 512 ? 128 : 96),
+                          s, p, cta2run);
 }
 
 template <int L, int NT, int G>

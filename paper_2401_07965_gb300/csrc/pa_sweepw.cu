@@ -568,7 +568,8 @@ cudaError_t launch_walk_t(const KParams& p, const WalkPlan& g, const uint32_t* c
     const cudaError_t e = cudaFuncSetAttribute(
         k_walk<D, LT, EA>, cudaFuncAttributeMaxDynamicSharedMemorySize, WALK_SMEM_MAX);
     if (e != cudaSuccess || attr_only || ncta == 0) return e;
-    const size_t sm = spread_smem((size_t)walk_smem(g, D, EA).total, ncta, g.NT, 96);
+    const size_t sm = spread_smem((const void*)k_walk<D, LT, EA>,
+                                  (size_t)walk_smem(g, D, EA).total, ncta, g.NT, 96);
     return launch_chained(k_walk<D, LT, EA>, ncta, (unsigned)g.NT, sm, s, p, g, cta2run);
 }
 

@@ -44,10 +44,14 @@ int static_of(const void* f) {
     return 0;
 }
 
+int limit_of(const void* f) {  // of the dynamic shared memory, on the current device
+    const auto lim = smem_limit.find({device, f});
+    return lim == smem_limit.end() ? 48 * 1024 - static_of(f) : lim->second;
+}
+
 cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, cudaStream_t s, unsigned cluster) {
     std::lock_guard<std::recursive_mutex> l(mu);
-    const auto lim = smem_limit.find({device, f});
-    const int most = lim == smem_limit.end() ? 48 * 1024 - static_of(f) : lim->second;
+    const int most = limit_of(f);
     Stream* st = stream_of(s);
     if (st && st->device != device) return cudaErrorInvalidResourceHandle;
     if ((long long)smem > most) return cudaErrorInvalidValue;
@@ -137,6 +141,7 @@ cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
 cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* a, const void* f) {
     std::memset(a, 0, sizeof(*a));
     a->sharedSizeBytes = (size_t)static_of(f);
+    a->maxDynamicSharedSizeBytes = limit_of(f);
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t*) {

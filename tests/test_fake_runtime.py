@@ -89,3 +89,41 @@ def test_steps_with_another_device_current(pa, n):
     b.step(n)
     assert all(x["device"] == 0 for x in fake_runtime.launches(pa._lib, first))
     assert pa._lib.fake_device() == 1
+
+
+SM_BYTES, SYSTEM = 228 * 1024, 1024  # shared memory of an SM; the system's part of every CTA
+
+
+@pytest.mark.parametrize("threads,groups,static", [(64, 16, 8512), (128, 8, 4416), (256, 4, 2368),
+                                                   (512, 1, 832)])
+def test_padded_sweeps_still_fit_their_share(pa, threads, groups, static):
+    """A sweep launch that the 152 SMs hold at once asks for more shared memory than it needs, so
+    that no SM takes more CTAs than ceil(CTAs / 152).  That many must fit an SM with the kernel's
+    static part, and a CTA of the family kernel beside them."""
+    family = 8816
+    pa._lib.fake_static_smem(b"k_sweep2d", static)
+    pa._lib.fake_static_smem(b"k_family", family)
+
+    def sweep(R):
+        b = _run(pa, 16, R, graph=False)
+        pa.pa_set_sweep_threads(b.ctx, threads)
+        first = pa._lib.fake_launches()
+        b.step(1)
+        x = [y for y in fake_runtime.launches(pa._lib, first) if "k_sweep2d" in y["name"]]
+        b.close()
+        assert len(x) == 1 and x[0]["grid"] == -(-R // (32 * groups))
+        return x[0]
+
+    per_cta = lambda x: x["smem"] + static + SYSTEM
+    need = sweep(32 * groups * 152 * 24)  # more than one round: what the kernel needs
+    by_regs = 65536 // (96 * need["block"])
+    raised = 0
+    for share in range(1, 12):
+        x = sweep(32 * groups * 152 * share - 100)
+        if share >= min(by_regs, SM_BYTES // per_cta(need)):
+            assert x["smem"] == need["smem"]
+            continue
+        raised += 1
+        assert share * per_cta(x) + family + SYSTEM <= SM_BYTES  # they fit, the family's beside
+        assert (share + 1) * per_cta(x) > SM_BYTES               # and no more of them
+    assert raised >= 2
