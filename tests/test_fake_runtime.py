@@ -127,3 +127,18 @@ def test_padded_sweeps_still_fit_their_share(pa, threads, groups, static):
         assert share * per_cta(x) + family + SYSTEM <= SM_BYTES  # they fit, the family's beside
         assert (share + 1) * per_cta(x) > SM_BYTES               # and no more of them
     assert raised >= 2
+
+
+@pytest.mark.parametrize("priority", [0, -1, -5])
+@pytest.mark.parametrize("R", [1000, 100000])  # one launch for the resampling, several
+def test_the_callers_stream_priority(pa, priority, R):
+    """Captured kernels have the priority of the caller's stream; the family branch is never above
+    it."""
+    b = _run(pa, 16, R, priority=priority)
+    first = pa._lib.fake_launches()
+    b.step(1)
+    new = fake_runtime.launches(pa._lib, first)
+    for x in new:
+        want = min(priority + 1, 0) if "k_family" in x["name"] else priority
+        assert x["priority"] == want, x
+    assert any("k_sweep2d" in x["name"] and x["captured"] for x in new)
