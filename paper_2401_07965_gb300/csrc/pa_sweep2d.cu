@@ -191,9 +191,11 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
     const int span = p.qcap_limit >= 0 && p.qcap_limit < S2::QW ? U : H;
     __syncthreads();
 
+    constexpr bool SPANS = L >= 64;  // how accepted flips go to 64 bits (add_accepts)
     unsigned long long accepts = 0;
-    for (uint32_t h = 0; h < nh; ++h) {
-        uint32_t acc = 0;
+    uint32_t acc = 0;
+    for (uint32_t h = 0; h < nh;) {
+    for (const uint32_t h1 = SPANS ? min(nh, h + ACC_SPAN) : nh; h < h1; ++h) {
         const uint32_t colour = h & 1u;
         if (h + 1 < nh) build_keys(h + 1);
         uint32_t* own = lat + gl * GS + colour * CS + y0 * S + xi;
@@ -317,8 +319,16 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
             }
             __syncwarp();
         }
-        accepts += acc;
+        if constexpr (!SPANS) {
+            accepts += acc;
+            acc = 0;
+        }
         if constexpr (TG > 32) __syncthreads();
+    }
+    if constexpr (SPANS) {
+        add_accepts(&sums.acc, acc, lane);
+        acc = 0;
+    }
     }
     __syncthreads();
 
@@ -370,7 +380,7 @@ __global__ void __launch_bounds__(NT, MINB) k_sweep2d(KParams p, const uint32_t*
         atomicAdd(&sU[g][lane], Uw);
         atomicAdd(&sNup[g][lane], nup);
     }
-    add_accepts(&sums.acc, accepts, lane);
+    if constexpr (!SPANS) add_accepts(&sums.acc, accepts, lane);
     __syncthreads();
 
     if (G == 1 && warp > 0) return;  // one group: its warp adds to the trace itself

@@ -423,9 +423,9 @@ __global__ void __launch_bounds__(NT3, 6) k_sweep3d(KParams p, const uint32_t* c
     __syncthreads();
 
     const uint32_t lml = (1u << lane) - 1u;
-    unsigned long long accepts = 0;
-    for (uint32_t h = 0; h < nh; ++h) {
-        uint32_t acc = 0;
+    uint32_t acc = 0;
+    for (uint32_t h = 0; h < nh;) {
+    for (const uint32_t h1 = min(nh, h + ACC_SPAN); h < h1; ++h) {
         const int colour = (int)(h & 1u);
         if (h + 1 < nh) build_tables(h + 1);
         const uint2* ct = stab + colour * H;
@@ -510,8 +510,10 @@ __global__ void __launch_bounds__(NT3, 6) k_sweep3d(KParams p, const uint32_t* c
             __syncwarp();
             if (k == S::ITERS) break;
         }
-        accepts += acc;
         __syncthreads();
+    }
+    add_accepts(&sAcc, acc, lane);
+    acc = 0;
     }
 
     // measurement: unsatisfied bonds U and up-count per replica, write back
@@ -556,7 +558,6 @@ __global__ void __launch_bounds__(NT3, 6) k_sweep3d(KParams p, const uint32_t* c
         atomicAdd(&sU[g][lane], U);
         atomicAdd(&sNup[g][lane], nup);
     }
-    add_accepts(&sAcc, accepts, lane);
     __syncthreads();
 
     for (int g = warp; g < G; g += NW) {

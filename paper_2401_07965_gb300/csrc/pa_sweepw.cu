@@ -278,9 +278,9 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
     if (nh > 0) build_keys(0u);
     __syncthreads();
 
-    unsigned long long accepts = 0;
-    for (uint32_t h = 0; h < nh; ++h) {
-        uint32_t acc = 0;
+    uint32_t acc = 0;
+    for (uint32_t h = 0; h < nh;) {
+    for (const uint32_t h1 = min(nh, h + ACC_SPAN); h < h1; ++h) {
         const uint32_t colour = h & 1u;
         if (h + 1 < nh) build_keys(h + 1);
         const uint32_t par = ((uint32_t)yy + colour) & 1u;  // x parity of the column's first site
@@ -421,9 +421,11 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
             }
             __syncwarp();
         }
-        accepts += acc;
         if (local) __syncwarp();
         else __syncthreads();
+    }
+    add_accepts(&sums.acc, acc, lane);
+    acc = 0;
     }
     __syncthreads();
 
@@ -534,7 +536,6 @@ __global__ void __launch_bounds__(640) k_walk(const __grid_constant__ KParams p,
                 make_uint4(out[0], out[1], out[2], out[3]);
         atomicAdd(&sNup[32 * g + lane], nup);
     }
-    add_accepts(&sums.acc, accepts, lane);
     __syncthreads();
 
     // a small lattice's levels are counted in the CTA first
