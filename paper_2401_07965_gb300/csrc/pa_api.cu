@@ -479,9 +479,9 @@ pa_status enqueue_step(pa_ctx* ctx, int64_t* launches, cudaStream_t stream,
     if (side) {
         PA_CUDA(cudaEventRecord(ctx->ev_fork, stream));
         PA_CUDA(cudaStreamWaitEvent(side, ctx->ev_fork, 0));
+    } else {
+        PA_CUDA(launch_family_finish(ctx->kp, 0, stream, launches));
     }
-    PA_CUDA(launch_family_finish(ctx->kp, 0, side ? side : stream, launches));
-    if (side) PA_CUDA(cudaEventRecord(ctx->ev_join, side));
     const bool timed = ctx->timing && !side;
     if (timed) {
         if (ctx->ev_used == ctx->ev_start.size()) {
@@ -493,6 +493,10 @@ pa_status enqueue_step(pa_ctx* ctx, int64_t* launches, cudaStream_t stream,
     PA_CUDA(launch_sweep(ctx->kp, ctx->threads, stream));
     if (launches) *launches += 1;
     if (timed) PA_CUDA(cudaEventRecord(ctx->ev_stop[ctx->ev_used++], stream));
+    if (side) {  // captured after the sweep: its CTAs come second where both are ready
+        PA_CUDA(launch_family_finish(ctx->kp, 0, side, launches));
+        PA_CUDA(cudaEventRecord(ctx->ev_join, side));
+    }
     if (ctx->kp.alpha >= 0.0) PA_CUDA(launch_weighted_sums(ctx->kp, 0, stream, launches));
     if (side) PA_CUDA(cudaStreamWaitEvent(stream, ctx->ev_join, 0));
     if (ctx->kp.ctl) {
@@ -565,8 +569,8 @@ pa_status build_graph(pa_ctx* ctx, int many) {
     cudaGraph_t g = nullptr;
     // Captured on streams of the context's own, whose priorities go to the kernels: the
     // caller's, and for the family branch the next lower one where there is one.  (With one
-    // priority for both a step takes as long as with the sweep above the branch: its padded
-    // CTAs spread evenly beside it.  With the branch after the sweep it takes 11 us more.)
+    // priority for both a step takes as long as with the sweep above the branch; with the
+    // branch in line after the sweep it takes 11 us more.)
     PA_CUDA(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
     int64_t n = 0;
     pa_status s = PA_OK;

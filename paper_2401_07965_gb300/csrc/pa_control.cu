@@ -412,7 +412,7 @@ pa_status pa_mlp_gradients(const float* params, const float* X, const float* Yt,
         : rows <= 64 ? launch_grad<64>(params, X, Yt, mask, B, rows, nb, norm, part, s)
                      : launch_grad<96>(params, X, Yt, mask, B, rows, nb, norm, part, s);
     if (e != cudaSuccess) return PA_ERR_CUDA;
-    return launch_chained(k_mlp_reduce, (MLP_NPARAM + 1 + 31) / 32, 256u, 0, s, part, (int)nb, grads,
+    return launch_chained(true, k_mlp_reduce, (MLP_NPARAM + 1 + 31) / 32, 256u, 0, s, part, (int)nb, grads,
                           loss) == cudaSuccess
                ? PA_OK
                : PA_ERR_CUDA;

@@ -287,8 +287,8 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
-                           cudaStream_t s, A... args) {
+cudaError_t launch_chained(bool chain, void (*kernel)(P...), unsigned grid, unsigned block,
+                           size_t smem, cudaStream_t s, A... args) {
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
@@ -298,7 +298,7 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, 
     c.dynamicSmemBytes = smem;
     c.stream = s;
     c.attrs = &at;
-    c.numAttrs = 1;
+    c.numAttrs = chain ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
@@ -315,17 +315,15 @@ cudaError_t launch_partial_init(const KParams& p, cudaStream_t s);
 cudaError_t launch_sweep(const KParams& p, int threads, cudaStream_t s);
 cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int64_t* launches);
 cudaError_t prepare_sweep(const KParams& p, int threads);
-cudaError_t launch_sweep2d(const KParams& p, cudaStream_t s, bool attr_only, bool* done);
+cudaError_t launch_sweep2d(const KParams& p, cudaStream_t s, bool attr_only, bool chain, bool* done);
 double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT);
-size_t spread_smem(const void* kernel, size_t sm, uint32_t ncta, int nt, int regs);
-cudaError_t family_attributes(cudaFuncAttributes* a);
 int sweep3d_groups(int L, int gm);
 cudaError_t launch_sweep3d(const KParams& p, int L, int G, const uint32_t* cta2run, uint32_t ncta,
                            cudaStream_t s, bool attr_only);
 int sweep2d_threads(int L, int threads, uint32_t ngrp);
 WalkPlan walk_plan(int d, int L, bool ea, uint32_t ngrp, uint32_t most_grp, int threads, int gm);
 cudaError_t launch_walk(const KParams& p, const WalkPlan& g, const uint32_t* cta2run, uint32_t ncta,
-                        cudaStream_t s, bool attr_only);
+                        cudaStream_t s, bool attr_only, bool chain);
 cudaError_t launch_control(const KParams& p, cudaStream_t s);
 int sweep_threads(int N);
 bool sweep_threads_supported(int t);

@@ -171,7 +171,7 @@ cudaError_t launch_overlap(const KParams& p, const int32_t* pairs, int n_pairs, 
         k_overlap_hist<false><<<grid, 256, 0, s>>>(p, pairs, G, bins, hist, acc, tickets);
     e = cudaGetLastError();
     if (e != cudaSuccess || !P) return e;
-    return launch_chained(k_overlap_P, (unsigned)((bins + OVP_T - 1) / OVP_T), (unsigned)OVP_T, 0, s, p,
+    return launch_chained(true, k_overlap_P, (unsigned)((bins + OVP_T - 1) / OVP_T), (unsigned)OVP_T, 0, s, p,
                           pairs, n_pairs, bins, (const uint32_t*)hist, P);
 }
 

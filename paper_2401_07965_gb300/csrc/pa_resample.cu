@@ -1079,8 +1079,6 @@ cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int
     return cudaGetLastError();
 }
 
-cudaError_t family_attributes(cudaFuncAttributes* a) { return cudaFuncGetAttributes(a, k_family); }
-
 cudaError_t launch_weighted_sums(const KParams& p, int mode, cudaStream_t s, int64_t* launches) {
     k_wsums<<<p.nblk_total, SCAN_THREADS, 0, s>>>(p, mode == 0 && !pop_takes(p));
     if (launches) *launches += 1;

@@ -237,7 +237,7 @@ extern "C" pa_status pa_weights_static(const int32_t* E, uint32_t R_prev, uint32
                                                      lnQ, na == 1 ? f : nullptr);
     if (na == 1) return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
     const unsigned nf = (unsigned)std::min<uint64_t>(((uint64_t)R_prev + 1023u) / 1024u, 152u * 8u);
-    return pa::launch_chained(k_static_f, nf, 256u, 0, st, sc, E, R_prev, dim * (int)N, f) == cudaSuccess
+    return pa::launch_chained(true, k_static_f, nf, 256u, 0, st, sc, E, R_prev, dim * (int)N, f) == cudaSuccess
                ? PA_OK
                : PA_ERR_CUDA;
 }

@@ -475,24 +475,14 @@ double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT) {
     return t / er * nt / (GP * tg);
 }
 
-// Dynamic shared memory for a sweep launch of ncta CTAs of nt threads (regs registers each)
-// of `kernel` that need sm bytes.  A launch that the 152 SMs hold at once ends with its fullest
-// SM, and beside another kernel (the family branch) its CTAs are not spread evenly: it asks for
-// so much that no SM takes more than its share (+-J L = 48, 626 CTAs where 7 fit an SM: the
-// step 249 us without, 227 us with the limit), less the room of a CTA of the family kernel.
-// The share must still fit: a CTA takes the kernel's static part and 1 KB of the system's, too.
-// (want + 1 CTAs with their needs fit an SM and want + 1 < 22, so the share is never below sm.)
-size_t spread_smem(const void* kernel, size_t sm, uint32_t ncta, int nt, int regs) {
-    constexpr size_t SM_BYTES = 228 * 1024, SYSTEM = 1024;
-    cudaFuncAttributes at, family;
-    const size_t want = (ncta + 151) / 152, by_regs = 65536 / (size_t)(nt * regs);
-    if (want == 0 || want >= by_regs || cudaFuncGetAttributes(&at, kernel) != cudaSuccess ||
-        family_attributes(&family) != cudaSuccess)
-        return sm;
-    const size_t fixed = at.sharedSizeBytes + SYSTEM;
-    if (want >= SM_BYTES / (sm + fixed)) return sm;
-    const size_t share = (SM_BYTES - family.sharedSizeBytes - SYSTEM) / want & ~(size_t)127;
-    return std::max(sm, std::min(share - fixed, (size_t)at.maxDynamicSharedSizeBytes));
+// Whether a sweep launch of ncta CTAs is chained to k_pop, that is, placed while k_pop's CTAs
+// still hold their SMs: only where the other SMs hold the sweep at an even share each.
+// Otherwise some SMs would get more than their share and hold the launch (L = 32, R = 4500, 141
+// CTAs on 152 SMs: 47.5 us a step chained, 36.6 not; L = 16, R = 9000, 282 CTAs, 18 of
+// k_pop: 33.8 and 32.5; where it fits, as for L = 16, R = 1000, a step is 1 us shorter chained).
+static bool chain_sweep(const KParams& p, uint32_t ncta) {
+    const uint32_t share = (ncta + 151) / 152;  // of an SM
+    return !pop_takes(p) || ncta + share * (uint32_t)(p.M * p.pop) <= share * 152;
 }
 
 int sweep_threads(int N) {
@@ -559,10 +549,10 @@ static cudaError_t prepare_t(int threads) {
 // they belong to the device that is current, and the same constants are set each time.
 cudaError_t prepare_sweep(const KParams& p, int threads) {
     bool done = false;
-    cudaError_t e = launch_sweep2d(p, nullptr, true, &done);
+    cudaError_t e = launch_sweep2d(p, nullptr, true, false, &done);
     if (e != cudaSuccess) return e;
     for (int k = 0; k < p.nw && e == cudaSuccess; ++k)
-        e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], nullptr, true);
+        e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], nullptr, true, false);
     if (e != cudaSuccess) return e;
     if (p.d == 2) return p.ea ? prepare_t<2, true>(threads) : prepare_t<2, false>(threads);
     return p.ea ? prepare_t<3, true>(threads) : prepare_t<3, false>(threads);
@@ -587,11 +577,12 @@ cudaError_t launch_sweep(const KParams& p, int threads, cudaStream_t s) {
     if (p.nw > 0) {  // the column walk: one launch per side
         cudaError_t e = cudaSuccess;
         for (int k = 0; k < p.nw && e == cudaSuccess; ++k)
-            e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], s, false);
+            e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], s, false,
+                            k > 0 || chain_sweep(p, p.wcta[k]));
         return e;
     }
     bool done = false;
-    const cudaError_t e = launch_sweep2d(p, s, false, &done);
+    const cudaError_t e = launch_sweep2d(p, s, false, chain_sweep(p, p.wcta[0]), &done);
     if (e != cudaSuccess || done) return e;
     return launch_group(p, 0, threads, s);
 }

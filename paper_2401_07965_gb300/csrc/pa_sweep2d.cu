@@ -408,7 +408,7 @@ constexpr size_t smem2d_max(int G) { return 227 * 1024 - 2048 - 520 * (size_t)G;
 
 template <int L, int NT, int G, bool EA>
 cudaError_t launch2d(const KParams& p, const uint32_t* cta2run, uint32_t ncta, cudaStream_t s,
-                     bool attr_only) {
+                     bool attr_only, bool chain) {
     constexpr size_t sm = Shape2<L, NT, G, EA>::SMEM;
     static_assert(sm <= smem2d_max(G), "2D sweep shared memory");
     constexpr int MINB = 65536 / (NT * 96);
@@ -416,16 +416,14 @@ cudaError_t launch2d(const KParams& p, const uint32_t* cta2run, uint32_t ncta, c
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)smem2d_max(G));
     if (e != cudaSuccess || attr_only || ncta == 0) return e;
-    return launch_chained(k_sweep2d<L, NT, G, EA, MINB>, ncta, (unsigned)NT,
-                          spread_smem((const void*)k_sweep2d<L, NT, G, EA, MINB>, sm, ncta, NT,
-                                      NT == 512 ? 128 : 96),
-                          s, p, cta2run);
+    return launch_chained(chain, k_sweep2d<L, NT, G, EA, MINB>, ncta, (unsigned)NT, sm, s, p,
+                          cta2run);
 }
 
 template <int L, int NT, int G>
-cudaError_t launch2d_ea(const KParams& p, cudaStream_t s, bool attr_only) {
-    return p.ea ? launch2d<L, NT, G, true>(p, p.wmap[0], p.wcta[0], s, attr_only)
-                : launch2d<L, NT, G, false>(p, p.wmap[0], p.wcta[0], s, attr_only);
+cudaError_t launch2d_ea(const KParams& p, cudaStream_t s, bool attr_only, bool chain) {
+    return p.ea ? launch2d<L, NT, G, true>(p, p.wmap[0], p.wcta[0], s, attr_only, chain)
+                : launch2d<L, NT, G, false>(p, p.wmap[0], p.wcta[0], s, attr_only, chain);
 }
 
 }  // namespace
@@ -458,24 +456,24 @@ int sweep2d_threads(int L, int threads, uint32_t ngrp) {
 // The 2D kernel for runs that all have the same power-of-two side L (16..128); *done =
 // false when the plan has none.  attr_only: set the kernel's function attributes only
 // (before a stream capture).
-cudaError_t launch_sweep2d(const KParams& p, cudaStream_t s, bool attr_only, bool* done) {
+cudaError_t launch_sweep2d(const KParams& p, cudaStream_t s, bool attr_only, bool chain, bool* done) {
     *done = p.G2 > 0;
     if (!*done) return cudaSuccess;
     switch (p.L_all * 1000 + p.TG2) {
-        case 16008: return launch2d_ea<16, 128, 16>(p, s, attr_only);
-        case 16016: return launch2d_ea<16, 128, 8>(p, s, attr_only);
-        case 16032: return launch2d_ea<16, 128, 4>(p, s, attr_only);
-        case 16064: return launch2d_ea<16, 64, 1>(p, s, attr_only);
-        case 16128: return launch2d_ea<16, 128, 1>(p, s, attr_only);
-        case 32032: return launch2d_ea<32, 128, 4>(p, s, attr_only);
-        case 32064: return launch2d_ea<32, 64, 1>(p, s, attr_only);
-        case 32128: return launch2d_ea<32, 128, 1>(p, s, attr_only);
-        case 32256: return launch2d_ea<32, 256, 1>(p, s, attr_only);
-        case 64128: return launch2d_ea<64, 128, 1>(p, s, attr_only);
-        case 64256: return launch2d_ea<64, 256, 1>(p, s, attr_only);
-        case 64512: return launch2d_ea<64, 512, 1>(p, s, attr_only);
-        case 128256: return launch2d_ea<128, 256, 1>(p, s, attr_only);
-        default: return launch2d_ea<128, 512, 1>(p, s, attr_only);
+        case 16008: return launch2d_ea<16, 128, 16>(p, s, attr_only, chain);
+        case 16016: return launch2d_ea<16, 128, 8>(p, s, attr_only, chain);
+        case 16032: return launch2d_ea<16, 128, 4>(p, s, attr_only, chain);
+        case 16064: return launch2d_ea<16, 64, 1>(p, s, attr_only, chain);
+        case 16128: return launch2d_ea<16, 128, 1>(p, s, attr_only, chain);
+        case 32032: return launch2d_ea<32, 128, 4>(p, s, attr_only, chain);
+        case 32064: return launch2d_ea<32, 64, 1>(p, s, attr_only, chain);
+        case 32128: return launch2d_ea<32, 128, 1>(p, s, attr_only, chain);
+        case 32256: return launch2d_ea<32, 256, 1>(p, s, attr_only, chain);
+        case 64128: return launch2d_ea<64, 128, 1>(p, s, attr_only, chain);
+        case 64256: return launch2d_ea<64, 256, 1>(p, s, attr_only, chain);
+        case 64512: return launch2d_ea<64, 512, 1>(p, s, attr_only, chain);
+        case 128256: return launch2d_ea<128, 256, 1>(p, s, attr_only, chain);
+        default: return launch2d_ea<128, 512, 1>(p, s, attr_only, chain);
     }
 }
 

@@ -565,24 +565,23 @@ constexpr int WALK_SMEM_MAX = 227 * 1024 - 1024;
 
 template <int D, int LT, bool EA>
 cudaError_t launch_walk_t(const KParams& p, const WalkPlan& g, const uint32_t* cta2run,
-                          uint32_t ncta, cudaStream_t s, bool attr_only) {
+                          uint32_t ncta, cudaStream_t s, bool attr_only, bool chain) {
     const cudaError_t e = cudaFuncSetAttribute(
         k_walk<D, LT, EA>, cudaFuncAttributeMaxDynamicSharedMemorySize, WALK_SMEM_MAX);
     if (e != cudaSuccess || attr_only || ncta == 0) return e;
-    const size_t sm = spread_smem((const void*)k_walk<D, LT, EA>,
-                                  (size_t)walk_smem(g, D, EA).total, ncta, g.NT, 96);
-    return launch_chained(k_walk<D, LT, EA>, ncta, (unsigned)g.NT, sm, s, p, g, cta2run);
+    return launch_chained(chain, k_walk<D, LT, EA>, ncta, (unsigned)g.NT,
+                          (size_t)walk_smem(g, D, EA).total, s, p, g, cta2run);
 }
 
 template <bool EA>
 cudaError_t launch_walk_ea(const KParams& p, const WalkPlan& g, const uint32_t* cta2run,
-                           uint32_t ncta, cudaStream_t s, bool attr_only) {
-    if (p.d == 2) return launch_walk_t<2, 0, EA>(p, g, cta2run, ncta, s, attr_only);
+                           uint32_t ncta, cudaStream_t s, bool attr_only, bool chain) {
+    if (p.d == 2) return launch_walk_t<2, 0, EA>(p, g, cta2run, ncta, s, attr_only, chain);
     switch (g.L) {
-        case 4: return launch_walk_t<3, 4, EA>(p, g, cta2run, ncta, s, attr_only);
-        case 6: return launch_walk_t<3, 6, EA>(p, g, cta2run, ncta, s, attr_only);
-        case 8: return launch_walk_t<3, 8, EA>(p, g, cta2run, ncta, s, attr_only);
-        default: return launch_walk_t<3, 0, EA>(p, g, cta2run, ncta, s, attr_only);
+        case 4: return launch_walk_t<3, 4, EA>(p, g, cta2run, ncta, s, attr_only, chain);
+        case 6: return launch_walk_t<3, 6, EA>(p, g, cta2run, ncta, s, attr_only, chain);
+        case 8: return launch_walk_t<3, 8, EA>(p, g, cta2run, ncta, s, attr_only, chain);
+        default: return launch_walk_t<3, 0, EA>(p, g, cta2run, ncta, s, attr_only, chain);
     }
 }
 
@@ -684,10 +683,10 @@ WalkPlan walk_plan(int d, int L, bool ea, uint32_t ngrp, uint32_t most_grp, int 
 // One launch of the walk over the CTAs of the runs of one side (cta2run: their run
 // indices, device memory).  attr_only: function attributes only (before a capture).
 cudaError_t launch_walk(const KParams& p, const WalkPlan& g, const uint32_t* cta2run, uint32_t ncta,
-                        cudaStream_t s, bool attr_only) {
+                        cudaStream_t s, bool attr_only, bool chain) {
     if (g.flat) return launch_sweep3d(p, g.L, g.GP, cta2run, ncta, s, attr_only);
-    return p.ea ? launch_walk_ea<true>(p, g, cta2run, ncta, s, attr_only)
-                : launch_walk_ea<false>(p, g, cta2run, ncta, s, attr_only);
+    return p.ea ? launch_walk_ea<true>(p, g, cta2run, ncta, s, attr_only, chain)
+                : launch_walk_ea<false>(p, g, cta2run, ncta, s, attr_only, chain);
 }
 
 }  // namespace pa

@@ -22,7 +22,7 @@ struct Launch {
     unsigned grid, block, cluster;
     size_t smem;
     int device, priority;
-    bool captured;
+    bool captured, chained;
 };
 
 std::recursive_mutex mu;
@@ -49,7 +49,8 @@ int limit_of(const void* f) {  // of the dynamic shared memory, on the current d
     return lim == smem_limit.end() ? 48 * 1024 - static_of(f) : lim->second;
 }
 
-cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, cudaStream_t s, unsigned cluster) {
+cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, cudaStream_t s, unsigned cluster,
+                   bool chained) {
     std::lock_guard<std::recursive_mutex> l(mu);
     const int most = limit_of(f);
     Stream* st = stream_of(s);
@@ -57,7 +58,7 @@ cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, cudaStream_t s, u
     if ((long long)smem > most) return cudaErrorInvalidValue;
     if (cluster > 8 && clusters_fit == 0) return cudaErrorLaunchOutOfResources;
     launches.push_back({names[f], g.x, b.x, cluster, smem, device, st ? st->priority : 0,
-                        st && st->capturing});
+                        st && st->capturing, chained});
     return cudaSuccess;
 }
 
@@ -82,13 +83,14 @@ void fake_clusters_fit(int n) { clusters_fit = n; }
 void fake_attr_hook(void (*f)()) { attr_hook = f; }
 void* fake_stream(int priority) { return new Stream{priority, device, false}; }
 int fake_launches() { return (int)launches.size(); }
-// field of launch k: 0 grid, 1 block, 2 cluster, 3 shared memory, 4 device, 5 priority, 6 captured
+// field of launch k: 0 grid, 1 block, 2 cluster, 3 shared memory, 4 device, 5 priority, 6 captured,
+// 7 chained
 long long fake_launch(int k, int field, char* name, int room) {
     const Launch& x = launches[k];
     std::strncpy(name, x.name.c_str(), room - 1);
     name[room - 1] = 0;
-    const long long v[7] = {x.grid, x.block, x.cluster, (long long)x.smem, x.device, x.priority,
-                            x.captured};
+    const long long v[8] = {x.grid, x.block, x.cluster, (long long)x.smem, x.device, x.priority,
+                            x.captured, x.chained};
     return v[field];
 }
 
@@ -120,14 +122,17 @@ cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) {
     return cudaSuccess;
 }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void**, size_t sm, cudaStream_t s) {
-    return last = launch((const void*)k, g, b, sm, s, 1);
+    return last = launch((const void*)k, g, b, sm, s, 1, false);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
     unsigned cluster = 1;
+    bool chained = false;
     for (unsigned k = 0; k < c->numAttrs; ++k)
         if (c->attrs[k].id == cudaLaunchAttributeClusterDimension)
             cluster = c->attrs[k].val.clusterDim.x;
-    return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, c->stream, cluster);
+        else if (c->attrs[k].id == cudaLaunchAttributeProgrammaticStreamSerialization)
+            chained = c->attrs[k].val.programmaticStreamSerializationAllowed != 0;
+    return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, c->stream, cluster, chained);
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
     if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) {

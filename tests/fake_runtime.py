@@ -10,7 +10,7 @@ import tempfile
 
 from paper_2401_07965_gb300 import build
 
-FIELDS = ("grid", "block", "cluster", "smem", "device", "priority", "captured")
+FIELDS = ("grid", "block", "cluster", "smem", "device", "priority", "captured", "chained")
 _binding = None
 
 

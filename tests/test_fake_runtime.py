@@ -91,42 +91,42 @@ def test_steps_with_another_device_current(pa, n):
     assert pa._lib.fake_device() == 1
 
 
-SM_BYTES, SYSTEM = 228 * 1024, 1024  # shared memory of an SM; the system's part of every CTA
-
-
-@pytest.mark.parametrize("threads,groups,static", [(64, 16, 8512), (128, 8, 4416), (256, 4, 2368),
-                                                   (512, 1, 832)])
-def test_padded_sweeps_still_fit_their_share(pa, threads, groups, static):
-    """A sweep launch that the 152 SMs hold at once asks for more shared memory than it needs, so
-    that no SM takes more CTAs than ceil(CTAs / 152).  That many must fit an SM with the kernel's
-    static part, and a CTA of the family kernel beside them."""
-    family = 8816
-    pa._lib.fake_static_smem(b"k_sweep2d", static)
-    pa._lib.fake_static_smem(b"k_family", family)
-
+@pytest.mark.parametrize("dim,L,threads", [(2, 16, 64), (2, 16, 128), (2, 16, 512), (2, 32, 256),
+                                           (2, 64, 128), (2, 48, 128)])
+def test_small_sweeps_leave_room_for_others(pa, dim, L, threads):
+    """A sweep launch asks for the shared memory it needs whatever its number of CTAs, so that
+    contexts on other streams share the SMs with it."""
     def sweep(R):
-        b = _run(pa, 16, R, graph=False)
+        b = _run(pa, L, R, dim=dim, graph=False)
         pa.pa_set_sweep_threads(b.ctx, threads)
         first = pa._lib.fake_launches()
         b.step(1)
-        x = [y for y in fake_runtime.launches(pa._lib, first) if "k_sweep2d" in y["name"]]
+        x = [y for y in fake_runtime.launches(pa._lib, first)
+             if "k_sweep2d" in y["name"] or "k_walk" in y["name"]]
         b.close()
-        assert len(x) == 1 and x[0]["grid"] == -(-R // (32 * groups))
+        assert len(x) == 1
         return x[0]
 
-    per_cta = lambda x: x["smem"] + static + SYSTEM
-    need = sweep(32 * groups * 152 * 24)  # more than one round: what the kernel needs
-    by_regs = 65536 // (96 * need["block"])
-    raised = 0
-    for share in range(1, 12):
-        x = sweep(32 * groups * 152 * share - 100)
-        if share >= min(by_regs, SM_BYTES // per_cta(need)):
-            assert x["smem"] == need["smem"]
-            continue
-        raised += 1
-        assert share * per_cta(x) + family + SYSTEM <= SM_BYTES  # they fit, the family's beside
-        assert (share + 1) * per_cta(x) > SM_BYTES               # and no more of them
-    assert raised >= 2
+    many = sweep(500000)
+    same = [x for x in map(sweep, (1000, 4800, 9000, 20000, 60000, 150000))
+            if (x["name"], x["block"]) == (many["name"], many["block"])]
+    assert len(same) >= 1 and all(x["smem"] == many["smem"] for x in same)
+
+
+@pytest.mark.parametrize("L,R", [(16, 1000), (16, 4800), (32, 2000), (32, 4500), (32, 9500),
+                                 (64, 10000), (24, 4500), (16, 60000)])
+def test_sweeps_chained_to_the_one_launch_resampling(pa, L, R):
+    """A sweep is placed while the one-launch resampling holds its SMs only where the others hold
+    it at an even share each."""
+    b = _run(pa, L, R)
+    first = pa._lib.fake_launches()
+    b.step(1)
+    new = fake_runtime.launches(pa._lib, first)
+    x = [y for y in new if "k_sweep2d" in y["name"] or "k_walk" in y["name"]]
+    pop = sum(y["grid"] for y in new if "k_pop" in y["name"])
+    assert len(x) == 1
+    share = -(-x[0]["grid"] // 152)
+    assert x[0]["chained"] == (pop == 0 or x[0]["grid"] <= share * (152 - pop))
 
 
 @pytest.mark.parametrize("priority", [0, -1, -5])
