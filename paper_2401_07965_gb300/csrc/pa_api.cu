@@ -421,7 +421,7 @@ void plan_sweep(pa_ctx* ctx, int gm, uint32_t* map, std::vector<uint32_t>& c3) {
                 all += (uint32_t)h.ngrp;
                 most = std::max(most, (uint32_t)h.ngrp);
             }
-        p.wplan[k] = walk_plan(p.d, L, p.ea != 0, all, most, want, gm);
+        p.wplan[k] = walk_plan(p.d, L, p.ea != 0, all, most, want, ctx->threads, gm);
         place(L, p.wplan[k].GP * p.wplan[k].CPT, &p.wmap[k], &p.wcta[k]);
     }
 }

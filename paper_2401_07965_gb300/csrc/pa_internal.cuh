@@ -216,7 +216,7 @@ struct WalkPlan {
     int NT;           // threads
     int span;         // rows walked before the second pass (fewer than H: the list's room)
     uint32_t mL, sL;  // division by L
-    int flat;         // nonzero: a side of pa_sweep3d.cu, GP groups per CTA
+    int flat;         // > 0: a side of pa_sweep3d.cu, GP groups per CTA; -1: k_group takes the side
 };
 
 // The group (index within the CTA) whose block keys are entry q of a builder that has gpw
@@ -316,12 +316,14 @@ cudaError_t launch_sweep(const KParams& p, int threads, cudaStream_t s);
 cudaError_t launch_family_finish(const KParams& p, int mode, cudaStream_t s, int64_t* launches);
 cudaError_t prepare_sweep(const KParams& p, int threads);
 cudaError_t launch_sweep2d(const KParams& p, cudaStream_t s, bool attr_only, bool chain, bool* done);
-double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT);
+double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT, size_t smem,
+                  double alone);
 int sweep3d_groups(int L, int gm);
 cudaError_t launch_sweep3d(const KParams& p, int L, int G, const uint32_t* cta2run, uint32_t ncta,
                            cudaStream_t s, bool attr_only);
 int sweep2d_threads(int L, int threads, uint32_t ngrp);
-WalkPlan walk_plan(int d, int L, bool ea, uint32_t ngrp, uint32_t most_grp, int threads, int gm);
+double group_time(int d, int N, bool ea, uint32_t ngrp, int threads);
+WalkPlan walk_plan(int d, int L, bool ea, uint32_t ngrp, uint32_t most_grp, int threads, int general, int gm);
 cudaError_t launch_walk(const KParams& p, const WalkPlan& g, const uint32_t* cta2run, uint32_t ncta,
                         cudaStream_t s, bool attr_only, bool chain);
 cudaError_t launch_control(const KParams& p, cudaStream_t s);

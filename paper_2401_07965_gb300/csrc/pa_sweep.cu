@@ -205,11 +205,12 @@ __host__ __device__ __forceinline__ int queue_capacity(int N) {
 // mode 1: measurement of the current population only (init / restore).
 // ---------------------------------------------------------------------------
 template <int D, bool EA, int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_group(KParams p, int mode) {
+__global__ void __launch_bounds__(NT) k_group(KParams p, int mode, int only) {
     extern __shared__ __align__(16) uint32_t smem[];
     // the CTA's run and its replica group within the run; the flattened CTA
     // index is the global replica group of the sweep draws
     const RunDesc& r = p.runs[p.grp2run[blockIdx.x]];
+    if (only > 0 && r.L != only) return;  // the launch for one side of a batch
     const Geo geo = {r.L, r.N, r.magicL, r.shiftL};
     uint32_t* ms = smem;
     uint8_t* jb = reinterpret_cast<uint8_t*>(smem + r.N);
@@ -264,7 +265,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_group(KParams p, int 
         for (int s = threadIdx.x; s < N; s += blockDim.x) jb[s] = r.jbits[s];
     __syncthreads();
 
-    unsigned long long acc = 0;
+    uint32_t acc = 0;
     if (mode == 0) {
         const uint32_t theta = r.stheta[i - 1];
         uint32_t thr[4];
@@ -292,7 +293,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_group(KParams p, int 
             qn[1] = 0;
         }
         __syncthreads();
-        for (uint32_t h = 0; h < nh; ++h) {
+        for (uint32_t h = 0; h < nh;) {
+        for (const uint32_t h1 = min(nh, h + ACC_SPAN); h < h1; ++h) {
             const int colour = (int)(h & 1u);
             // the table of the next half-sweep goes to the other buffer
             if (h + 1 < nh && threadIdx.x < 8)
@@ -356,6 +358,9 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_group(KParams p, int 
             }
             __syncthreads();
         }
+        add_accepts(&sAcc, acc, lane);
+        acc = 0;
+        }
     }
 
     // measurement: unsatisfied bonds U and up-count per replica, write back
@@ -407,8 +412,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_group(KParams p, int 
     }
     atomicAdd(&sU[lane], U);
     atomicAdd(&sNup[lane], nup);
-    // accepted flips of the CTA
-    add_accepts(&sAcc, acc, lane);
     __syncthreads();
 
     if (warp == 0) {
@@ -451,28 +454,35 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_group(KParams p, int 
 }
 
 // Relative time of a column-walk sweep of ngrp groups with tg threads of `regs` registers
-// each, GP groups side by side in a CTA and CPT sets of them one after the other, and
-// `rows` rows per thread between two second passes.  An SM
+// each, GP groups side by side in a CTA and CPT sets of them one after the other, `rows` rows
+// per thread between two second passes and smem bytes of shared memory per CTA.  An SM
 // with w warps per scheduler works at the rate w / (w + 1.6); up to three rounds of the
 // groups that the 152 SMs hold take as long as the rounds of the fullest SM, more take the
 // average load and a part of a round; lanes past the last column and few rows cost their
-// share: few rows leave the second pass's rounds part empty and repeat its set-up.  Fitted
-// to 2D L = 32, 625 groups (16, 8, 4, 2 rows: 1737, 2423, 2762, 2247 updates/ns) and 3125
+// share: few rows leave the second pass's rounds part empty and repeat its set-up.  A CTA that
+// has nothing beside it on its SM when it waits at its barriers takes `alone` times as long.
+// Fitted to 2D L = 32, 625 groups (16, 8, 4, 2 rows: 1737, 2423, 2762, 2247 updates/ns) and 3125
 // groups (3490, 3877, 3725) and L = 64, 94 groups (16, 8, 4 rows: 1243, 1823, 1919), 625
-// (3329, 3208, 2640) and 3125 (4669, 4352, 3512); it takes the best of each.
-double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT) {
+// (3329, 3208, 2640) and 3125 (4669, 4352, 3512), where it takes the best of each.  Over all
+// plans of 17 other 2D and 6 3D sides, 32 to 6250 groups, its choice is 1.6% slower than the
+// best one on average, 15% at most (4.3% and 57% without the shared memory: L = 54, 2813
+// groups 1184 us a step, 742 with it).
+double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT, size_t smem,
+                  double alone) {
     const double er = rows >= 16 ? 1.0 : rows >= 12 ? 0.97 : rows >= 8 ? 0.93 : rows >= 6 ? 0.9
                       : rows >= 4 ? 0.85 : rows >= 2 ? 0.65 : 0.45;
     const int G = GP * CPT, nt = std::max(32, (GP * tg + 31) / 32 * 32);
-    // groups an SM holds: each of its four schedulers has registers for whole warps
-    const int hold = std::max(1, 4 * (16384 / (32 * regs)) / (nt / 32)) * G;
+    // groups an SM holds: each of its four schedulers has registers for whole warps; a CTA's
+    // shared memory with 2 KB for the static part and the system's
+    const int by_regs = 4 * (16384 / (32 * regs)) / (nt / 32), by_smem = (int)(228 * 1024 / (smem + 2048));
+    const int ctas = std::max(1, std::min(by_regs, by_smem)), hold = ctas * G;
     const int ncta = (int)((ngrp + G - 1) / G);
     const int most = std::min<int>((ncta + 151) / 152 * G, (int)ngrp);
     auto round = [&](double n) { return n > 0.0 ? n + 1.6 * 128.0 * CPT / tg : 0.0; };  // n at once
     const double t = most <= 3 * hold
                          ? most / hold * round(hold) + round(most % hold)
                          : (ngrp / 152.0 + 0.3 * hold) * round(hold) / hold;
-    return t / er * nt / (GP * tg);
+    return t / er * nt / (GP * tg) * (std::min(ctas, (ncta + 151) / 152) == 1 ? alone : 1.0);
 }
 
 // Whether a sweep launch of ncta CTAs is chained to k_pop, that is, placed while k_pop's CTAs
@@ -496,10 +506,17 @@ bool sweep_threads_supported(int t) {
     return t == 64 || t == 128 || t == 256 || t == 384 || t == 512;
 }
 
-static size_t group_smem(const KParams& p) {
-    const size_t words_per_entry = 7 + (size_t)p.d;
-    return (size_t)p.maxN * 4 + (p.ea ? (size_t)((p.maxN + 15) / 16) * 16 : 0) +
-           words_per_entry * 4 * (size_t)queue_capacity(p.maxN);
+static size_t group_smem(int d, int N, bool ea) {
+    const size_t words_per_entry = 7 + (size_t)d;
+    return (size_t)N * 4 + (ea ? (size_t)((N + 15) / 16) * 16 : 0) +
+           words_per_entry * 4 * (size_t)queue_capacity(N);
+}
+
+// k_group's time in the units of sweep_time(): its site costs 1.35 times the walk's (the best of
+// 1.25 to 1.45 over the 2D sides 4 to 160 and 32 to 4688 groups that both kernels ran)
+double group_time(int d, int N, bool ea, uint32_t ngrp, int threads) {
+    return 1.35 * sweep_time(N / 2 / threads, ngrp, 1, threads, 64, 1, group_smem(d, N, ea) + 1552,
+                            1.0);
 }
 
 template <int D, bool EA, int NT>
@@ -509,29 +526,30 @@ static cudaError_t prepare_nt() {
 }
 
 template <int D, bool EA, int NT>
-static cudaError_t launch_group_nt(const KParams& p, int mode, cudaStream_t s) {
+static cudaError_t launch_group_nt(const KParams& p, int mode, int only, cudaStream_t s) {
     cudaError_t e = prepare_nt<D, EA, NT>();
     if (e != cudaSuccess) return e;
-    k_group<D, EA, NT><<<p.ngrp_total, NT, group_smem(p), s>>>(p, mode);
+    k_group<D, EA, NT><<<p.ngrp_total, NT, group_smem(p.d, p.maxN, p.ea != 0), s>>>(p, mode, only);
     return cudaGetLastError();
 }
 
 template <int D, bool EA>
-static cudaError_t launch_group_t(const KParams& p, int mode, int threads, cudaStream_t s) {
+static cudaError_t launch_group_t(const KParams& p, int mode, int only, int threads, cudaStream_t s) {
     switch (threads) {
-        case 64: return launch_group_nt<D, EA, 64>(p, mode, s);
-        case 128: return launch_group_nt<D, EA, 128>(p, mode, s);
-        case 384: return launch_group_nt<D, EA, 384>(p, mode, s);
-        case 512: return launch_group_nt<D, EA, 512>(p, mode, s);
-        default: return launch_group_nt<D, EA, 256>(p, mode, s);
+        case 64: return launch_group_nt<D, EA, 64>(p, mode, only, s);
+        case 128: return launch_group_nt<D, EA, 128>(p, mode, only, s);
+        case 384: return launch_group_nt<D, EA, 384>(p, mode, only, s);
+        case 512: return launch_group_nt<D, EA, 512>(p, mode, only, s);
+        default: return launch_group_nt<D, EA, 256>(p, mode, only, s);
     }
 }
 
-static cudaError_t launch_group(const KParams& p, int mode, int threads, cudaStream_t s) {
-    if (p.d == 2) return p.ea ? launch_group_t<2, true>(p, mode, threads, s)
-                              : launch_group_t<2, false>(p, mode, threads, s);
-    return p.ea ? launch_group_t<3, true>(p, mode, threads, s)
-                : launch_group_t<3, false>(p, mode, threads, s);
+// only: the runs of that side (0: all)
+static cudaError_t launch_group(const KParams& p, int mode, int only, int threads, cudaStream_t s) {
+    if (p.d == 2) return p.ea ? launch_group_t<2, true>(p, mode, only, threads, s)
+                              : launch_group_t<2, false>(p, mode, only, threads, s);
+    return p.ea ? launch_group_t<3, true>(p, mode, only, threads, s)
+                : launch_group_t<3, false>(p, mode, only, threads, s);
 }
 
 template <int D, bool EA>
@@ -552,7 +570,8 @@ cudaError_t prepare_sweep(const KParams& p, int threads) {
     cudaError_t e = launch_sweep2d(p, nullptr, true, false, &done);
     if (e != cudaSuccess) return e;
     for (int k = 0; k < p.nw && e == cudaSuccess; ++k)
-        e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], nullptr, true, false);
+        if (p.wplan[k].flat >= 0)
+            e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], nullptr, true, false);
     if (e != cudaSuccess) return e;
     if (p.d == 2) return p.ea ? prepare_t<2, true>(threads) : prepare_t<2, false>(threads);
     return p.ea ? prepare_t<3, true>(threads) : prepare_t<3, false>(threads);
@@ -570,21 +589,22 @@ cudaError_t launch_init_spins(const KParams& p, const RunDesc* host_runs, cudaSt
 }
 
 cudaError_t launch_measure(const KParams& p, int threads, cudaStream_t s) {
-    return launch_group(p, 1, threads, s);
+    return launch_group(p, 1, 0, threads, s);
 }
 
 cudaError_t launch_sweep(const KParams& p, int threads, cudaStream_t s) {
-    if (p.nw > 0) {  // the column walk: one launch per side
+    if (p.nw > 0) {  // one launch per side
         cudaError_t e = cudaSuccess;
         for (int k = 0; k < p.nw && e == cudaSuccess; ++k)
-            e = launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], s, false,
-                            k > 0 || chain_sweep(p, p.wcta[k]));
+            e = p.wplan[k].flat < 0 ? launch_group(p, 0, p.wplan[k].L, threads, s)
+                                    : launch_walk(p, p.wplan[k], p.wmap[k], p.wcta[k], s, false,
+                                                  k > 0 || chain_sweep(p, p.wcta[k]));
         return e;
     }
     bool done = false;
     const cudaError_t e = launch_sweep2d(p, s, false, chain_sweep(p, p.wcta[0]), &done);
     if (e != cudaSuccess || done) return e;
-    return launch_group(p, 0, threads, s);
+    return launch_group(p, 0, 0, threads, s);
 }
 
 }  // namespace pa

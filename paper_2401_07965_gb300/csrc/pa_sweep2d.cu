@@ -442,7 +442,7 @@ int sweep2d_threads(int L, int threads, uint32_t ngrp) {
         int best = tg[k][0];
         double top = 1e30;
         for (int t : tg[k]) {
-            const double v = sweep_time(L * L / 2 / t, ngrp, t <= 32 ? 128 / t : 1, t, t == 512 ? 128 : 96, 1);
+            const double v = sweep_time(L * L / 2 / t, ngrp, t <= 32 ? 128 / t : 1, t, t == 512 ? 128 : 96, 1, 0, 1.0);
             if (v < top) {
                 top = v;
                 best = t;

@@ -17,10 +17,10 @@ __device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
 
 // Accepted flips of a CTA in 64 bits: a step may have 2^24 sweeps.  A thread counts ACC_SPAN
 // half-sweeps in 32 bits (it makes at most 2^14 flips in one) and its warp calls this after
-// each span; k_sweep2d below L = 64 adds each half-sweep to a 64-bit count instead, and
-// k_group counts in 64 bits.  (Time against one 32-bit count: the outer loop over the spans
-// -1.3% in k_walk, 0 at L = 64, +2.3% at L = 32; the 64-bit count +2 to 4% in k_walk, +0.8%
-// at L = 64, +0.5% at L = 32.)
+// each span; k_sweep2d below L = 64 adds each half-sweep to a 64-bit count instead.  (Time
+// against one 32-bit count: the outer loop over the spans -1.3% in k_walk, 0 at L = 64 and in
+// k_group, +2.3% at L = 32; a 64-bit count +2 to 4% in k_walk, +2% in k_group, +0.8% at L = 64,
+// +0.5% at L = 32.)
 constexpr uint32_t ACC_SPAN = 1u << 16;
 __device__ __forceinline__ void add_accepts(unsigned long long* sum, unsigned long long a, int lane) {
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);

@@ -585,13 +585,14 @@ cudaError_t launch_walk_ea(const KParams& p, const WalkPlan& g, const uint32_t* 
     }
 }
 
-void finish_plan(WalkPlan& g, int d, bool ea) {
+// the plan's strides for its columns, groups, sets and span; returns its shared memory
+int finish_plan(WalkPlan& g, int d, bool ea) {
     const int L = g.L, TPR = L / 2;
+    g.NT = (g.GP * g.NC + 31) / 32 * 32;
     auto size = [&](int S) {
         g.S = S;
         g.CS = walk_cs(L * S);
         g.GS = 2 * g.CS + ((g.NC - 2 * g.CS) % 32 + 32) % 32;
-        g.span = g.H;
         return walk_smem(g, d, ea).total;
     };
     // 2D chunks of a warp on distinct banks, where a stride does it and there is room
@@ -602,22 +603,22 @@ void finish_plan(WalkPlan& g, int d, bool ea) {
                 if (size(t) <= WALK_SMEM_MAX) S = t;
                 break;
             }
-    // the list holds every site of a pass: fewer rows per pass where it would not fit
-    size(S);
-    while (g.span > 4 && walk_smem(g, d, ea).total > WALK_SMEM_MAX) g.span = (g.span / 2 + 3) & ~3;
+    return size(S);
 }
 
 }  // namespace
 
 // The walk's geometry for the runs of side L of a context: ngrp replica groups in all,
-// at most most_grp in one run; threads per group wanted (0: the rule's own choice).
+// at most most_grp in one run; threads per group wanted (0: the rule's own choice); general:
+// the threads k_group would have.  The least sweep_time() of the plans that fit:
 //  - columns: 3D all L^2/2 of a group; 2D L/2 times the number of chunks, a divisor of L
-//    with an even chunk height: the least sweep_time() (with the groups side by side),
-//    or the most columns that stay within `threads`;
-//  - groups side by side and sets of them: the least sweep_time(), with up to about 14
-//    rows per thread between two second passes (a small lattice's column has 4 to 8;
-//    L = 4: up to 2 sets, more cost residency); gm doubles the sets.
-WalkPlan walk_plan(int d, int L, bool ea, uint32_t ngrp, uint32_t most_grp, int threads, int gm) {
+//    with an even chunk height (a wish takes the most columns that stay within `threads`);
+//  - groups side by side, up to about 320 threads, and sets of them, up to about 14 rows per
+//    thread between two second passes (a small lattice's column has 4 to 8; L = 4: up to 2
+//    sets, more cost residency); gm doubles the sets;
+//  - the span, rows between two second passes: the list takes 8 bytes for every site of a span,
+//    the lattice 4 for every site, so a long column's list costs CTAs of an SM.
+WalkPlan walk_plan(int d, int L, bool ea, uint32_t ngrp, uint32_t most_grp, int threads, int general, int gm) {
     WalkPlan g;
     std::memset(&g, 0, sizeof(g));
     const int TPR = L / 2;
@@ -628,51 +629,68 @@ WalkPlan walk_plan(int d, int L, bool ea, uint32_t ngrp, uint32_t most_grp, int 
         g.CPT = 1;
         return g;
     }
-    int NCH = 1, GP2 = 0;
-    double top = 1e30;
-    if (d == 2)
+    WalkPlan best = g;
+    double least = 1e30;
+    auto columns = [&](int n) {
+        g.NC = d == 3 ? TPR * L : TPR * n;
+        g.H = d == 3 ? L : L / n;
+    };
+    auto consider = [&](int gp, int cpt) {
+        g.GP = gp;
+        g.CPT = cpt * gm;
+        for (g.span = g.H;; g.span = (g.span / 2 + 1) & ~1) {
+            const int sm = finish_plan(g, d, ea);
+            if (sm <= WALK_SMEM_MAX) {
+                const int rows = g.H / ((g.H + g.span - 1) / g.span) * cpt;
+                const double t = sweep_time(rows, ngrp, gp, g.NC, regs, cpt, (size_t)sm, 1.15);
+                if (t < least - 1e-9) {
+                    least = t;
+                    best = g;
+                }
+            }
+            if (g.span <= 4) break;
+        }
+    };
+    // all that fit beside each other, with every number of sets
+    auto consider_all = [&](int widest) {
+        const int most = std::min<int>((int)std::min<uint32_t>(most_grp, 512u), 512 / g.NC);
+        const int sets = L == 4 && d == 3 ? 2 : std::max(1, (14 + g.H / 2) / g.H);
+        for (int cpt = 1; cpt <= sets; ++cpt)
+            for (int gp = 1; gp == 1 || (gp <= most && (d == 3 || gp <= 16) && gp * g.NC <= widest); ++gp) consider(gp, cpt);
+    };
+    if (d == 3) {
+        columns(1);
+        consider_all(352);
+    } else {
+        int wish = 1;
         for (int n = 1; n <= L / 2 && TPR * n <= 512; ++n) {
             if (L % n != 0 || (L / n) % 2 != 0) continue;
             if (threads > 0) {
-                if (TPR * n <= threads) NCH = n;
+                if (TPR * n <= threads) wish = n;
                 continue;
             }
-            for (int gp = 1; gp <= 16 && gp * TPR * n <= 320; ++gp) {
-                const double v = sweep_time(L / n, ngrp, gp, TPR * n, regs, 1);
-                if (v < top - 1e-9) {
-                    top = v;
-                    NCH = n;
-                    GP2 = gp;
-                }
-            }
+            columns(n);
+            consider_all(320);
         }
-    g.NC = d == 3 ? TPR * L : TPR * NCH;
-    g.H = d == 3 ? L : L / NCH;
-    const int most = std::max(1, std::min<int>((int)std::min<uint32_t>(most_grp, 512u), 512 / g.NC));
-    g.CPT = L == 4 && d == 3 ? 2 : std::max(1, (14 + g.H / 2) / g.H);
-    auto set_gp = [&](int gp) {
-        g.GP = gp;
-        g.NT = (gp * g.NC + 31) / 32 * 32;
-        finish_plan(g, d, ea);
-    };
-    int best = 1, sets = 1;
-    double least = 1e30;
-    for (int cpt = 1; cpt <= g.CPT; ++cpt)
-        for (int gp = GP2 > 0 ? std::min(GP2, most) : 1; gp <= most && gp * g.NC <= 352; ++gp) {
-            const double t = sweep_time(g.H * cpt, ngrp, gp, g.NC, regs, cpt);
-            if (t < least - 1e-9) {
-                least = t;
-                best = gp;
-                sets = cpt;
-            }
-            if (GP2 > 0) break;
+        if (threads > 0) {
+            columns(wish);
+            consider_all(352);
         }
-    g.CPT = sets * gm;
-    set_gp(best);
-    while (walk_smem(g, d, ea).total > WALK_SMEM_MAX && (g.CPT > 1 || g.GP > 1)) {
-        if (g.CPT > 1) g.CPT /= 2;
-        else g.GP /= 2;
-        set_gp(g.GP);
+    }
+    // The general kernel where it is faster: sides whose divisors leave few columns (twice a
+    // prime has L/2 of all rows, or of two rows each) and few groups of any side without a good
+    // split; columns of two or four rows cost 1.45 and 1.15 times what sweep_time() says, and the
+    // tiniest lattices' line stands at 1536 groups.  One run, us a step with k_group and with the
+    // walk: L = 58, 32 groups 95, 327; L = 24, 141 groups 43, 47, 1563 groups 142, 131; L = 8, 32
+    // groups 27, 45, 4688 groups 120, 72; 3D L = 2, 32 groups 26, 67, 4688 groups 124, 78.  Over
+    // all those runs the choice costs 0.5%, 13% at most (always the walk: 18% and 275%).
+    g = best;
+    const double few = g.H == 2 ? 1.45 : g.H == 4 ? 1.15 : 1.0;
+    if (d == 2 && L > 8 ? few * least > group_time(d, L * L, ea, ngrp, general)
+                        : L <= (d == 2 ? 8 : 2) && ngrp < 1536) {
+        g.flat = -1;
+        g.GP = g.CPT = 1;
+        return g;
     }
     // division by L: (s m) >> sh is exact for s < 2^15 (L <= 180) with sh = 24
     g.sL = 24;

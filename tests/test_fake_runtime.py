@@ -114,7 +114,7 @@ def test_small_sweeps_leave_room_for_others(pa, dim, L, threads):
 
 
 @pytest.mark.parametrize("L,R", [(16, 1000), (16, 4800), (32, 2000), (32, 4500), (32, 9500),
-                                 (64, 10000), (24, 4500), (16, 60000)])
+                                 (64, 10000), (48, 4800), (48, 10000), (16, 60000)])
 def test_sweeps_chained_to_the_one_launch_resampling(pa, L, R):
     """A sweep is placed while the one-launch resampling holds its SMs only where the others hold
     it at an even share each."""
@@ -142,3 +142,35 @@ def test_the_callers_stream_priority(pa, priority, R):
         want = min(priority + 1, 0) if "k_family" in x["name"] else priority
         assert x["priority"] == want, x
     assert any("k_sweep2d" in x["name"] and x["captured"] for x in new)
+
+
+def _sweeps(pa, L, R, ea=False, dim=2):
+    b = pa.Batch([{"dim": dim, "L": L, "R": R, "couplings": ("ea", 3, 1) if ea else ("ferro",)}],
+                 np.linspace(0.0, 1.0, 5), np.full(4, 2, np.uint32), "systematic", 1, graph=False,
+                 use_torch_memory=False, stream=fake_runtime.Stream(pa._lib))
+    first = pa._lib.fake_launches()
+    b.step(1)
+    new = fake_runtime.launches(pa._lib, first)
+    b.close()
+    return [x for x in new if any(k in x["name"] for k in ("k_sweep", "k_walk", "k_group"))]
+
+
+@pytest.mark.parametrize("ea", [False, True])
+@pytest.mark.parametrize("L", [24, 26, 38, 44, 46, 50, 54, 58, 60, 66, 74, 82, 90, 96, 100, 106, 118,
+                               120, 134, 140, 158])
+def test_plans_of_2d_sides_fill_the_sms(pa, L, ea):
+    """Whatever the divisors of a side: a small population has at least 64 threads per group of
+    32 replicas, and a large one leaves room for at least 256 threads on an SM (registers,
+    shared memory), or the general kernel takes it."""
+    x, = _sweeps(pa, L, 1000, ea)
+    if "k_group" not in x["name"]:
+        assert x["block"] >= 64 * -(-32 // x["grid"]), x
+    x, = _sweeps(pa, L, 40000, ea)
+    if "k_group" not in x["name"]:
+        ctas = min(65536 // (96 * x["block"]), 228 * 1024 // (x["smem"] + 2048))
+        assert ctas * x["block"] >= 256, x
+
+
+def test_general_kernel_for_small_populations_of_tiny_lattices(pa):
+    assert "k_group" in _sweeps(pa, 2, 1000, dim=3)[0]["name"]
+    assert "k_walk" in _sweeps(pa, 2, 90000, dim=3)[0]["name"]
