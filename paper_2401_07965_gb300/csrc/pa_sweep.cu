@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(NT) k_group(KParams p, int mode, int only) {
 // (3329, 3208, 2640) and 3125 (4669, 4352, 3512), where it takes the best of each.  Over all
 // plans of 17 other 2D and 6 3D sides, 32 to 6250 groups, its choice is 1.6% slower than the
 // best one on average, 15% at most (4.3% and 57% without the shared memory: L = 54, 2813
-// groups 1184 us a step, 742 with it).
+// groups 1184 us a step, 788 with it).
 double sweep_time(int rows, uint32_t ngrp, int GP, int tg, int regs, int CPT, size_t smem,
                   double alone) {
     const double er = rows >= 16 ? 1.0 : rows >= 12 ? 0.97 : rows >= 8 ? 0.93 : rows >= 6 ? 0.9
