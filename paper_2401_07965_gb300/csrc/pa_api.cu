@@ -802,6 +802,7 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
         mostl = std::max(mostl, h.nlev);
     }
     p.pop = pop_ctas(mostR, mostl, M, p.method, &p.pop_threads, &p.pop_levels);
+    if (!pop_fits(p)) p.pop = 0;
 
     // The sweep's launches: the 2D kernel when all runs have one of its sides; else the
     // column walk, one launch per distinct side (at most four), each over the CTAs of the

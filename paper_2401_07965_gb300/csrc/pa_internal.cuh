@@ -308,6 +308,7 @@ cudaError_t launch_measure(const KParams& p, int threads, cudaStream_t s);
 cudaError_t launch_resample(const KParams& p, cudaStream_t s, int64_t* launches);
 int pop_ctas(uint32_t most_R, int most_levels, int M, int method, int* threads,
              int* levels);
+bool pop_fits(const KParams& p);
 cudaError_t launch_pop(const KParams& p, cudaStream_t s);
 inline bool pop_takes(const KParams& p) { return p.pop && !p.lb_hold; }
 cudaError_t launch_weighted_sums(const KParams& p, int mode, cudaStream_t s, int64_t* launches);

@@ -459,9 +459,9 @@ int pop_ctas(uint32_t most_R, int most_levels, int M, int method, int* threads, 
     return cs <= POP_CTAS && P <= POP_LEVELS && (int64_t)M * cs <= 128 ? cs : 0;
 }
 
+// one launch, or (fits != nullptr) how many of its clusters the device holds at a time
 template <int NT, bool PARTIAL>
-static cudaError_t launch(const KParams& p, cudaStream_t s) {
-    const size_t sm = 2 * sizeof(double) * (size_t)p.pop_levels;
+static cudaError_t launch(const KParams& p, cudaStream_t s, int* fits) {
     // the limit is the kernel's, whoever launches it: always the largest, so that a context on
     // another thread never lowers it between this call and the launch
     cudaError_t e = cudaFuncSetAttribute(k_pop<NT, PARTIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -476,22 +476,34 @@ static cudaError_t launch(const KParams& p, cudaStream_t s) {
     cudaLaunchConfig_t c = {};
     c.gridDim = dim3((unsigned)(p.M * p.pop));
     c.blockDim = dim3(NT);
-    c.dynamicSmemBytes = sm;
+    c.dynamicSmemBytes = 2 * sizeof(double) * (size_t)p.pop_levels;
     c.stream = s;
     c.attrs = &at;
     c.numAttrs = 1;
+    if (fits) return cudaOccupancyMaxActiveClusters(fits, k_pop<NT, PARTIAL>, &c);
     return cudaLaunchKernelEx(&c, k_pop<NT, PARTIAL>, p);
 }
 
 template <bool PARTIAL>
-static cudaError_t launch(const KParams& p, cudaStream_t s) {
-    return p.pop_threads == 256   ? launch<256, PARTIAL>(p, s)
-           : p.pop_threads == 512 ? launch<512, PARTIAL>(p, s)
-                                  : launch<1024, PARTIAL>(p, s);
+static cudaError_t launch(const KParams& p, cudaStream_t s, int* fits) {
+    return p.pop_threads == 256   ? launch<256, PARTIAL>(p, s, fits)
+           : p.pop_threads == 512 ? launch<512, PARTIAL>(p, s, fits)
+                                  : launch<1024, PARTIAL>(p, s, fits);
+}
+
+// Whether the device can place the context's clusters.  Up to eight CTAs every device can; for
+// more, SMs of one GPC must be free for all of them, which a partition of a GPU may not have.
+bool pop_fits(const KParams& p) {
+    if (p.pop <= 8) return true;
+    int plain = 0, partial = 0;
+    const bool known = launch<false>(p, nullptr, &plain) == cudaSuccess &&
+                       launch<true>(p, nullptr, &partial) == cudaSuccess;
+    if (!known) cudaGetLastError();  // not an error of the caller's: the general kernels run
+    return known && plain > 0 && partial > 0;
 }
 
 cudaError_t launch_pop(const KParams& p, cudaStream_t s) {
-    return p.alpha >= 0.0 ? launch<true>(p, s) : launch<false>(p, s);
+    return p.alpha >= 0.0 ? launch<true>(p, s, nullptr) : launch<false>(p, s, nullptr);
 }
 
 }  // namespace pa

@@ -79,7 +79,7 @@ void fake_reset(int n_devices) {  // the attributes stay, as a process keeps the
 void fake_set_device(int d) { device = d; }
 int fake_device() { return device; }
 void fake_static_smem(const char* part, int bytes) { static_smem[part] = bytes; }
-void fake_clusters_fit(int n) { clusters_fit = n; }
+void fake_clusters_fit(int n) { clusters_fit = n; }  // clusters of more than eight CTAs
 void fake_attr_hook(void (*f)()) { attr_hook = f; }
 void* fake_stream(int priority) { return new Stream{priority, device, false}; }
 int fake_launches() { return (int)launches.size(); }

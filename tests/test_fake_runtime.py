@@ -174,3 +174,19 @@ def test_plans_of_2d_sides_fill_the_sms(pa, L, ea):
 def test_general_kernel_for_small_populations_of_tiny_lattices(pa):
     assert "k_group" in _sweeps(pa, 2, 1000, dim=3)[0]["name"]
     assert "k_walk" in _sweeps(pa, 2, 90000, dim=3)[0]["name"]
+
+
+@pytest.mark.parametrize("R", [1000, 8000, 30000])
+@pytest.mark.parametrize("alpha", [None, 0.5])
+def test_clusters_that_the_device_cannot_place(pa, R, alpha):
+    """Where no cluster of more than eight CTAs finds its SMs (a partition of a GPU), larger
+    populations take the general resampling kernels instead of failing."""
+    pa._lib.fake_clusters_fit(0)
+    b = _run(pa, 16, R)
+    if alpha is not None:
+        b.set_partial_resampling(alpha)
+    first = pa._lib.fake_launches()
+    b.step(1)
+    names = [x["name"] for x in fake_runtime.launches(pa._lib, first)]
+    assert any("k_pop" in n for n in names) == (R == 1000)
+    assert any("k_resample" in n for n in names) == (R > 1000)
