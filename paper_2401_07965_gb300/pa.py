@@ -550,7 +550,7 @@ class Population:
             from . import tune
             th = int(np.median(self.thetas)) if len(self.thetas) else 0
             specs, so = self._tune_specs(), getattr(self, "_stream_obj", None)
-            sweep_threads = tune.best_sweep_threads_batch(specs, theta=th, stream=so)
+            sweep_threads = tune.choose_sweep_threads_batch(specs, theta=th, stream=so)
             groups = tune.best_sweep_groups_batch(specs, theta=th, stream=so)
             if groups > 1:
                 pa_set_sweep_groups(self.ctx, groups)
@@ -664,7 +664,7 @@ class Batch:
             from . import tune
             th = int(np.median(self.thetas)) if len(self.thetas) else 0
             specs, so = self._tune_specs(), getattr(self, "_stream_obj", None)
-            sweep_threads = tune.best_sweep_threads_batch(specs, theta=th, stream=so)
+            sweep_threads = tune.choose_sweep_threads_batch(specs, theta=th, stream=so)
             groups = tune.best_sweep_groups_batch(specs, theta=th, stream=so)
             if groups > 1:
                 pa_set_sweep_groups(self.ctx, groups)

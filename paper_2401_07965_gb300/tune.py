@@ -1,36 +1,51 @@
 """Autotuner for the launch configuration of the sweep kernel.
 
-The sweep kernel runs one CTA per 32 replicas; how many threads share a CTA
-(64-512) trades per-CTA parallelism against the number of CTAs resident per
-SM and the rounding of the grid into waves, which depends on the lattice and
-on the population size.  The grouped 3D kernel has a fixed CTA size and holds
-several replica groups per CTA; the tuner picks between that count and twice
-it.  The tuner times each candidate on a throw-away run of
-the same shape (same lattice, couplings kind, R and theta; results never
-depend on the choice) and remembers the fastest per device and shape, in
+A sweep CTA holds one or several groups of 32 replicas; how many threads share a group
+trades the latency of a sweep against the rounds of CTAs that the SMs hold, which depends on
+the lattice and on the population size.  The library chooses by a rule; the tuner times that
+choice and the variants that pa_set_sweep_threads names (64-512), and for the 3D kernels of
+sides 4..16 the number of replica groups per CTA and twice it.  Each candidate runs on a
+throw-away run of the same shape (same lattice, couplings kind, R and theta; results never
+depend on the choice), and the fastest is remembered per device, library source and shape, in
 memory and in a small JSON cache file.
 """
 from __future__ import annotations
 
+import functools
 import hashlib
 import json
 import os
 
 import numpy as np
 
-from . import pa
+from . import build, pa
 
 CANDIDATES = (64, 128, 256, 384, 512)
 _CACHE = {}
 _CACHE_FILE = os.path.join(os.path.expanduser("~"), ".cache", "pa_gb300_tune.json")
 
 
-def _key(dim, L, R, ea, theta):
+@functools.lru_cache(maxsize=1)
+def _source():
+    """Names the library's source: choices timed on other kernels do not count."""
+    h = hashlib.sha256()
+    for path in sorted(build._deps()):
+        with open(path, "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:12]
+
+
+def _device():
     try:
         import torch
         dev = torch.cuda.get_device_name()
     except Exception:
         dev = "cuda"
+    return f"{dev}|{_source()}"
+
+
+def _key(dim, L, R, ea, theta):
+    dev = _device()
     return f"{dev}|d{dim}|L{L}|R{R}|ea{int(ea)}|theta{theta}"
 
 
@@ -62,11 +77,7 @@ def best_sweep_threads(dim, L, R, couplings=("ferro",), theta=10, candidates=CAN
 
 
 def _batch_key(specs, theta):
-    try:
-        import torch
-        dev = torch.cuda.get_device_name()
-    except Exception:
-        dev = "cuda"
+    dev = _device()
     if len(specs) == 1:
         s = specs[0]
         ea = s.get("couplings", ("ferro",))[0] != "ferro"
@@ -87,27 +98,57 @@ def best_sweep_threads_batch(specs, theta=10, candidates=CANDIDATES, rounds=2, u
         _load()
         if key in _CACHE:
             return int(_CACHE[key])
-    n = rounds * len(candidates) + 1
-    betas = np.linspace(0.0, 0.5, n + 1)
+    best = _rates(specs, theta, candidates, rounds, stream)
+    best.pop(0)
+    choice = max(best, key=best.get)
+    _CACHE[key] = int(choice)
+    if use_cache:
+        _save()
+    return int(choice)
+
+
+def choose_sweep_threads_batch(specs, theta=10, candidates=CANDIDATES, rounds=2, use_cache=True,
+                               stream=None):
+    """What sweep_threads="auto" sets: 0 to leave the launch to the library's rule, or the
+    candidate that beats it by more than a percent (timed like best_sweep_threads_batch)."""
+    key = _batch_key(specs, theta) + "|auto"
+    if use_cache:
+        _load()
+        if key in _CACHE:
+            return int(_CACHE[key])
+    best = _rates(specs, theta, candidates, rounds, stream)
+    rule = best.pop(0)
+    choice = max(best, key=best.get)
+    if best[choice] <= 1.01 * rule:
+        choice = 0
+    _CACHE[key] = int(choice)
+    if use_cache:
+        _save()
+    return int(choice)
+
+
+def _rates(specs, theta, candidates, rounds, stream):
+    """Sweep rate of the library's rule (0) and of every candidate."""
+    n = rounds * (len(candidates) + 1) + 1
+    # one step to the temperatures of interest, then nearly equal ones: the kernels' work
+    # depends on the thresholds
+    betas = np.concatenate([[0.0], 0.4 + 1e-3 * np.arange(n)])
     thetas = np.full(n, theta, np.uint32)
     run = pa.Batch([dict(s) for s in specs], betas, thetas, "systematic", 12345, stream=stream,
                    graph=False)
     run.step(1)  # first launch of each kernel outside the timings
     best = {}
     pa.pa_enable_timing(run.ctx, True)
-    for _ in range(rounds):
-        for t in candidates:
+    # the rule first: it is in force until the first call of pa_set_sweep_threads
+    for t in (0,) * rounds + tuple(candidates) * rounds:
+        if t:
             pa.pa_set_sweep_threads(run.ctx, t)
-            run.step(1)
-            ms, cnt, upd = pa.pa_sweep_timing(run.ctx)
-            rate = upd / max(ms, 1e-9)
-            best[t] = max(best.get(t, 0.0), rate)
+        run.step(1)
+        ms, cnt, upd = pa.pa_sweep_timing(run.ctx)
+        rate = upd / max(ms, 1e-9)
+        best[t] = max(best.get(t, 0.0), rate)
     run.close()
-    choice = max(best, key=best.get)
-    _CACHE[key] = int(choice)
-    if use_cache:
-        _save()
-    return int(choice)
+    return best
 
 
 def best_sweep_groups_batch(specs, theta=10, rounds=2, use_cache=True, stream=None):
