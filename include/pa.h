@@ -236,10 +236,14 @@ int64_t pa_launch_count(const pa_ctx *ctx);
 
 /* Launch configuration of the sweep kernel: how many threads share the lattice of
  * 32 replicas, from few (64) to many (128, 256, 384, 512); each side has its own
- * variants for them.  Until the call the library chooses by the number of replicas.
- * Results do not depend on it, only the speed; the package's autotuner times the
- * candidates and picks one.  Synchronises the context's stream when the value
- * changes.  PA_ERR_ARG for other values. */
+ * variants for them.  Until the call the library chooses by the number of replicas, for
+ * the shortest step of one context that has the GPU to itself: a small population then
+ * gets as many threads per group as help.  Several contexts on streams of their own do
+ * more in all with fewer (2D L = 64, R = 3000, eight contexts: a step of all 290 us, 247
+ * with 256 threads; one alone 66 and 71).  Results do not depend on it, only the speed; the package's autotuner times the library's choice
+ * and the candidates.  Synchronises the context's stream when the value changes, so not
+ * to be called while the stream is captured.  PA_ERR_ARG for other values.
+ * pa_get_sweep_threads: the value set, before that the general kernel's. */
 pa_status pa_set_sweep_threads(pa_ctx *ctx, int32_t threads);
 int32_t pa_get_sweep_threads(const pa_ctx *ctx);
 
@@ -397,8 +401,9 @@ pa_status pa_set_partial_resampling(pa_ctx *ctx, double alpha);
  * PA_ERR_ARG otherwise. */
 pa_status pa_overlap(pa_ctx *ctx, const int32_t *run_a, const int32_t *run_b, int32_t n_pairs,
                      uint32_t *hist_dev, double *P_out);
-/* Replay each temperature step as one captured CUDA graph (default on; needs a
- * non-NULL stream; timing mode launches directly). */
+/* Replay temperature steps as captured CUDA graphs, one step or eight to a graph (default
+ * on; needs a non-NULL stream; timing mode launches directly).  The captured kernels keep
+ * the priority that the stream had at the capture. */
 pa_status pa_set_graph(pa_ctx *ctx, int32_t on);
 
 /* ---- learned schedule -----------------------------------------------------

@@ -804,9 +804,9 @@ pa_status pa_batch_init(pa_ctx** out, const pa_run_spec* specs, int32_t M,
     p.pop = pop_ctas(mostR, mostl, M, p.method, &p.pop_threads, &p.pop_levels);
     if (!pop_fits(p)) p.pop = 0;
 
-    // The sweep's launches: the 2D kernel when all runs have one of its sides; else the
-    // column walk, one launch per distinct side (at most four), each over the CTAs of the
-    // runs of that side in run order; with more sides the general kernel.
+    // The sweep's launches: the 2D kernel when all runs have one of its sides; else one launch
+    // per distinct side (at most four), of the column walk over the CTAs of the runs of that
+    // side in run order, or of the general kernel; with more sides the general kernel.
     std::vector<uint32_t> c3;
     {
         std::vector<int> Ls;

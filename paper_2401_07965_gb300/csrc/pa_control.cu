@@ -93,8 +93,9 @@ __global__ void __launch_bounds__(64) k_mlp_fwd(const uint16_t* __restrict__ par
 // gradient are 64 x 64 x GR each: a thread holds a 4 x 2 tile of the result and reads a
 // 128-bit and a 64-bit word of shared memory per 8 fused multiply-adds.
 // What bounds it: shared-memory latency on one CTA per SM (30 k flops per row).  GR = 32, 64
-// or 96, the least that takes the rows of one of 152 CTAs in one pass: 12040 rows are 151
-// CTAs of 80 rows; two passes of 64 with 256 threads took 33 us, one pass 22 us (the whole
+// or 96, the least that takes the rows of one of 152 CTAs in one pass, and passes of 96 from 97
+// rows on (14592 rows 24 us, 14593 to 29184 39; with the forward pass in a kernel of its own 63,
+// 70 to 96).  12040 rows are 151 CTAs of 80 rows; two passes of 64 with 256 threads took 33 us, one pass 22 us (the whole
 // update of 12040 rows: 66 us with the forward pass stored and read back, 31 with one kernel,
 // 29 with the reduction chained to it).
 // --------------------------------------------------------------------------
@@ -383,6 +384,8 @@ size_t mlp_blocks(int B) { return (size_t)(B + ROWS - 1) / ROWS; }
 
 extern "C" {
 
+// The gradients' parts take a third of it; the rest, a row's activations, is what the call has
+// asked for and checked since the forward pass stored them, and stays so for its callers.
 size_t pa_mlp_scratch_bytes(int32_t B) {
     if (B <= 0) return 0;
     const size_t nb = mlp_blocks(B);

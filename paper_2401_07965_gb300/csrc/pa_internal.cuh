@@ -98,7 +98,8 @@ __device__ __forceinline__ void mulhilo(uint32_t a, uint32_t b, uint32_t& hi, ui
     lo = (uint32_t)p;
 }
 
-// floor(2^40 x / S), the quotient rounded to FP64 first, for 0 <= x < 2^24 S, y = 1 / S rounded.  Two residual corrections of x y give the rounded quotient (Markstein, IBM
+// floor(2^40 x / S), the quotient rounded to FP64 first, for 0 <= x < 2^24 S, y = 1 / S
+// rounded.  Two residual corrections of x y give the rounded quotient (Markstein, IBM
 // J. Res. Dev. 34, 1990): 5 operations of the FP64 pipe instead of a division's 20.  Below
 // 2^-45 S the result is 0, and from there on no operation meets a subnormal unless S is tiny
 // (partial resampling alone: a level sum is at least 1).
@@ -250,11 +251,13 @@ struct KParams {
     int lb_hold;             // test: scan block 0 withholds its prefix (the waits run out)
     const double* clnc;      // c ln c for c = 0 .. CLN_TAB (0 for c < 2), from the host's log
     int L_all;               // the side L shared by every run of the batch (0 if they differ)
-    // column-walk plan: one launch per distinct side (nw = 0: the general kernel)
+    // sweeps by side: one launch per distinct side (nw = 0: the 2D kernel or, without its plan,
+    // the general kernel)
     int nw;
     int g3mul;                 // 3D: sets of groups per CTA, the side's count times this (1 or 2)
     WalkPlan wplan[4];
-    int G2, TG2;               // 2D kernel (nw = 0): groups per CTA (0: the general kernel), threads of each
+    int G2, TG2;               // 2D kernel (nw = 0): groups per CTA (0: the general kernel),
+                               // threads of each
     int pop;                   // k_pop: CTAs per run (0: the general kernels),
     int pop_threads, pop_levels;  // their threads, entries of their level arrays
     const uint32_t* wmap[4];   // CTA -> run of each launch
@@ -278,7 +281,8 @@ constexpr int SCAN_CHUNK = SCAN_THREADS * SCAN_ITEMS;
 // then, so those waiting take no place from them.  Without that call the next kernel is
 // placed when this one ends.  Every CTA of a chained kernel waits before it ends, so the
 // end of a kernel is the end of all before it.  Only launches whose predecessor is always a
-// kernel of this library are chained.  What it saves is the gap between two launches: the
+// kernel of this library are chained, and a sweep only where it finds its places beside k_pop
+// (chain_sweep(); chain = false is an ordinary launch).  What it saves is the gap between two launches: the
 // sweep after k_pop, 2D L = 16, R = 1000 41.9 -> 40.9 us a step, +-J L = 48, R = 20001 217.6
 // -> 212.5; the three sides of a 3D batch 1093 -> 1075; pa_weights_static, 10^5 energies
 // 14.4 -> 12.3; the training gradients and their sum, 12040 rows, with Adam 30.6 -> 28.7.

@@ -9,11 +9,10 @@
 // What bounds it: latency, 14 to 20 thousand cycles (8 to 11 us) of short phases: a block scan
 // with its cluster barrier 2 (one for the rules that need one prefix, three for the drawn
 // ones), the level weights 5, the draws or the copy numbers 3 to 6, the scatter 2, the
-// variance's tree 1.5.  Temperature steps with ten sweeps: 2D L = 16,
-// R = 1000, multinomial (four kernels before) 57 -> 42 us, 41 with the sweep chained to it; L = 64, R = 3000, systematic, with
-// the learned schedule 60 -> 53; +-J L = 48, R = 20001, Poisson 231 -> 219; L = 64,
-// R = 10^4, systematic, partial resampling (seven kernels, the family statistics after the
-// sweep) 202 -> 185.
+// variance's tree 1.5.  Temperature steps with ten sweeps, the general kernels -> this one, both
+// without chained launches: 2D L = 16, R = 1000, multinomial 57 -> 42 us; L = 64, R = 3000,
+// systematic, with the learned schedule 60 -> 53; +-J L = 48, R = 20001, Poisson 231 -> 219;
+// L = 64, R = 10^4, systematic, partial resampling 202 -> 185.
 #include <cooperative_groups.h>
 
 #include <algorithm>

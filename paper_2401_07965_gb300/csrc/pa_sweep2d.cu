@@ -43,8 +43,9 @@
 // R = 4 10^5 (156 instructions per site word; 189 in the halo layout with its queue).
 // L = 64, theta = 10, beta 0 -> 1, updates/ns, before -> now: R = 10^5 4352 -> 4660,
 // R = 20000 (theta 5) 3006 -> 3304, R = 3000 1639 -> 1890; L = 32, R = 1024000
-// 3811 -> 4797; L = 16, R = 1000 88 -> 117.  80 registers instead of 96 lose 2%, 64 10%;
-// eight rows per loop pass instead of four 1-4%.
+// 3811 -> 4797; L = 16, R = 1000 88 -> 117.  The 96 registers that five CTAs of 128 threads
+// leave are short by a few: ptxas spills 16 bytes at L = 64, 76 with four groups of L = 32.  80
+// registers instead of 96 lose 2%, 64 10%; eight rows per loop pass instead of four 1-4%.
 #include "pa_walk.cuh"
 
 namespace pa {

@@ -1,7 +1,7 @@
 // pa_sweepw.cu -- the temperature step's replica copy, theta checkerboard
 // Metropolis sweeps and measurement (Sec. 2 steps 2-4) by column walks, for 3D
 // lattices (except L = 10, 12, 14) and 2D lattices of the sides that pa_sweep2d.cu
-// does not take.  Random numbers, decisions and results are those of k_group's sweep mode.
+// does not take, where walk_plan() finds them faster than the general kernel.  Random numbers, decisions and results are those of k_group's sweep mode.
 //
 // Layout.  32 replicas in the multi-spin form (one word per site, bit r =
 // replica r), the two colours in arrays of their own: the site of column slot

@@ -152,8 +152,8 @@ def _rates(specs, theta, candidates, rounds, stream):
 
 
 def best_sweep_groups_batch(specs, theta=10, rounds=2, use_cache=True, stream=None):
-    """Group multiple (1 or 2) of the fastest grouped 3D sweep for a batch of runs: 1 when
-    the runs do not use the grouped kernel, else both are timed on a throw-away batch of
+    """Group multiple (1 or 2) of the fastest 3D sweep for a batch of runs: 1 when
+    pa_set_sweep_groups refuses 2 for them, else both are timed on a throw-away batch of
     the same runs (results never depend on the choice) and the faster is remembered."""
     if any(s["dim"] != 3 for s in specs):
         return 1
