@@ -38,7 +38,7 @@
 //
 // What bounds it: logic operations and wide multiplies share an issue resource (a probe
 // with 6 warps per scheduler: 2 cycles for a logic operation, 2 more for a wide multiply
-// beside them, 0.5 for a plain one), so a site costs about 2.17 cycles per scheduler for
+// beside them, 0.1 for a plain one), so a site costs about 2.17 cycles per scheduler for
 // each of its 79 + 34 of them, 7 for the rest: 261 of the 266 cycles measured at L = 64,
 // R = 4 10^5 (156 instructions per site word; 189 in the halo layout with its queue).
 // L = 64, theta = 10, beta 0 -> 1, updates/ns, before -> now: R = 10^5 4352 -> 4660,
