@@ -242,8 +242,8 @@ int64_t pa_launch_count(const pa_ctx *ctx);
  * more in all with fewer (2D L = 64, R = 3000, eight contexts: a step of all 290 us, 247
  * with 256 threads; one alone 66 and 71).  Results do not depend on it, only the speed; the
  * package's autotuner times the library's choice and the candidates.  Synchronises the
- * context's stream when the value changes, so not to be called while the stream is
- * captured.  PA_ERR_ARG for other values.
+ * context's stream when the value changes (while the caller captures the stream, the next
+ * step after the capture does).  PA_ERR_ARG for other values.
  * pa_get_sweep_threads: the value set, before that the general kernel's. */
 pa_status pa_set_sweep_threads(pa_ctx *ctx, int32_t threads);
 int32_t pa_get_sweep_threads(const pa_ctx *ctx);

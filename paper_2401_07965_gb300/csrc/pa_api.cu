@@ -103,6 +103,7 @@ struct pa_ctx {
     bool finished = false;                  // beta_f reached under the controller
     uint32_t* d_cta = nullptr;              // CTA -> run map of the sweep launches (device)
     bool auto_threads = true;               // the rule's threads until the caller sets them
+    bool replan_due = false;                // set while the stream was captured
     bool grouped3 = false;                  // 3D sides whose sets of groups may be doubled
     CtlDev* d_ctl = nullptr;
     double* d_gbeta = nullptr;
@@ -441,7 +442,15 @@ void drop_graphs(pa_ctx* ctx) {
 
 // rebuild the plan (after a change of threads or of the group multiple): no step in
 // flight may read the old one
+// (while the caller captures the stream: from the first step after the capture on)
 pa_status replan(pa_ctx* ctx, int gm) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    // an error means a capture, too: the legacy stream's while another stream is captured
+    const bool known = cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    ctx->kp.g3mul = gm;
+    ctx->replan_due = !known || cap != cudaStreamCaptureStatusNone;
+    if (ctx->replan_due) return PA_OK;
     PA_CUDA(cudaStreamSynchronize(ctx->stream));
     std::vector<uint32_t> c3;
     plan_sweep(ctx, gm, ctx->d_cta, c3);
@@ -914,6 +923,10 @@ pa_status pa_step(pa_ctx* ctx, int32_t n) {
         if (ctx->host_step + n > ctx->n_steps) n = ctx->n_steps - ctx->host_step;
     }
     if (ctx->host_step + n > ctx->n_steps) return PA_ERR_DONE;
+    if (ctx->replan_due) {
+        const pa_status s = replan(ctx, ctx->kp.g3mul);
+        if (s != PA_OK) return s;
+    }
     const bool graph = ctx->use_graph && !ctx->timing && ctx->stream != nullptr;
     if (graph && ctx->graph_threads != ctx->threads) drop_graphs(ctx);
     while (n > 0) {

@@ -81,6 +81,7 @@ int fake_device() { return device; }
 void fake_static_smem(const char* part, int bytes) { static_smem[part] = bytes; }
 void fake_clusters_fit(int n) { clusters_fit = n; }  // clusters of more than eight CTAs
 void fake_attr_hook(void (*f)()) { attr_hook = f; }
+void fake_capture(void* s, int on) { stream_of((cudaStream_t)s)->capturing = on != 0; }
 void* fake_stream(int priority) { return new Stream{priority, device, false}; }
 int fake_launches() { return (int)launches.size(); }
 // field of launch k: 0 grid, 1 block, 2 cluster, 3 shared memory, 4 device, 5 priority, 6 captured,
@@ -231,7 +232,13 @@ cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t* g) {
     *g = (cudaGraph_t) new int(0);
     return cudaSuccess;
 }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* st) {
+    *st = s && stream_of(s)->capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+    return s && stream_of(s)->capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) {
     *e = (cudaEvent_t) new int(0);

@@ -47,6 +47,7 @@ def load():
         lib = mod._lib
         lib.fake_stream.restype = C.c_void_p
         lib.fake_launch.restype = C.c_longlong
+        lib.fake_capture.argtypes = [C.c_void_p, C.c_int]
         lib.fake_static_smem.argtypes = [C.c_char_p, C.c_int]
         _binding = mod
     _binding._lib.fake_reset(1)

@@ -190,3 +190,20 @@ def test_clusters_that_the_device_cannot_place(pa, R, alpha):
     names = [x["name"] for x in fake_runtime.launches(pa._lib, first)]
     assert any("k_pop" in n for n in names) == (R == 1000)
     assert any("k_resample" in n for n in names) == (R > 1000)
+
+
+def test_sweep_threads_while_the_stream_is_captured(pa):
+    """The call is taken while the caller captures the stream; the launch follows it from the
+    first step after the capture on."""
+    s = fake_runtime.Stream(pa._lib)
+    b = pa.Batch([{"dim": 2, "L": 64, "R": 1000}], np.linspace(0.0, 1.0, 9),
+                 np.full(8, 2, np.uint32), "systematic", 1, graph=False, use_torch_memory=False,
+                 stream=s)
+    pa.pa_set_sweep_threads(b.ctx, 64)
+    pa._lib.fake_capture(s.cuda_stream, 1)
+    pa.pa_set_sweep_threads(b.ctx, 512)
+    b.step(1)
+    pa._lib.fake_capture(s.cuda_stream, 0)
+    b.step(1)
+    x = [y["block"] for y in fake_runtime.launches(pa._lib) if "k_sweep2d" in y["name"]]
+    assert x == [128, 512] and pa.pa_get_sweep_threads(b.ctx) == 512
